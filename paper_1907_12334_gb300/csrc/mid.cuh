@@ -1,0 +1,774 @@
+// mid.cuh -- mu-cycles of Algorithm 1 with a whole item hierarchy on chip.
+//
+// Two kernels run the recursion for one item per CTA, every grid they touch in
+// shared memory:
+//   k_item  an item of a low stage from its interpolated initial guess to
+//           convergence (FP64 residual, stopping decision, cycle, FP64 update,
+//           repeated inside the kernel);
+//   k_mid   the mu calls on the diagonals at and below kMidD inside the W-cycle
+//           of a larger item.
+//
+// Why.  A W-cycle visits diagonal d 2^(L-d) times, so its cost is a chain of
+// small dependent phases, two thirds of them on diagonals <= 3 (at most 102
+// unknowns).  What bounds it is the latency of that chain, not bytes or flops:
+// run as phases, the two calls at diagonal 4 took 65 us with the GPU otherwise
+// idle, and 132 us at 192 samples of 256 x 256.  Two things shorten it:
+//
+//  - The mu calls on diagonal 3 start from u = 0 and are linear in their
+//    right-hand side, so per sample and clipped triangle they are one matrix
+//    M (at most 72 x 72).  k_lowop builds its columns by running the calls on
+//    unit vectors, once per solve, in the arithmetic of the cycles; a
+//    call is then one matrix-vector product instead of about 170 phases.
+//  - Launch boundaries between visits become CTA barriers, and a visit keeps
+//    each thread's coefficients and right-hand side in registers.
+//
+// Layout.  Grid (p,q) is stored as its 2^(p+q) cells, cell (i,j) at j 2^p + i,
+// i < nx, j < ny.  Column 0 and row 0 are boundary nodes; the east
+// boundary of a row is the next row's column 0, and the north boundary is row 0
+// of the next grid (grids of a diagonal are ordered by p, so the next row 0 is
+// at least as long) or the pad behind the diagonal.  All boundary values of u
+// are therefore zeros at c +- 1 and c +- nx, every grid of diagonal d takes
+// exactly 2^(d+2) words, and the east and north faces of a node sit at the
+// node's own index.
+//
+// Work split.  A thread owns pairs of neighbouring cells (2m, 2m+1) of a
+// diagonal, all its grids in one index range; a pair holds one red and one
+// black node, so every half sweep uses every thread, and the face between the
+// two and the partner's value never leave the registers.
+#pragma once
+
+namespace msg {
+
+constexpr int kOpD = 3;      // the diagonal replaced by its matrix
+constexpr int kOpN = 72;     // unknowns of the full diagonal kOpD
+constexpr int kMidD = 6;     // highest diagonal of k_mid: three items fit one SM
+constexpr int kMidMax = 9;   // highest diagonal of any hierarchy held on chip
+constexpr int kItemL32 = 9;  // stages solved whole by k_item (FP32 cycles): (5,6) takes 155 KB
+constexpr int kItemL64 = 8;  // the same in FP64: (5,5) takes 170 KB
+constexpr int kMidThreads = 256;
+
+// ---------------------------------------------------------------- matrices --
+
+// Clipped triangles below diagonal kOpD that items of stage > kOpD have:
+// (pic, qic) = (min(p, 4), min(q, 4)), p + q >= kOpD + 3.
+constexpr int kOpClasses = 8;
+__host__ __device__ constexpr int op_pic(int c) { return c == 0 ? 1 : c == 1 ? 4 : c == 2 ? 2 : c == 3 ? 4 : c == 4 ? 3 : c == 5 ? 3 : 4; }
+__host__ __device__ constexpr int op_qic(int c) { return c == 0 ? 4 : c == 1 ? 1 : c == 2 ? 4 : c == 3 ? 2 : c == 4 ? 3 : c == 5 ? 4 : c == 6 ? 3 : 4; }
+// unknowns of the class on diagonal kOpD, and the row stride of its matrix:
+// two threads share a row, and ld / 2 = 4 (odd) keeps their 16-byte loads on disjoint banks
+__host__ __device__ constexpr int op_n(int pic, int qic)
+{
+    int n = 0;
+    for (int p = 1; p <= 4; ++p) {
+        const int q = kOpD + 2 - p;
+        if (p <= pic && q <= qic) n += ((1 << p) - 1) * ((1 << q) - 1);
+    }
+    return n;
+}
+__host__ __device__ constexpr int op_ld(int n) { return n <= 24 ? 24 : n <= 40 ? 40 : n <= 56 ? 56 : 72; }
+// does a sample with finest grid (P, Q) have items of the class?
+__host__ __device__ constexpr bool op_has(int pic, int qic, int P, int Q)
+{
+    return pic <= P && qic <= Q && (pic < 4 ? pic : P) + (qic < 4 ? qic : Q) >= kOpD + 3;
+}
+// offset of the class's matrix in the sample's block; (0, 0): size of the block
+__host__ __device__ inline int op_offset(int pic, int qic, int P, int Q)
+{
+    int o = 0;
+    for (int c = 0; c < kOpClasses; ++c) {
+        if (op_pic(c) == pic && op_qic(c) == qic) return o;
+        const int n = op_n(op_pic(c), op_qic(c));
+        if (op_has(op_pic(c), op_qic(c), P, Q)) o += n * op_ld(n);
+    }
+    return o;
+}
+// row / column of interior node (i, j) of grid (p, kOpD + 2 - p) in a class's matrix
+__host__ __device__ inline int op_index(int p, int i, int j, int qic)
+{
+    int o = 0;
+    for (int pp = 1; pp < p; ++pp)
+        if (kOpD + 2 - pp <= qic) o += ((1 << pp) - 1) * ((1 << (kOpD + 2 - pp)) - 1);
+    return o + (j - 1) * ((1 << p) - 1) + (i - 1);
+}
+
+// One matrix per CTA: sample blockIdx.x, clipped triangle (pic, qic).  Lane x
+// runs the mu calls on unit vector x through the phase program of the
+// low-diagonal tables (below), whose entries are uniform over the lanes; the
+// blockDim.y rows of the block share the entries of a phase.  Bound by the
+// latency of about 170 short phases; the whole block is a few per cent of one
+// residual-to-residual step of the solve.
+template <class T>
+__global__ void __launch_bounds__(768) k_lowop(const SampleInfo* samples, int pic, int qic, const T* img, int64_t istride,
+                                              int ify, const LowDesc* descs, const uint4* ent, const uint2* rprog,
+                                              LowPlanes lp, int mu, T omega, T* op)
+{
+    const SampleInfo S = samples[blockIdx.x];
+    if (!op_has(pic, qic, S.P, S.Q)) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const LowDesc& D = descs[low_class(pic, qic, kOpD)];
+    const int n = op_n(pic, qic), ld = op_ld(n), nc = n, nent = D.e1 - D.e0, nops = D.nops;
+    uint4* sent = (uint4*)smem_raw;
+    uint2* sprog = (uint2*)(sent + nent);
+    T* fx = (T*)(sprog + ((nops + 1) & ~1));
+    T* fy = fx + lp.nfx;
+    T* u = fy + lp.nfy;  // [slot][column]
+    T* b = u + lp.nu * nc;
+    T* r = b + lp.nu * nc;
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x, nt = blockDim.x * blockDim.y;
+    for (int k = tid; k < nent; k += nt) sent[k] = ent[D.e0 + k];
+    for (int k = tid; k < nops; k += nt) sprog[k] = rprog[D.prog + k];
+    const T* im = img + (int64_t)blockIdx.x * istride;
+    for (int k = tid; k < lp.nfx; k += nt) fx[k] = im[k];
+    for (int k = tid; k < lp.nfy; k += nt) fy[k] = im[ify + k];
+    for (int k = tid; k < 2 * lp.nu * nc; k += nt) u[k] = T(0);
+    __syncthreads();
+    const int col = threadIdx.x, g = threadIdx.y, ng = blockDim.y;
+    // slot of unknown t in the u and b planes
+    auto slot_of = [&](int t) {
+        for (int k = 0; k < lp.ngrid; ++k) {
+            const LowGrid G = lp.g[k];
+            if (G.p + G.q - 2 != kOpD || G.p > pic || G.q > qic) continue;
+            const int nx1 = (1 << G.p) - 1, ny1 = (1 << G.q) - 1;
+            if (t < nx1 * ny1) return G.gu + low_rb(nx1, ny1, 1 + t % nx1, 1 + t / nx1);
+            t -= nx1 * ny1;
+        }
+        return 0;
+    };
+    if (g == 0 && col < n) b[slot_of(col) * nc + col] = T(1);
+    __syncthreads();
+    for (int call = 0; call < mu; ++call)
+        for (int o = 0; o < nops; ++o) {
+            const uint2 w = sprog[o];
+            const int kind = w.x & 7, cnt = (int)(w.x >> 3), off = (int)w.y;
+            if (col < nc)
+                for (int e = g; e < cnt; e += ng) {
+                    const uint4 v = sent[off + e];
+                    auto U = [&](uint32_t s) { return u[s * nc + col]; };
+                    const uint32_t c = v.x & 0xFFFF;
+                    if (kind <= LK_RESID) {
+                        const int xw = v.z >> 16, ys = v.w & 0xFFFF;
+                        const T aw = fx[xw], ae = fx[xw + 1], as = fy[ys], an = fy[ys + 1];
+                        const T x = aw * U(v.x >> 16) + ae * U(v.y & 0xFFFF), y = as * U(v.y >> 16) + an * U(v.z & 0xFFFF);
+                        if (kind == LK_RESID) r[(v.w >> 16) * nc + col] = b[c * nc + col] - ((aw + ae + as + an) * U(c) - x - y);
+                        else u[c * nc + col] = (b[c * nc + col] + (x + y)) * rcp_of(aw + ae + as + an);
+                    } else if (kind == LK_RESTRICT) {
+                        const int rx = v.x >> 16, ry = v.y & 0xFFFF, wy = v.y >> 16;
+                        const bool hx = v.z & 1, hy = v.z & 2;
+                        T vx = T(0), vy = T(0);
+                        if (hx) vx = T(0.25) * (r[(rx - 1) * nc + col] + T(2) * r[rx * nc + col] + r[(rx + 1) * nc + col]);
+                        if (hy) vy = T(0.25) * (r[(ry - wy) * nc + col] + T(2) * r[ry * nc + col] + r[(ry + wy) * nc + col]);
+                        b[c * nc + col] = (hx && hy) ? T(0.5) * vx + T(0.5) * vy : (hx ? vx : vy);
+                        u[c * nc + col] = T(0);
+                    } else {
+                        const int xw = v.x >> 16, ys = v.y & 0xFFFF;
+                        const bool hx = (v.w >> 16) & 1, hy = (v.w >> 17) & 1;
+                        T vx = T(0), vy = T(0), corr;
+                        if (hx) vx = T(0.5) * (U(v.y >> 16) + U(v.z & 0xFFFF));
+                        if (hy) vy = T(0.5) * (U(v.z >> 16) + U(v.w & 0xFFFF));
+                        if (hx && hy) {
+                            const T cx = fx[xw] + fx[xw + 1], cy = fy[ys] + fy[ys + 1], x2 = cx * cx, y2 = cy * cy;
+                            const T s = rcp_of(x2 + y2);
+                            corr = (x2 * s) * vx + (y2 * s) * vy;
+                        } else {
+                            corr = hx ? vx : vy;
+                        }
+                        u[c * nc + col] += omega * corr;
+                    }
+                }
+            __syncthreads();
+        }
+    T* M = op + S.op_off + op_offset(pic, qic, S.P, S.Q);
+    for (int k = tid; k < n * ld; k += nt) {
+        const int t = k / ld, s = k - t * ld;
+        M[k] = s < n ? u[slot_of(t) * nc + s] : T(0);
+    }
+}
+
+// ------------------------------------------------------------------ visits --
+
+// One item's hierarchy (pic, qic: its top grid clipped to the diagonals held)
+// on chip: diagonals lo..hi; below lo (when lo = kOpD + 1) the matrix.
+template <class T>
+struct MidItem {
+    T* u;   // per diagonal: cells of its grids, then a pad of zeros (the last grid's north boundary)
+    T* b;   // cells
+    T* ax;  // cells
+    T* ay;
+    T* r;   // residual of the diagonal being restricted: the red node of each pair (every cell when nu1 = 0)
+    T* M;   // the matrix (lo = kOpD + 1)
+    T* b3;  // its right-hand side, compact
+    T* u3;  // its result: the cells of diagonal kOpD
+    const int2* at;  // first word of each diagonal in b, ax, ay (x) and in u (y)
+    int pic, qic, lo, hi;
+    int n3, ld3;
+};
+
+__host__ __device__ __forceinline__ int mid_plo(int d, int qic) { return d + 2 - qic > 1 ? d + 2 - qic : 1; }
+__host__ __device__ __forceinline__ int mid_phi(int d, int pic) { return d + 1 < pic ? d + 1 : pic; }
+__host__ __device__ __forceinline__ int mid_cells(int d, int pic, int qic)
+{
+    const int ng = mid_phi(d, pic) - mid_plo(d, qic) + 1;
+    return ng > 0 ? ng << (d + 2) : 0;
+}
+__host__ __device__ __forceinline__ int mid_pad(int d, int pic) { return 4 + (1 << mid_phi(d, pic)); }
+
+// words of the arrays of an item: cells of diagonals lo..hi, their pads, the residual
+struct MidWords { int cells, pads, r; };
+__host__ __device__ __forceinline__ MidWords mid_words(int pic, int qic, int lo, int hi, int nu1)
+{
+    MidWords w{0, 0, 0};
+    for (int d = lo; d <= hi; ++d) {
+        const int c = mid_cells(d, pic, qic), r = nu1 == 0 ? c : c >> 1;
+        w.cells += c;
+        w.pads += mid_pad(d, pic);
+        w.r = r > w.r ? r : w.r;
+    }
+    return w;
+}
+constexpr int kU3 = 4 * 32 + 20;  // cells of diagonal kOpD and their pad
+__host__ __device__ __forceinline__ int mid_total(int pic, int qic, int lo, int hi, int nu1)
+{
+    const MidWords w = mid_words(pic, qic, lo, hi, nu1);
+    int t = 4 * w.cells + w.pads + w.r;
+    if (lo > 0) {
+        const int n = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
+        t += n * op_ld(n) + kOpN + kU3;
+    }
+    return t;
+}
+
+// The pointers of an item whose words start at sm (16-byte aligned), and the table
+// of its diagonals (written by thread 0; a CTA barrier comes before its first use).
+template <class T>
+__device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic, int lo, int hi, int nu1)
+{
+    MidItem<T> m;
+    const MidWords w = mid_words(pic, qic, lo, hi, nu1);
+    m.pic = pic; m.qic = qic; m.lo = lo; m.hi = hi;
+    m.n3 = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
+    m.ld3 = op_ld(m.n3);
+    m.M = sm;
+    m.b3 = m.M + (lo > 0 ? m.n3 * m.ld3 : 0);
+    m.u3 = m.b3 + (lo > 0 ? kOpN : 0);
+    m.ax = m.u3 + (lo > 0 ? kU3 : 0);
+    m.ay = m.ax + w.cells;
+    m.b = m.ay + w.cells;
+    m.r = m.b + w.cells;
+    m.u = m.r + w.r;
+    m.at = at;
+    if (threadIdx.x == 0) {
+        int c = 0, pad = 0;
+        for (int d = lo; d <= hi; ++d) {
+            at[d] = make_int2(c, c + pad);
+            c += mid_cells(d, pic, qic);
+            pad += mid_pad(d, pic);
+        }
+    }
+    return m;
+}
+
+// pointers of one diagonal
+template <class T>
+struct MidDiag {
+    T* u;
+    T* b;
+    const T* ax;
+    const T* ay;
+    int plo, ng;
+};
+template <class T>
+__device__ __forceinline__ MidDiag<T> mid_diag(const MidItem<T>& m, int d)
+{
+    MidDiag<T> v;
+    const int2 o = m.at[d];
+    v.u = m.u + o.y;
+    v.b = m.b + o.x;
+    v.ax = m.ax + o.x;
+    v.ay = m.ay + o.x;
+    v.plo = mid_plo(d, m.qic);
+    v.ng = mid_phi(d, m.pic) - v.plo + 1;
+    return v;
+}
+
+template <class T> struct Vec2;
+template <> struct Vec2<float> { typedef float2 V; };
+template <> struct Vec2<double> { typedef double2 V; };
+template <class T>
+__device__ __forceinline__ typename Vec2<T>::V ld2(const T* p) { return *reinterpret_cast<const typename Vec2<T>::V*>(p); }
+
+// A thread's pair of cells during a visit: the red and the black node.  The
+// coefficients and b are divided by the node's diagonal, so that an update is
+// u = b + sum a u and the residual is diagonal * (b + sum a u - u); the kappa
+// weights, ratios of squared coefficients of one node, do not see the division.
+template <class T>
+struct Pair {
+    T pR, oR, sR, nR, bR, uR;  // red: face to the partner, outer horizontal, south and north face
+    T pK, oK, sK, nK, bK, uK;  // black
+    T dR;                      // diagonal of the red node
+    int cR;                    // its cell (relative to the diagonal); the black node's: cR - eR
+    int eR;                    // outer horizontal neighbour of the red node: cR + eR; of the black one: cR - 2 eR
+    int nx;                    // row stride; 0: no node (row 0)
+    bool vR, vK;
+};
+
+template <class T>
+__device__ __forceinline__ void pair_load(Pair<T>& P, const MidDiag<T>& g, int d, int m, bool in)
+{
+    const int cA = 2 * m, p = g.plo + (m >> (d + 1)), cell = cA & ((4 << d) - 1);
+    const int i = cell & ((1 << p) - 1), j = cell >> p;
+    P.vR = P.vK = false;
+    P.cR = P.eR = P.nx = 0;
+    P.pR = P.oR = P.sR = P.nR = P.bR = P.uR = P.pK = P.oK = P.sK = P.nK = P.bK = P.uK = P.dR = T(0);
+    if (!in || j == 0) return;
+    const int nx = 1 << p;
+    const bool hasA = i > 0, redB = j & 1;  // cell (i, j), i even, is red when j is even
+    const T aw = g.ax[cA - 1];              // (i = 0: the last face of the row below, not used)
+    const auto ae = ld2(g.ax + cA), an = ld2(g.ay + cA), as = ld2(g.ay + cA - nx), bb = ld2(g.b + cA), uu = ld2(g.u + cA);
+    const T dA = aw + ae.x + as.x + an.x, dB = ae.x + ae.y + as.y + an.y;
+    const T iA = hasA ? rcp_of(dA) : T(0), iB = rcp_of(dB), iR = redB ? iB : iA, iK = redB ? iA : iB;
+    P.nx = nx;
+    P.cR = cA + (redB ? 1 : 0);
+    P.eR = redB ? 1 : -1;
+    P.vR = redB || hasA;
+    P.vK = !redB || hasA;
+    P.dR = redB ? dB : dA;
+    P.pR = iR * ae.x; P.pK = iK * ae.x;
+    P.oR = iR * (redB ? ae.y : aw); P.oK = iK * (redB ? aw : ae.y);
+    P.sR = iR * (redB ? as.y : as.x); P.sK = iK * (redB ? as.x : as.y);
+    P.nR = iR * (redB ? an.y : an.x); P.nK = iK * (redB ? an.x : an.y);
+    P.bR = iR * (redB ? bb.y : bb.x); P.bK = iK * (redB ? bb.x : bb.y);
+    P.uR = redB ? uu.y : uu.x; P.uK = redB ? uu.x : uu.y;
+}
+
+// b + sum a u of the red / black node
+template <class T>
+__device__ __forceinline__ T pair_red(const Pair<T>& a, const T* u)
+{
+    return a.bR + ((a.pR * a.uK + a.oR * u[a.cR + a.eR]) + (a.sR * u[a.cR - a.nx] + a.nR * u[a.cR + a.nx]));
+}
+template <class T>
+__device__ __forceinline__ T pair_black(const Pair<T>& a, const T* u)
+{
+    const int c = a.cR - a.eR;
+    return a.bK + ((a.pK * a.uR + a.oK * u[c - a.eR]) + (a.sK * u[c - a.nx] + a.nK * u[c + a.nx]));
+}
+
+// nu red-black Gauss-Seidel sweeps over the thread's pairs; zero: u is zero on
+// entry, so the first red half sweep has no neighbours to read.
+template <class T, int NP>
+__device__ __forceinline__ void mid_sweeps(Pair<T> (&P)[NP], T* u, int nu, bool zero)
+{
+    for (int s = 0; s < nu; ++s) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            Pair<T>& a = P[k];
+            if (!a.vR) continue;
+            a.uR = zero ? a.bR : pair_red(a, u);
+            u[a.cR] = a.uR;
+        }
+        zero = false;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            Pair<T>& a = P[k];
+            if (!a.vK) continue;
+            a.uK = pair_black(a, u);
+            u[a.cR - a.eR] = a.uK;
+        }
+        __syncthreads();
+    }
+}
+
+// Eq. (2.3) into the children of diagonal d from m.r.  RED: m.r holds the red
+// node of each pair (pair k of a row: column 2k of an even row, 2k + 1 of an odd
+// one) and the black nodes are zero, so half of the weights drop out.
+template <class T, bool RED>
+__device__ __forceinline__ void mid_restrict(const MidItem<T>& m, int d)
+{
+    const int pplo = mid_plo(d, m.qic), plo = mid_plo(d - 1, m.qic), ngc = mid_phi(d - 1, m.pic) - plo + 1;
+    const bool op = d == m.lo && m.lo > 0;
+    T *cb = nullptr, *cu = nullptr;
+    if (!op) {
+        const MidDiag<T> c = mid_diag(m, d - 1);
+        cb = c.b;
+        cu = c.u;
+    }
+    for (int k = threadIdx.x; k < (ngc << d); k += blockDim.x) {
+        // cells A = (i, j), i even, and B = (i + 1, j) of child (p, q)
+        const int cA = 2 * k, p = plo + (k >> d), q = d + 1 - p, cell = cA & ((2 << d) - 1);
+        const int nx = 1 << p, i = cell & (nx - 1), j = cell >> p;
+        if (j == 0) continue;
+        const bool hx = p < m.pic, hy = q < m.qic;
+        T xA = T(0), xB = T(0), yA = T(0), yB = T(0);
+        if constexpr (RED) {
+            if (hx) {  // grid (p+1, q): row j has nx pairs, around columns 2i and 2i + 2
+                const T* r = m.r + ((p + 1 - pplo) << (d + 1)) + (j << p) + i;
+                const T r0 = r[0], r1 = r[1];
+                if (j & 1) {
+                    xA = T(0.25) * (r[-1] + r0);
+                    xB = T(0.25) * (r0 + r1);
+                } else {
+                    xA = T(0.5) * r0;
+                    xB = T(0.5) * r1;
+                }
+            }
+            if (hy) {  // grid (p, q+1): rows 2j - 1 .. 2j + 1 of nx / 2 pairs
+                const int h = nx >> 1;
+                const T* r = m.r + ((p - pplo) << (d + 1)) + j * nx + (i >> 1);
+                yA = T(0.5) * r[0];
+                yB = T(0.25) * (r[-h] + r[h]);
+            }
+        } else {
+            if (hx) {
+                const T* r = m.r + ((p + 1 - pplo) << (d + 2)) + (j << (p + 1)) + 2 * i;
+                const T rm = r[-1];
+                const auto r0 = ld2(r), r2 = ld2(r + 2);
+                xA = T(0.25) * (rm + T(2) * r0.x + r0.y);
+                xB = T(0.25) * (r0.y + T(2) * r2.x + r2.y);
+            }
+            if (hy) {
+                const T* r = m.r + ((p - pplo) << (d + 2)) + (j << (p + 1)) + i;
+                const auto r0 = ld2(r - nx), r1 = ld2(r), r2 = ld2(r + nx);
+                yA = T(0.25) * (r0.x + T(2) * r1.x + r2.x);
+                yB = T(0.25) * (r0.y + T(2) * r1.y + r2.y);
+            }
+        }
+        const T vA = (hx && hy) ? T(0.5) * xA + T(0.5) * yA : (hx ? xA : yA);
+        const T vB = (hx && hy) ? T(0.5) * xB + T(0.5) * yB : (hx ? xB : yB);
+        if (op) {
+            const int t = op_index(p, i, j, m.qic);  // unknown of cell A; B is the next one
+            if (i > 0) m.b3[t] = vA;
+            m.b3[t + 1] = vB;
+        } else {
+            if (i > 0) {
+                cb[cA] = vA;
+                cu[cA] = T(0);
+            }
+            cb[cA + 1] = vB;
+            cu[cA + 1] = T(0);
+        }
+    }
+}
+
+// First half of a visit of diagonal d: nu1 sweeps, the residual, Eq. (2.3) into
+// diagonal d-1 (whose correction restarts from zero).  After a black half sweep
+// the residual of a black node is zero up to the rounding of its own update, so
+// only the red nodes' is formed.
+template <class T, int NP>
+__device__ __forceinline__ void mid_pre(const MidItem<T>& m, int d, int nu1, bool zero)
+{
+    const MidDiag<T> g = mid_diag(m, d);
+    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x;
+    Pair<T> P[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) pair_load(P[k], g, d, tid + k * nt, tid + k * nt < np);
+    if (d == 0) {  // one unknown: solved exactly
+        if (P[0].vR) g.u[P[0].cR] = P[0].bR;
+        __syncthreads();
+        return;
+    }
+    mid_sweeps<T, NP>(P, g.u, nu1, zero);
+    if (nu1 > 0) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+            const Pair<T>& a = P[k];
+            if (a.nx) m.r[tid + k * nt] = a.vR ? a.dR * (pair_red(a, g.u) - a.uR) : T(0);
+        }
+        __syncthreads();
+        mid_restrict<T, true>(m, d);
+    } else {
+        for (int k = tid; k < (g.ng << (d + 2)); k += nt) {
+            const int p = g.plo + (k >> (d + 2)), cell = k & ((4 << d) - 1), nx = 1 << p;
+            if ((cell & (nx - 1)) == 0 || cell < nx) continue;
+            const T aw = g.ax[k - 1], ae = g.ax[k], as = g.ay[k - nx], an = g.ay[k];
+            m.r[k] = g.b[k] - ((aw + ae + as + an) * g.u[k] - (aw * g.u[k - 1] + ae * g.u[k + 1]) -
+                               (as * g.u[k - nx] + an * g.u[k + nx]));
+        }
+        __syncthreads();
+        mid_restrict<T, false>(m, d);
+    }
+    __syncthreads();
+}
+
+// Second half: Eq. (2.4) with the kappa weights of Eq. (2.5), then nu2 sweeps.
+// The first red half sweep reads black nodes only and overwrites the red ones, so
+// the correction is formed at the black nodes (at both when nu2 = 0).
+template <class T, int NP>
+__device__ __forceinline__ void mid_post(const MidItem<T>& m, int d, int nu2, T omega)
+{
+    const MidDiag<T> g = mid_diag(m, d);
+    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x;
+    const int plo = mid_plo(d - 1, m.qic);
+    const T* cu = d == m.lo && m.lo > 0 ? m.u3 : mid_diag(m, d - 1).u;
+    Pair<T> P[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int mm = tid + k * nt;
+        Pair<T>& a = P[k];
+        pair_load(a, g, d, mm, mm < np);
+        if (a.nx == 0) continue;
+        const int p = g.plo + (mm >> (d + 1)), q = d + 2 - p, cell = (2 * mm) & ((4 << d) - 1);
+        const int i = cell & (a.nx - 1), j = cell >> p;
+        const bool hx = p > 1, hy = q > 1;
+        T xA = T(0), xB = T(0), yA = T(0), yB = T(0);
+        if (hx) {  // grid (p-1, q): row j, columns i/2 and i/2 + 1
+            const T* c = cu + ((p - 1 - plo) << (d + 1)) + (j << (p - 1)) + (i >> 1);
+            xA = c[0];
+            xB = T(0.5) * (xA + c[1]);
+        }
+        if (hy) {  // grid (p, q-1): rows j/2 and, between two of them, j/2 + 1
+            const T* c = cu + ((p - plo) << (d + 1)) + ((j >> 1) << p) + i;
+            const auto c0 = ld2(c);
+            yA = c0.x;
+            yB = c0.y;
+            if (j & 1) {
+                const auto c1 = ld2(c + a.nx);
+                yA = T(0.5) * (yA + c1.x);
+                yB = T(0.5) * (yB + c1.y);
+            }
+        }
+        const bool redB = a.eR > 0;
+        if (a.vK) {
+            const T x = redB ? xA : xB, y = redB ? yA : yB;
+            T e = hx ? x : y;
+            if (hx && hy) {
+                const T cx = a.pK + a.oK, cy = a.sK + a.nK, x2 = cx * cx, y2 = cy * cy, w = rcp_of(x2 + y2);
+                e = (x2 * w) * x + (y2 * w) * y;
+            }
+            a.uK += omega * e;
+            g.u[a.cR - a.eR] = a.uK;
+        }
+        if (nu2 == 0 && a.vR) {
+            const T x = redB ? xB : xA, y = redB ? yB : yA;
+            T e = hx ? x : y;
+            if (hx && hy) {
+                const T cx = a.pR + a.oR, cy = a.sR + a.nR, x2 = cx * cx, y2 = cy * cy, w = rcp_of(x2 + y2);
+                e = (x2 * w) * x + (y2 * w) * y;
+            }
+            a.uR += omega * e;
+            g.u[a.cR] = a.uR;
+        }
+    }
+    __syncthreads();
+    mid_sweeps<T, NP>(P, g.u, nu2, false);
+}
+
+// u3 = M b3: two threads a row.
+template <class T>
+__device__ __forceinline__ void mid_matrix(const MidItem<T>& m)
+{
+    const int half = m.ld3 >> 1;
+    for (int t2 = threadIdx.x; t2 < ((2 * m.n3 + 31) & ~31); t2 += blockDim.x) {
+        const int t = t2 >> 1, h = t2 & 1;
+        T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
+        if (t < m.n3) {
+            const T* row = m.M + t * m.ld3 + h * half;
+            const T* v = m.b3 + h * half;
+            for (int k = 0; k < half; k += 4) {
+                const auto a = ld2(row + k), b = ld2(row + k + 2), x = ld2(v + k), y = ld2(v + k + 2);
+                s0 += a.x * x.x;
+                s1 += a.y * x.y;
+                s2 += b.x * y.x;
+                s3 += b.y * y.y;
+            }
+        }
+        T s = (s0 + s1) + (s2 + s3);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (h == 0 && t < m.n3) {
+            // cell of unknown t
+            const int plo = mid_plo(kOpD, m.qic);
+            int p = plo, o = t;
+            for (;; ++p) {
+                const int nn = ((1 << p) - 1) * ((1 << (kOpD + 2 - p)) - 1);
+                if (o < nn) break;
+                o -= nn;
+            }
+            const int nx1 = (1 << p) - 1, j = 1 + o / nx1, i = 1 + o - (j - 1) * nx1;
+            m.u3[((p - plo) << (kOpD + 2)) + (j << p) + i] = s;
+        }
+    }
+    __syncthreads();
+}
+
+template <class T>
+__device__ __forceinline__ void mid_pre_any(const MidItem<T>& m, int d, int nu1, bool zero)
+{
+    const int np = mid_cells(d, m.pic, m.qic) >> 1;
+    if (np <= blockDim.x) mid_pre<T, 1>(m, d, nu1, zero);
+    else if (np <= 2 * blockDim.x) mid_pre<T, 2>(m, d, nu1, zero);
+    else mid_pre<T, 4>(m, d, nu1, zero);
+}
+template <class T>
+__device__ __forceinline__ void mid_post_any(const MidItem<T>& m, int d, int nu2, T omega)
+{
+    const int np = mid_cells(d, m.pic, m.qic) >> 1;
+    if (np <= blockDim.x) mid_post<T, 1>(m, d, nu2, omega);
+    else if (np <= 2 * blockDim.x) mid_post<T, 2>(m, d, nu2, omega);
+    else mid_post<T, 4>(m, d, nu2, omega);
+}
+
+// One mu-cycle of Algorithm 1 on diagonal m.hi, the recursion as a loop:
+// `made` counts the calls already made below each diagonal, four bits each.
+// Diagonal 0 does not change between the mu calls of one visit (one unknown,
+// solved exactly), so it is called once.
+template <class T>
+__device__ __forceinline__ void mid_cycle(const MidItem<T>& m, int mu, int nu1, int nu2, T omega, bool zero)
+{
+    int d = m.hi;
+    uint64_t made = 0;
+    for (;;) {
+        mid_pre_any(m, d, nu1, zero);
+        if (d > m.lo) {
+            made &= ~(15ull << (4 * d));
+            zero = true;
+            --d;
+            continue;
+        }
+        if (m.lo > 0) {
+            mid_matrix(m);
+            mid_post_any(m, d, nu2, omega);
+        }
+        for (;;) {
+            if (d == m.hi) return;
+            ++d;
+            made += 1ull << (4 * d);
+            const int k = (int)(made >> (4 * d)) & 15;
+            if (k < (d == 1 ? 1 : mu)) {
+                zero = false;
+                --d;
+                break;
+            }
+            mid_post_any(m, d, nu2, omega);
+        }
+    }
+}
+
+// Coefficients, zeros and the matrix of an item into shared memory.
+template <class T>
+__device__ __forceinline__ void mid_fill(const MidItem<T>& m, const SampleInfo& S, const T* ax, const T* ay, const T* op)
+{
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const MidWords w = mid_words(m.pic, m.qic, m.lo, m.hi, 1);
+    int c0 = 0;
+    for (int d = m.lo; d <= m.hi; ++d) {
+        const int nc = mid_cells(d, m.pic, m.qic), plo = mid_plo(d, m.qic);
+        for (int k = tid; k < nc; k += nt) {
+            const int p = plo + (k >> (d + 2)), cell = k & ((4 << d) - 1);
+            const int i = cell & ((1 << p) - 1), j = cell >> p;
+            const int64_t o = S.node_off + grid_offset(p, d + 2 - p, S.Q) + j * ((1 << p) + 1) + i;
+            m.ax[c0 + k] = ax[o];
+            m.ay[c0 + k] = ay[o];
+        }
+        c0 += nc;
+    }
+    for (int k = tid; k < w.cells + w.pads; k += nt) m.u[k] = T(0);
+    if (m.lo > 0) {
+        const T* M = op + S.op_off + op_offset(m.pic < 4 ? m.pic : 4, m.qic < 4 ? m.qic : 4, S.P, S.Q);
+        for (int k = 2 * tid; k < m.n3 * m.ld3; k += 2 * nt)
+            *reinterpret_cast<typename Vec2<T>::V*>(m.M + k) = ld2(M + k);
+        for (int k = tid; k < kOpN; k += nt) m.b3[k] = T(0);
+        for (int k = tid; k < kU3; k += nt) m.u3[k] = T(0);
+    }
+}
+
+// The mu calls at diagonal kMidD inside a visit of diagonal kMidD + 1 of a larger item.
+template <class T>
+__global__ void __launch_bounds__(kMidThreads, sizeof(T) == 4 ? 3 : 1)
+    k_mid(DevCtx cx, T* su, const T* sbx, const T* sby, const T* ax, const T* ay, const T* op, CycleParams cp)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const TaskRef t = resolve(cx);
+    const SampleInfo& S = cx.samples[t.s];
+    const int pi = t.seg->pi, qi = t.seg->qi;
+    __shared__ int2 at[kMidMax + 1];
+    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, min(pi, kMidD + 1), min(qi, kMidD + 1), kOpD + 1, kMidD, cp.nu1);
+    mid_fill(m, S, ax, ay, op);
+    __syncthreads();
+    const MidDiag<T> g = mid_diag(m, kMidD);
+    const int nc = g.ng << (kMidD + 2), tid = threadIdx.x, nt = blockDim.x;
+    for (int k = tid; k < nc; k += nt) {
+        const int p = g.plo + (k >> (kMidD + 2)), q = kMidD + 2 - p, cell = k & ((4 << kMidD) - 1);
+        const int i = cell & ((1 << p) - 1), j = cell >> p;
+        if (i == 0 || j == 0) continue;
+        const int64_t o = t.scr + grid_offset(p, q, qi) + j * ((1 << p) + 1) + i;
+        const bool hx = p < pi, hy = q < qi;
+        g.b[k] = (hx && hy) ? T(0.5) * sbx[o] + T(0.5) * sby[o] : (hx ? sbx[o] : sby[o]);
+    }
+    __syncthreads();
+    for (int call = 0; call < cp.mu; ++call) mid_cycle(m, cp.mu, cp.nu1, cp.nu2, (T)cp.omega, call == 0);
+    for (int p = g.plo; p < g.plo + g.ng; ++p) {
+        const int q = kMidD + 2 - p, nx = 1 << p, W = nx + 1, n = W * ((1 << q) + 1);
+        T* dst = su + t.scr + grid_offset(p, q, qi);
+        const T* src = g.u + ((p - g.plo) << (kMidD + 2));
+        for (int v = tid; v < n; v += nt) {
+            const int j = v / W, i = v - j * W;
+            dst[v] = src[j * nx + i];  // boundary nodes are zeros of the layout
+        }
+    }
+}
+
+// An item of a low stage, solved whole: Algorithm 2's initial guess, then
+// defect-correction cycles until the residual meets eps (or the item stops), the
+// decision of k_residual word for word.
+template <class T>
+__global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, int L, double* u64, const double* ax64, const double* ay64,
+                                                          const T* ax, const T* ay, const T* op, CycleParams cp, int max_cycles,
+                                                          double eps, int* cycles, double* relres, int* status)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_act;
+    const TaskRef t = resolve(cx);
+    const SampleInfo& S = cx.samples[t.s];
+    const int p = t.seg->pi, q = t.seg->qi, nx = 1 << p, ny = 1 << q, W = nx + 1;
+    const int64_t off = S.node_off + grid_offset(p, q, S.Q);
+    double* u = u64 + off;
+    const double* fx = ax64 + off;
+    const double* fy = ay64 + off;
+    __shared__ int2 at[kMidMax + 1];
+    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, p, q, L > kOpD ? kOpD + 1 : 0, L, cp.nu1);
+    mid_fill(m, S, ax, ay, op);
+    item_guess(S, p, q, u64, ax64, ay64);
+    __syncthreads();
+    const MidDiag<T> g = mid_diag(m, L);
+    const int n = (nx - 1) * (ny - 1);
+    double first = 0.0;
+    for (int step = 0;; ++step) {
+        __syncthreads();
+        double acc = 0.0;
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const int i = 1 + k % (nx - 1), j = 1 + k / (nx - 1), c = j * W + i;
+            const double aw = fx[c - 1], ae = fx[c], as = fy[c - W], an = fy[c];
+            const double Au = (aw + ae + as + an) * u[c] - (aw * u[c - 1] + ae * u[c + 1]) - (as * u[c - W] + an * u[c + W]);
+            const double r = 1.0 - Au;
+            acc += r * r;
+            g.b[(j << p) + i] = (T)r;
+            g.u[(j << p) + i] = T(0);
+        }
+        const double ss = block_sum(acc);
+        if (threadIdx.x == 0) {
+            const double rr = sqrt(ss / (double)n);
+            int act = 1;
+            if (step == 0) first = rr;
+            else if (!(rr == rr) || isinf(rr)) { act = 0; atomicOr(&status[t.s], MSG_SAMPLE_NONFINITE); }
+            else if (rr <= eps) act = 0;
+            else if (step >= max_cycles || (rr > 1.0 && rr > first)) {
+                act = 0;
+                atomicOr(&status[t.s], MSG_SAMPLE_NOT_CONVERGED);
+            }
+            s_act = act;
+            if (!act) {
+                cycles[t.item] = step;
+                relres[t.item] = rr;
+            }
+        }
+        __syncthreads();
+        if (!s_act) return;
+        mid_cycle(m, cp.mu, cp.nu1, cp.nu2, (T)cp.omega, true);
+        for (int k = threadIdx.x; k < n; k += blockDim.x) {
+            const int i = 1 + k % (nx - 1), j = 1 + k / (nx - 1);
+            u[j * W + i] += (double)g.u[(j << p) + i];
+        }
+    }
+}
+
+}  // namespace msg

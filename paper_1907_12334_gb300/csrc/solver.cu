@@ -11,12 +11,15 @@
 // approximately from e = 0 on the item's scratch hierarchy, and u += e in FP64.
 // For a linear cycle this is the same iteration as cycling on (u, 1).
 //
-// Launch structure of one cycle for all active items of a stage: diagonals
-// d > cut of the items' hierarchies are visited by one launch per visit half
-// (PRE: zero/smooth nu1/restrict; POST: prolong/smooth nu2) with one CTA per
-// (item, grid) task; everything at or below the cut runs inside one launch
-// (LOW) in which each warp executes the recursion of Algorithm 1 as a flat
-// program in shared memory for a few items of one shape class in lockstep.
+// Launch structure.  Stages up to kItemL32 (FP64 cycles: kItemL64) are one launch
+// each, an item per CTA from its initial guess to convergence (mid.cuh).  One cycle
+// for all active items of a later stage: diagonals d > cut of the items'
+// hierarchies are visited by one launch per visit half (PRE: zero/smooth
+// nu1/restrict; POST: prolong/smooth nu2); everything at or below the cut runs
+// inside one launch (LOW), k_mid with cut kMidD (mid.cuh).  When the caller sets
+// the cut (tune_low_cut), every stage has this second form and LOW is k_lowv, in
+// which each warp executes the recursion of Algorithm 1 as a flat program in
+// shared memory for a few items of one shape class in lockstep.
 //
 // Storage (all node-indexed with the boundary, see common.cuh):
 //   u64          solution of every grid of every sample (FP64)
@@ -51,6 +54,7 @@ struct SampleInfo {
     int64_t node_off;  // start of the sample's rectangle in u64 / coefficient arrays
     int64_t field_off; // start of the sample's field in Z
     int64_t q_off;     // start of the sample's P*Q outputs
+    int64_t op_off;    // start of its low-diagonal matrices (mid.cuh)
 };
 
 // One launch covers a list of segments; segment i owns blocks
@@ -1411,11 +1415,9 @@ __device__ __forceinline__ double cubic_at(const double* c, int stride, int m, i
     return (-cm1 + 9.0 * c0 + 9.0 * c1 - c2) / 16.0;
 }
 
-__global__ void k_interp(DevCtx cx, double* u64, const double* ax64, const double* ay64)
+__device__ void item_guess(const SampleInfo& S, int p, int q, double* u64, const double* ax64, const double* ay64)
 {
-    TaskRef t = resolve(cx);
-    const SampleInfo& S = cx.samples[t.s];
-    const int p = t.seg->pi, q = t.seg->qi, nx = 1 << p, ny = 1 << q, W = nx + 1;
+    const int nx = 1 << p, ny = 1 << q, W = nx + 1;
     double* u = u64 + S.node_off + grid_offset(p, q, S.Q);
     const double* ax = ax64 + S.node_off + grid_offset(p, q, S.Q);
     const double* ay = ay64 + S.node_off + grid_offset(p, q, S.Q);
@@ -1442,6 +1444,12 @@ __global__ void k_interp(DevCtx cx, double* u64, const double* ax64, const doubl
         }
         u[c] = corr;
     }
+}
+
+__global__ void k_interp(DevCtx cx, double* u64, const double* ax64, const double* ay64)
+{
+    TaskRef t = resolve(cx);
+    item_guess(cx.samples[t.s], t.seg->pi, t.seg->qi, u64, ax64, ay64);
 }
 
 // Block reduction of a double in a fixed order (result valid on thread 0).
@@ -1573,6 +1581,12 @@ __global__ void k_qoi(DevCtx cx, const double* u64, const double* Z, int qoi, do
         if (threadIdx.x == 0) Qout[t.item] = dy * s;
     }
 }
+
+}  // namespace msg
+
+#include "mid.cuh"
+
+namespace msg {
 
 // ------------------------------------------------------------------ plan --
 
@@ -1891,7 +1905,7 @@ struct Plan {
     std::vector<std::vector<ItemType>> stage_items; // [L]
     std::vector<int64_t> stage_nitems;              // [L]: flags (items) of the stage
     std::vector<Segment> all_segs;                  // one segment per grid type over all samples
-    int64_t total_nodes = 0, total_field = 0, total_q = 0, scratch_nodes = 0;
+    int64_t total_nodes = 0, total_field = 0, total_q = 0, total_op = 0, scratch_nodes = 0;
     int64_t max_stage_items = 0, max_segs = 0;
 };
 
@@ -1966,6 +1980,8 @@ void build_plan(const int32_t* PQ, int64_t S, Plan& pl)
         pl.total_nodes += rect_nodes(si.P, si.Q);
         pl.total_field += field_nodes(si.P, si.Q);
         pl.total_q += (int64_t)si.P * si.Q;
+        si.op_off = pl.total_op;
+        pl.total_op += op_offset(0, 0, si.P, si.Q);
         auto key = std::make_pair(si.P, si.Q);
         auto it = gid.find(key);
         if (it == gid.end()) {
@@ -2033,7 +2049,27 @@ void build_plan(const int32_t* PQ, int64_t S, Plan& pl)
     }
 }
 
+// The cycles run on chip (mid.cuh) unless the caller sets the cut of the
+// low-diagonal kernel: that keeps the recursion below the cut as phases.
+bool on_chip(const msg_params& prm) { return prm.tune_low_cut == 0; }
+// highest stage solved by k_item (-1: none)
+int item_stages(const msg_params& prm) { return !on_chip(prm) ? -1 : prm.precision == MSG_PREC_MIXED ? kItemL32 : kItemL64; }
+// shared memory of the largest item of a stage, and of k_mid
+size_t item_smem(int L, const msg_params& prm)
+{
+    const size_t es = prm.precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
+    int most = 0;
+    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, L, prm.nu1));
+    return es * most;
+}
+size_t mid_smem(const msg_params& prm)
+{
+    const size_t es = prm.precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
+    return es * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kMidD, prm.nu1);
+}
+
 struct WsLayout {
+    size_t op;  // low-diagonal matrices (mid.cuh)
     size_t samples, perm, gpos, groups, allsegs;
     size_t nstep, cycles_i, relres_i;
     size_t u64, ax64, ay64, ax32, ay32;
@@ -2059,7 +2095,7 @@ WsLayout layout_of(const Plan& pl, const msg_params& prm)
         std::vector<LowDesc> desc;
         w.low_desc = take(sizeof(LowDesc) * kLowClassesMax);
         w.low_ent = take(sizeof(uint4) * low_tables().ent.size());
-        w.low_prog = take(sizeof(uint2) * low_resolve(prm, desc).size());
+        w.low_prog = take(sizeof(uint2) * low_resolve(prm, desc, !on_chip(prm)).size());
     }
     {
         const LowPlanes& lp = low_tables().planes[kLowMax];
@@ -2077,10 +2113,12 @@ WsLayout layout_of(const Plan& pl, const msg_params& prm)
         w.ax32 = take(sizeof(float) * pl.total_nodes);
         w.ay32 = take(sizeof(float) * pl.total_nodes);
     }
+    if (on_chip(prm)) w.op = take(es * pl.total_op);
     for (int L = 0; L <= pl.Lmax; ++L) {
         int64_t nseg = 0, scr = 0;
         for (const ItemType& it : pl.stage_items[L]) nseg += 1 + (int64_t)it.pi * it.qi;
-        for (const Group& g : pl.stage_groups[L]) scr += g.scr_per_sample * g.count;
+        if (L > item_stages(prm))
+            for (const Group& g : pl.stage_groups[L]) scr += g.scr_per_sample * g.count;
         w.segs.push_back(take(sizeof(Segment) * nseg));
         w.tasks.push_back(take(sizeof(LowTask) * (pl.stage_nitems[L] + pl.stage_items[L].size() * kLowWarpsMax)));
         w.slist.push_back(take(sizeof(int) * pl.stage_nitems[L]));
@@ -2153,7 +2191,15 @@ struct SolveCtx {
     const LowDesc* low_desc;
     const uint4* low_ent;
     const uint2* low_prog;  // resolved programs of all classes
+    int op_pcap;            // program words of the longest class of diagonal kOpD, even
 };
+
+// Threads per CTA of k_item: a thread holds at most four pairs of a diagonal.
+template <class T>
+static int item_threads(int L)
+{
+    return L <= 2 ? 32 : L <= 4 ? 64 : L <= 6 ? 128 : 256;
+}
 
 // Stage L of FMSG for the samples handed over by stage L-1: cubic
 // interpolation when a sample enters, then defect-correction cycles of every
@@ -2176,7 +2222,8 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
     int* counter = (int*)(C.ws + wl.counter[L]);
     Segment* dsegs = (Segment*)(C.ws + wl.segs[L]);
     LowTask* dtasks = (LowTask*)(C.ws + wl.tasks[L]);
-    const int cut = C.low.cut;
+    const bool chip = on_chip(C.prm);
+    const int cut = chip ? kMidD : C.low.cut;
     const double es = sizeof(T);
 
     // item types of each group at this stage, and per-sample countdown of open items
@@ -2235,7 +2282,7 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
             // (the warps of a CTA take tasks of one segment: idle warps pad each segment's last CTA)
             ntasks = 0;
             low_flops = 0;
-            for (size_t k = 0; k < ns; ++k) {
+            for (size_t k = 0; k < ns && !chip; ++k) {
                 const Segment& sgk = h_segs[k];
                 const int cls = low_class(std::min(sgk.pi, dl + 1), std::min(sgk.qi, dl + 1), dl);
                 low_flops += (double)sgk.count * C.low.flops[cls];
@@ -2404,6 +2451,14 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
         DevCtx ic = ctx_of(0, item_nseg);
         bool launch_err = false;
         auto launch_low = [&](int d, int calls) {
+            if (chip) {
+                prof_begin(K_LOW, st);
+                k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem(C.prm), st>>>(
+                    ic, su, sbx, sby, C.ax, C.ay, (const T*)(C.ws + wl.op), C.cp);
+                prof_end(K_LOW, st, low_bytes, 0.0, d);
+                launch_err |= cudaGetLastError() != cudaSuccess;
+                return;
+            }
             if (ntasks == 0) return;
             const LowPlanes& lp = low_tables().planes[d];
             const int wpb = C.low.warps;
@@ -2516,6 +2571,57 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
     return finish(MSG_OK);
 }
 
+// Matrices of the low diagonals, then stages 0 .. nlow-1, each one launch of
+// k_item over the stage's items of every sample.
+template <class T>
+static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
+{
+    const Plan& pl = C.pl;
+    T* op = (T*)(C.ws + C.wl.op);
+    for (int c = 0; c < kOpClasses; ++c) {
+        const int pic = op_pic(c), qic = op_qic(c), n = op_n(pic, qic);
+        bool any = false;
+        for (const Group& g : pl.groups) any |= op_has(pic, qic, g.P, g.Q);
+        if (!any) continue;
+        const LowPlanes& lp = low_tables().planes[kOpD];
+        const LowPlanes& lpm = low_tables().planes[kLowMax];
+        const dim3 blk((n + 31) / 32 * 32, 768 / ((n + 31) / 32 * 32));
+        const size_t smem = sizeof(uint4) * C.low.ecap[kOpD] + sizeof(uint2) * C.op_pcap +
+                            sizeof(T) * (lp.nfx + lp.nfy + (size_t)(2 * lp.nu + lp.nr) * n);
+        prof_begin(K_COEFFS, st);
+        k_lowop<T><<<(unsigned)pl.S, blk, smem, st>>>(C.base.samples, pic, qic, (const T*)(C.ws + C.wl.low_img),
+                                                     lpm.nfx + lpm.nfy, lpm.nfx, C.low_desc, C.low_ent, C.low_prog, lp,
+                                                     C.prm.mu, (T)C.prm.omega, op);
+        prof_end(K_COEFFS, st, 0.0, 0.0);
+        MSG_CHECK_LAUNCH();
+    }
+    for (int L = 0; L < nlow; ++L) {
+        std::vector<Segment> segs;
+        int64_t b = 0;
+        double work = 0;
+        for (const ItemType& it : pl.stage_items[L]) {
+            const Group& g = pl.groups[it.g];
+            segs.push_back(Segment{it.g, it.pi, it.qi, it.pi, it.qi, b, g.count, g.start, it.scr_slot, it.stage_base});
+            b += g.count;
+            work += (double)g.count * pts(it.pi, it.qi);
+        }
+        if (b == 0) continue;
+        MSG_CUDA_TRY(cudaMemcpyAsync(C.ws + C.wl.segs[L], segs.data(), sizeof(Segment) * segs.size(), cudaMemcpyHostToDevice, st));
+        DevCtx c = C.base;
+        c.slist = (const int*)(C.ws + C.wl.perm);
+        c.groups = C.dgroups + pl.groups.size() * (1 + L);
+        c.segs = (const Segment*)(C.ws + C.wl.segs[L]);
+        c.nseg = (int)segs.size();
+        prof_begin(K_LOW, st);
+        k_item<T><<<(unsigned)b, item_threads<T>(L), item_smem(L, C.prm), st>>>(
+            c, L, C.u64, C.ax64, C.ay64, C.ax, C.ay, op, C.cp, C.prm.max_cycles, C.prm.eps, C.cyc, C.rel, C.stat);
+        prof_end(K_LOW, st, work * 40.0, 0.0, L);
+        MSG_CHECK_LAUNCH();
+        MSG_CUDA_TRY(cudaStreamSynchronize(st));
+    }
+    return MSG_OK;
+}
+
 template <class T>
 static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_params& prm, const double* Z,
                      double* Qout, int32_t* stat, int32_t* cycles_out, double* relres_out, cudaStream_t st)
@@ -2535,7 +2641,7 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
                   (int*)(ws + wl.nstep), (int*)(ws + wl.cycles_i), (double*)(ws + wl.relres_i),
                   CycleParams{prm.mu, prm.nu1, prm.nu2, prm.omega}, prm.tune_block ? prm.tune_block : kVisitThreads,
                   (size_t)(prm.tune_visit_smem ? prm.tune_visit_smem : kVisitSmemKB) * 1024, low_shape(prm), (const LowDesc*)(ws + wl.low_desc), (const uint4*)(ws + wl.low_ent),
-                  (const uint2*)(ws + wl.low_prog)};
+                  (const uint2*)(ws + wl.low_prog), 0};
     float* ax32 = mixed ? (float*)(ws + wl.ax32) : nullptr;
     float* ay32 = mixed ? (float*)(ws + wl.ay32) : nullptr;
     C.ax = mixed ? (const T*)ax32 : (const T*)(ws + wl.ax64);
@@ -2571,13 +2677,15 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
         // tables of the low-diagonal program: class descriptors, node entries, programs
         const LowTables& lt = low_tables();
         std::vector<LowDesc> desc;
-        const std::vector<uint2> rp = low_resolve(prm, desc);
+        const std::vector<uint2> rp = low_resolve(prm, desc, !on_chip(prm));
         MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_desc, desc.data(), sizeof(LowDesc) * desc.size(),
                                      cudaMemcpyHostToDevice, st));
         MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_ent, lt.ent.data(), sizeof(uint4) * lt.ent.size(),
                                      cudaMemcpyHostToDevice, st));
         MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_prog, rp.data(), sizeof(uint2) * rp.size(),
                                      cudaMemcpyHostToDevice, st));
+        for (const LowDesc& D : desc)
+            if (D.dl == kOpD) C.op_pcap = std::max(C.op_pcap, (D.nops + 1) & ~1);
         // the sources are host vectors: finish the copies before they go out of scope
         MSG_CUDA_TRY(cudaStreamSynchronize(st));
     }
@@ -2593,23 +2701,33 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_item<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
     MSG_CUDA_TRY(cudaStreamSynchronize(st));
 
-    // ---- one worker (host thread + stream) per stage
-    const int nst = pl.Lmax + 1;
+    // ---- low stages on chip, one launch each (the stream orders a stage after its children's)
+    const int nst = pl.Lmax + 1, nlow = std::min(nst, item_stages(prm) + 1);
+    if (on_chip(prm)) {
+        int rc = low_stages<T>(C, nlow, st);
+        if (rc != MSG_OK) return rc;
+    }
+
+    // ---- one worker (host thread + stream) per further stage
     StageQueues Qs;
     Qs.ready.assign(nst, {});
     Qs.done.assign(nst, 0);
-    Qs.ready[0] = pl.perm;
+    for (int L = 0; L < nlow; ++L) Qs.done[L] = 1;
+    if (nlow < nst) Qs.ready[nlow] = pl.perm;
     std::vector<cudaStream_t> streams(nst, nullptr);
-    for (int L = 0; L < nst; ++L) MSG_CUDA_TRY(cudaStreamCreateWithFlags(&streams[L], cudaStreamNonBlocking));
+    for (int L = nlow; L < nst; ++L) MSG_CUDA_TRY(cudaStreamCreateWithFlags(&streams[L], cudaStreamNonBlocking));
     std::vector<int> rcs(nst, MSG_OK);
     std::vector<std::string> errs(nst);
     int dev = 0;
     cudaGetDevice(&dev);
     {
         std::vector<std::thread> th;
-        for (int L = 0; L < nst; ++L)
+        for (int L = nlow; L < nst; ++L)
             th.emplace_back([&, L] {
                 cudaSetDevice(dev);
                 rcs[L] = stage_worker<T>(C, L, Qs, streams[L]);
@@ -2617,8 +2735,8 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
             });
         for (auto& t : th) t.join();
     }
-    for (int L = 0; L < nst; ++L) cudaStreamDestroy(streams[L]);
-    for (int L = 0; L < nst; ++L)
+    for (int L = nlow; L < nst; ++L) cudaStreamDestroy(streams[L]);
+    for (int L = nlow; L < nst; ++L)
         if (rcs[L] != MSG_OK) { set_error("stage " + std::to_string(L) + ": " + errs[L]); return rcs[L]; }
 
     // ---- QoI of every grid

@@ -1,0 +1,48 @@
+"""The on-chip cycles (csrc/mid.cuh) against the phase-by-phase kernels.
+
+``tune_low_cut`` = 4 keeps the recursion below diagonal 4 as table phases and
+every stage on the host schedule; the default runs stages up to 9 (FP64: 8) whole
+in one kernel, the recursion below diagonal 6 of larger items in another, and the
+calls on diagonal 3 as one matrix.  Both iterate every grid to the same residual,
+so Q agrees to what that residual allows (1e-8 relative, the mixed path's
+tolerance; FP64 cycles 1e-10), and the cycle counts to one cycle wherever eps lies
+above the rounding floor of the FP64 residual (below it, rounding decides the stop):
+the floor is 2^-52 |A| |u| with |A| <= 2 a_max (4^p + 4^q) and |u| <= 1 / (8 a_min).
+"""
+import numpy as np
+import pytest
+
+from paper_1907_12334_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+DEV = "cuda:0"
+
+# one-column and one-row hierarchies, each clipped triangle of the matrix, the
+# last stage of k_item and the first ones after it, wide and tall
+SHAPES = [(1, 1), (1, 5), (5, 1), (2, 4), (4, 2), (3, 3), (4, 5), (5, 6), (1, 10), (10, 1), (6, 6), (7, 5), (2, 9)]
+
+
+@pytest.mark.parametrize("mu,nu1,nu2,precision", [(2, 2, 2, "MIXED"), (1, 1, 1, "MIXED"), (3, 2, 1, "MIXED"),
+                                                  (2, 0, 3, "MIXED"), (2, 3, 0, "MIXED"), (2, 2, 2, "FP64"),
+                                                  (1, 0, 2, "FP64")])
+def test_on_chip_cycles_match_the_phase_kernels(mu, nu1, nu2, precision):
+    from paper_1907_12334_gb300 import build, msg
+
+    build.build()
+    Z = torch.from_numpy(np.concatenate([inputs.smooth_field(P, Q, 1.5) for P, Q in SHAPES])).to(DEV)
+    pq = np.array(SHAPES, dtype=np.int32)
+    kw = dict(mu=mu, nu1=nu1, nu2=nu2, eps=1e-11, max_cycles=400, precision=getattr(msg, f"MSG_PREC_{precision}"))
+    a = [t.cpu().numpy() for t in msg.solve(pq, Z, msg.SolverParams(**kw))]
+    b = [t.cpu().numpy() for t in msg.solve(pq, Z, msg.SolverParams(tune_low_cut=4, **kw))]
+    assert np.array_equal(a[1], b[1])
+    np.testing.assert_allclose(a[0], b[0], rtol=1e-8 if precision == "MIXED" else 1e-10)
+    k = 0
+    for P, Q in SHAPES:
+        contrast = np.exp(np.ptp(inputs.smooth_field(P, Q, 1.5)))
+        for p in range(1, P + 1):
+            for q in range(1, Q + 1):
+                floor = 2.0 ** -52 * 2 * contrast * (4.0 ** p + 4.0 ** q) / 8
+                assert floor > kw["eps"] or abs(int(a[2][k]) - int(b[2][k])) <= 1, (P, Q, p, q)
+                k += 1
