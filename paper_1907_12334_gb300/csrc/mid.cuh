@@ -99,13 +99,13 @@ __host__ __device__ inline int op_index(int p, int i, int j, int qic)
 // residual-to-residual step of the solve.
 template <class T>
 __global__ void __launch_bounds__(768) k_lowop(const SampleInfo* samples, int pic, int qic, const T* img, int64_t istride,
-                                              int ify, const LowDesc* descs, const uint4* ent, const uint2* rprog,
+                                              int ify, const LowDesc* desc, const uint4* ent, const uint2* rprog,
                                               LowPlanes lp, int mu, T omega, T* op)
 {
     const SampleInfo S = samples[blockIdx.x];
     if (!op_has(pic, qic, S.P, S.Q)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const LowDesc& D = descs[low_class(pic, qic, kOpD)];
+    const LowDesc& D = *desc;
     const int n = op_n(pic, qic), ld = op_ld(n), nc = n, nent = D.e1 - D.e0, nops = D.nops;
     uint4* sent = (uint4*)smem_raw;
     uint2* sprog = (uint2*)(sent + nent);
@@ -186,18 +186,56 @@ __global__ void __launch_bounds__(768) k_lowop(const SampleInfo* samples, int pi
 
 // ------------------------------------------------------------------ visits --
 
+// An array of T in shared memory by its 32-bit address: element addresses are one
+// integer add, and an access is one instruction with an immediate offset.  (Through
+// C++ pointers the visits spent 90 % of their instructions on 64-bit address
+// arithmetic and control.)
+template <class T> struct Vec2;
+template <> struct Vec2<float> { typedef float2 V; };
+template <> struct Vec2<double> { typedef double2 V; };
+template <class T>
+struct Sm {
+    uint32_t a;
+    typedef typename Vec2<T>::V V;
+    __device__ __forceinline__ Sm at(int i) const { return Sm{a + (uint32_t)i * (uint32_t)sizeof(T)}; }
+    __device__ __forceinline__ T ld() const
+    {
+        T v;
+        if constexpr (sizeof(T) == 4) asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+        else asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+        return v;
+    }
+    __device__ __forceinline__ V ld2() const  // two elements, 2 sizeof(T) aligned
+    {
+        V v;
+        if constexpr (sizeof(T) == 4) asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+        else asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+        return v;
+    }
+    __device__ __forceinline__ void st(T v) const
+    {
+        if constexpr (sizeof(T) == 4) asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+        else asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+    }
+    __device__ __forceinline__ void st2(T x, T y) const
+    {
+        if constexpr (sizeof(T) == 4) asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(x), "f"(y) : "memory");
+        else asm volatile("st.shared.v2.f64 [%0], {%1, %2};" ::"r"(a), "d"(x), "d"(y) : "memory");
+    }
+};
+
 // One item's hierarchy (pic, qic: its top grid clipped to the diagonals held)
 // on chip: diagonals lo..hi; below lo (when lo = kOpD + 1) the matrix.
 template <class T>
 struct MidItem {
-    T* u;   // per diagonal: cells of its grids, then a pad of zeros (the last grid's north boundary)
-    T* b;   // cells
-    T* ax;  // cells
-    T* ay;
-    T* r;   // residual of the diagonal being restricted: the red node of each pair (every cell when nu1 = 0)
-    T* M;   // the matrix (lo = kOpD + 1)
-    T* b3;  // its right-hand side, compact
-    T* u3;  // its result: the cells of diagonal kOpD
+    Sm<T> u;   // per diagonal: cells of its grids, then a pad of zeros (the last grid's north boundary)
+    Sm<T> b;   // cells
+    Sm<T> ax;  // cells
+    Sm<T> ay;
+    Sm<T> r;   // residual of the diagonal being restricted: the red node of each pair (every cell when nu1 = 0)
+    Sm<T> M;   // the matrix (lo = kOpD + 1)
+    Sm<T> b3;  // its right-hand side, compact
+    Sm<T> u3;  // its result: the cells of diagonal kOpD
     const int2* at;  // first word of each diagonal in b, ax, ay (x) and in u (y)
     int pic, qic, lo, hi;
     int n3, ld3;
@@ -247,14 +285,14 @@ __device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic
     m.pic = pic; m.qic = qic; m.lo = lo; m.hi = hi;
     m.n3 = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
     m.ld3 = op_ld(m.n3);
-    m.M = sm;
-    m.b3 = m.M + (lo > 0 ? m.n3 * m.ld3 : 0);
-    m.u3 = m.b3 + (lo > 0 ? kOpN : 0);
-    m.ax = m.u3 + (lo > 0 ? kU3 : 0);
-    m.ay = m.ax + w.cells;
-    m.b = m.ay + w.cells;
-    m.r = m.b + w.cells;
-    m.u = m.r + w.r;
+    m.M = Sm<T>{(uint32_t)__cvta_generic_to_shared(sm)};
+    m.b3 = m.M.at(lo > 0 ? m.n3 * m.ld3 : 0);
+    m.u3 = m.b3.at(lo > 0 ? kOpN : 0);
+    m.ax = m.u3.at(lo > 0 ? kU3 : 0);
+    m.ay = m.ax.at(w.cells);
+    m.b = m.ay.at(w.cells);
+    m.r = m.b.at(w.cells);
+    m.u = m.r.at(w.r);
     m.at = at;
     if (threadIdx.x == 0) {
         int c = 0, pad = 0;
@@ -267,13 +305,10 @@ __device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic
     return m;
 }
 
-// pointers of one diagonal
+// arrays of one diagonal
 template <class T>
 struct MidDiag {
-    T* u;
-    T* b;
-    const T* ax;
-    const T* ay;
+    Sm<T> u, b, ax, ay;
     int plo, ng;
 };
 template <class T>
@@ -281,102 +316,118 @@ __device__ __forceinline__ MidDiag<T> mid_diag(const MidItem<T>& m, int d)
 {
     MidDiag<T> v;
     const int2 o = m.at[d];
-    v.u = m.u + o.y;
-    v.b = m.b + o.x;
-    v.ax = m.ax + o.x;
-    v.ay = m.ay + o.x;
+    v.u = m.u.at(o.y);
+    v.b = m.b.at(o.x);
+    v.ax = m.ax.at(o.x);
+    v.ay = m.ay.at(o.x);
     v.plo = mid_plo(d, m.qic);
     v.ng = mid_phi(d, m.pic) - v.plo + 1;
     return v;
 }
 
-template <class T> struct Vec2;
-template <> struct Vec2<float> { typedef float2 V; };
-template <> struct Vec2<double> { typedef double2 V; };
-template <class T>
-__device__ __forceinline__ typename Vec2<T>::V ld2(const T* p) { return *reinterpret_cast<const typename Vec2<T>::V*>(p); }
-
-// A thread's pair of cells during a visit: the red and the black node.  The
+// A thread's pair of nodes during a visit: the red and the black one.  The
 // coefficients and b are divided by the node's diagonal, so that an update is
 // u = b + sum a u and the residual is diagonal * (b + sum a u - u); the kappa
 // weights, ratios of squared coefficients of one node, do not see the division.
+// A boundary node takes part with zero coefficients and stays zero, so the half
+// sweeps have no branches; a pair of row 0 or past the end keeps both
+// nodes on one zero word (eR = nx = 0).
 template <class T>
 struct Pair {
     T pR, oR, sR, nR, bR, uR;  // red: face to the partner, outer horizontal, south and north face
     T pK, oK, sK, nK, bK, uK;  // black
     T dR;                      // diagonal of the red node
-    int cR;                    // its cell (relative to the diagonal); the black node's: cR - eR
-    int eR;                    // outer horizontal neighbour of the red node: cR + eR; of the black one: cR - 2 eR
-    int nx;                    // row stride; 0: no node (row 0)
-    bool vR, vK;
+    uint32_t aR;               // address of u at the red node; the black one's: aR - e
+    uint32_t e;                // bytes to the red node's outer horizontal neighbour (the black one's: -e)
+    uint32_t w;                // bytes of a row
 };
 
+// From the faces and values of nodes A (even column, u at address aA) and B: aw, am,
+// ae the faces west of A, between, east of B; s, n the south and north ones.  ok: a row
+// of nodes; hasA: A is not the west boundary; redB: B is the red node.
 template <class T>
-__device__ __forceinline__ void pair_load(Pair<T>& P, const MidDiag<T>& g, int d, int m, bool in)
+__device__ __forceinline__ void pair_set(Pair<T>& P, uint32_t aA, int nx, bool ok, bool hasA, bool redB, T aw, T am, T ae,
+                                         T sA, T sB, T nA, T nB, T bA, T bB, T uA, T uB)
 {
-    const int cA = 2 * m, p = g.plo + (m >> (d + 1)), cell = cA & ((4 << d) - 1);
-    const int i = cell & ((1 << p) - 1), j = cell >> p;
-    P.vR = P.vK = false;
-    P.cR = P.eR = P.nx = 0;
-    P.pR = P.oR = P.sR = P.nR = P.bR = P.uR = P.pK = P.oK = P.sK = P.nK = P.bK = P.uK = P.dR = T(0);
-    if (!in || j == 0) return;
-    const int nx = 1 << p;
-    const bool hasA = i > 0, redB = j & 1;  // cell (i, j), i even, is red when j is even
-    const T aw = g.ax[cA - 1];              // (i = 0: the last face of the row below, not used)
-    const auto ae = ld2(g.ax + cA), an = ld2(g.ay + cA), as = ld2(g.ay + cA - nx), bb = ld2(g.b + cA), uu = ld2(g.u + cA);
-    const T dA = aw + ae.x + as.x + an.x, dB = ae.x + ae.y + as.y + an.y;
-    const T iA = hasA ? rcp_of(dA) : T(0), iB = rcp_of(dB), iR = redB ? iB : iA, iK = redB ? iA : iB;
-    P.nx = nx;
-    P.cR = cA + (redB ? 1 : 0);
-    P.eR = redB ? 1 : -1;
-    P.vR = redB || hasA;
-    P.vK = !redB || hasA;
+    constexpr uint32_t es = sizeof(T);
+    const T dA = aw + am + sA + nA, dB = am + ae + sB + nB;
+    const T iA = hasA ? rcp_of(dA) : T(0), iB = ok ? rcp_of(dB) : T(0), iR = redB ? iB : iA, iK = redB ? iA : iB;
+    P.w = ok ? nx * es : 0u;
+    P.aR = aA + (ok && redB ? es : 0u);
+    P.e = ok ? (redB ? es : 0u - es) : 0u;
     P.dR = redB ? dB : dA;
-    P.pR = iR * ae.x; P.pK = iK * ae.x;
-    P.oR = iR * (redB ? ae.y : aw); P.oK = iK * (redB ? aw : ae.y);
-    P.sR = iR * (redB ? as.y : as.x); P.sK = iK * (redB ? as.x : as.y);
-    P.nR = iR * (redB ? an.y : an.x); P.nK = iK * (redB ? an.x : an.y);
-    P.bR = iR * (redB ? bb.y : bb.x); P.bK = iK * (redB ? bb.x : bb.y);
-    P.uR = redB ? uu.y : uu.x; P.uK = redB ? uu.x : uu.y;
+    P.pR = iR * am; P.pK = iK * am;
+    P.oR = iR * (redB ? ae : aw); P.oK = iK * (redB ? aw : ae);
+    P.sR = iR * (redB ? sB : sA); P.sK = iK * (redB ? sA : sB);
+    P.nR = iR * (redB ? nB : nA); P.nK = iK * (redB ? nA : nB);
+    P.bR = iR * (redB ? bB : bA); P.bK = iK * (redB ? bA : bB);
+    P.uR = redB ? uB : uA; P.uK = redB ? uA : uB;
+}
+
+// Pair m of diagonal d; dump: the zero word for pairs past the end.
+template <class T>
+__device__ __forceinline__ void pair_load(Pair<T>& P, const MidDiag<T>& g, int d, int m, int np, int dump)
+{
+    const bool in = m < np;
+    const int cA = in ? 2 * m : dump, p = g.plo + (in ? m >> (d + 1) : 0), cell = cA & ((4 << d) - 1);
+    const int nx = 1 << p, i = cell & (nx - 1), j = cell >> p;
+    const bool ok = in && j > 0, hasA = ok && i > 0, redB = j & 1;  // (i, j), i even, is red when j is even
+    const int c = ok ? cA : 1 << g.plo;  // any node's cell where there is none
+    const Sm<T> x = g.ax.at(c), y = g.ay.at(c);
+    const T aw = x.at(-1).ld();
+    const auto ae = x.ld2(), an = y.ld2(), as = y.at(ok ? -nx : 0).ld2(), bb = g.b.at(c).ld2(), uu = g.u.at(c).ld2();
+    pair_set(P, g.u.at(cA).a, nx, ok, hasA, redB, aw, ae.x, ae.y, as.x, as.y, an.x, an.y, bb.x, bb.y, ok ? uu.x : T(0),
+             ok ? uu.y : T(0));
 }
 
 // b + sum a u of the red / black node
 template <class T>
-__device__ __forceinline__ T pair_red(const Pair<T>& a, const T* u)
+__device__ __forceinline__ T pair_red(const Pair<T>& a)
 {
-    return a.bR + ((a.pR * a.uK + a.oR * u[a.cR + a.eR]) + (a.sR * u[a.cR - a.nx] + a.nR * u[a.cR + a.nx]));
+    const T o = Sm<T>{a.aR + a.e}.ld(), s = Sm<T>{a.aR - a.w}.ld(), n = Sm<T>{a.aR + a.w}.ld();
+    return a.bR + ((a.pR * a.uK + a.oR * o) + (a.sR * s + a.nR * n));
 }
 template <class T>
-__device__ __forceinline__ T pair_black(const Pair<T>& a, const T* u)
+__device__ __forceinline__ T pair_black(const Pair<T>& a)
 {
-    const int c = a.cR - a.eR;
-    return a.bK + ((a.pK * a.uR + a.oK * u[c - a.eR]) + (a.sK * u[c - a.nx] + a.nK * u[c + a.nx]));
+    const uint32_t k = a.aR - a.e;
+    const T o = Sm<T>{k - a.e}.ld(), s = Sm<T>{k - a.w}.ld(), n = Sm<T>{k + a.w}.ld();
+    return a.bK + ((a.pK * a.uR + a.oK * o) + (a.sK * s + a.nK * n));
 }
 
 // nu red-black Gauss-Seidel sweeps over the thread's pairs; zero: u is zero on
-// entry, so the first red half sweep has no neighbours to read.
+// entry, so the first red half sweep has no neighbours to read.  A half sweep reads
+// nodes of the other colour only: all its loads come before its stores.
+// on: bit k, this warp has pairs in round k (the same for its lanes).
 template <class T, int NP>
-__device__ __forceinline__ void mid_sweeps(Pair<T> (&P)[NP], T* u, int nu, bool zero)
+__device__ __forceinline__ void mid_sweeps(Pair<T> (&P)[NP], uint32_t on, int nu, bool zero)
 {
     for (int s = 0; s < nu; ++s) {
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            Pair<T>& a = P[k];
-            if (!a.vR) continue;
-            a.uR = zero ? a.bR : pair_red(a, u);
-            u[a.cR] = a.uR;
-        }
+        for (int k = 0; k < NP; ++k)
+            if (on >> k & 1) P[k].uR = zero ? P[k].bR : pair_red(P[k]);
+#pragma unroll
+        for (int k = 0; k < NP; ++k)
+            if (on >> k & 1) Sm<T>{P[k].aR}.st(P[k].uR);
         zero = false;
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < NP; ++k) {
-            Pair<T>& a = P[k];
-            if (!a.vK) continue;
-            a.uK = pair_black(a, u);
-            u[a.cR - a.eR] = a.uK;
-        }
+        for (int k = 0; k < NP; ++k)
+            if (on >> k & 1) P[k].uK = pair_black(P[k]);
+#pragma unroll
+        for (int k = 0; k < NP; ++k)
+            if (on >> k & 1) Sm<T>{P[k].aR - P[k].e}.st(P[k].uK);
         __syncthreads();
     }
+}
+
+template <int NP>
+__device__ __forceinline__ uint32_t pairs_of_warp(int np)
+{
+    uint32_t on = 0;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) on |= (uint32_t)((threadIdx.x & ~31) + k * blockDim.x < np) << k;
+    return on;
 }
 
 // Eq. (2.3) into the children of diagonal d from m.r.  RED: m.r holds the red
@@ -387,12 +438,8 @@ __device__ __forceinline__ void mid_restrict(const MidItem<T>& m, int d)
 {
     const int pplo = mid_plo(d, m.qic), plo = mid_plo(d - 1, m.qic), ngc = mid_phi(d - 1, m.pic) - plo + 1;
     const bool op = d == m.lo && m.lo > 0;
-    T *cb = nullptr, *cu = nullptr;
-    if (!op) {
-        const MidDiag<T> c = mid_diag(m, d - 1);
-        cb = c.b;
-        cu = c.u;
-    }
+    const int2 o = m.at[op ? d : d - 1];
+    const Sm<T> cb = m.b.at(o.x), cu = m.u.at(o.y);  // not used when op
     for (int k = threadIdx.x; k < (ngc << d); k += blockDim.x) {
         // cells A = (i, j), i even, and B = (i + 1, j) of child (p, q)
         const int cA = 2 * k, p = plo + (k >> d), q = d + 1 - p, cell = cA & ((2 << d) - 1);
@@ -402,50 +449,42 @@ __device__ __forceinline__ void mid_restrict(const MidItem<T>& m, int d)
         T xA = T(0), xB = T(0), yA = T(0), yB = T(0);
         if constexpr (RED) {
             if (hx) {  // grid (p+1, q): row j has nx pairs, around columns 2i and 2i + 2
-                const T* r = m.r + ((p + 1 - pplo) << (d + 1)) + (j << p) + i;
-                const T r0 = r[0], r1 = r[1];
-                if (j & 1) {
-                    xA = T(0.25) * (r[-1] + r0);
-                    xB = T(0.25) * (r0 + r1);
-                } else {
-                    xA = T(0.5) * r0;
-                    xB = T(0.5) * r1;
-                }
+                const Sm<T> r = m.r.at(((p + 1 - pplo) << (d + 1)) + (j << p) + i);
+                const T rm = r.at(-1).ld(), r0 = r.ld(), r1 = r.at(1).ld();
+                xA = (j & 1) ? T(0.25) * (rm + r0) : T(0.5) * r0;
+                xB = (j & 1) ? T(0.25) * (r0 + r1) : T(0.5) * r1;
             }
             if (hy) {  // grid (p, q+1): rows 2j - 1 .. 2j + 1 of nx / 2 pairs
                 const int h = nx >> 1;
-                const T* r = m.r + ((p - pplo) << (d + 1)) + j * nx + (i >> 1);
-                yA = T(0.5) * r[0];
-                yB = T(0.25) * (r[-h] + r[h]);
+                const Sm<T> r = m.r.at(((p - pplo) << (d + 1)) + j * nx + (i >> 1));
+                yA = T(0.5) * r.ld();
+                yB = T(0.25) * (r.at(-h).ld() + r.at(h).ld());
             }
         } else {
             if (hx) {
-                const T* r = m.r + ((p + 1 - pplo) << (d + 2)) + (j << (p + 1)) + 2 * i;
-                const T rm = r[-1];
-                const auto r0 = ld2(r), r2 = ld2(r + 2);
+                const Sm<T> r = m.r.at(((p + 1 - pplo) << (d + 2)) + (j << (p + 1)) + 2 * i);
+                const T rm = r.at(-1).ld();
+                const auto r0 = r.ld2(), r2 = r.at(2).ld2();
                 xA = T(0.25) * (rm + T(2) * r0.x + r0.y);
                 xB = T(0.25) * (r0.y + T(2) * r2.x + r2.y);
             }
             if (hy) {
-                const T* r = m.r + ((p - pplo) << (d + 2)) + (j << (p + 1)) + i;
-                const auto r0 = ld2(r - nx), r1 = ld2(r), r2 = ld2(r + nx);
+                const Sm<T> r = m.r.at(((p - pplo) << (d + 2)) + (j << (p + 1)) + i);
+                const auto r0 = r.at(-nx).ld2(), r1 = r.ld2(), r2 = r.at(nx).ld2();
                 yA = T(0.25) * (r0.x + T(2) * r1.x + r2.x);
                 yB = T(0.25) * (r0.y + T(2) * r1.y + r2.y);
             }
         }
-        const T vA = (hx && hy) ? T(0.5) * xA + T(0.5) * yA : (hx ? xA : yA);
+        T vA = (hx && hy) ? T(0.5) * xA + T(0.5) * yA : (hx ? xA : yA);
         const T vB = (hx && hy) ? T(0.5) * xB + T(0.5) * yB : (hx ? xB : yB);
         if (op) {
-            const int t = op_index(p, i, j, m.qic);  // unknown of cell A; B is the next one
-            if (i > 0) m.b3[t] = vA;
-            m.b3[t + 1] = vB;
+            const Sm<T> t = m.b3.at(op_index(p, i, j, m.qic));  // unknown of cell A; B is the next one
+            if (i > 0) t.st(vA);
+            t.at(1).st(vB);
         } else {
-            if (i > 0) {
-                cb[cA] = vA;
-                cu[cA] = T(0);
-            }
-            cb[cA + 1] = vB;
-            cu[cA + 1] = T(0);
+            if (i == 0) vA = T(0);  // the boundary stays zero
+            cb.at(cA).st2(vA, vB);
+            cu.at(cA).st2(T(0), T(0));
         }
     }
 }
@@ -458,21 +497,24 @@ template <class T, int NP>
 __device__ __forceinline__ void mid_pre(const MidItem<T>& m, int d, int nu1, bool zero)
 {
     const MidDiag<T> g = mid_diag(m, d);
-    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x;
-    Pair<T> P[NP];
+    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x, dump = 2 * np + (1 << (g.plo + g.ng - 1));
+    const uint32_t on = pairs_of_warp<NP>(np);
+    Pair<T> P[NP] = {};
 #pragma unroll
-    for (int k = 0; k < NP; ++k) pair_load(P[k], g, d, tid + k * nt, tid + k * nt < np);
+    for (int k = 0; k < NP; ++k)
+        if (on >> k & 1) pair_load(P[k], g, d, tid + k * nt, np, dump);
     if (d == 0) {  // one unknown: solved exactly
-        if (P[0].vR) g.u[P[0].cR] = P[0].bR;
+        if (on & 1) Sm<T>{P[0].aR}.st(P[0].bR);
         __syncthreads();
         return;
     }
-    mid_sweeps<T, NP>(P, g.u, nu1, zero);
+    mid_sweeps<T, NP>(P, on, nu1, zero);
     if (nu1 > 0) {
 #pragma unroll
         for (int k = 0; k < NP; ++k) {
-            const Pair<T>& a = P[k];
-            if (a.nx) m.r[tid + k * nt] = a.vR ? a.dR * (pair_red(a, g.u) - a.uR) : T(0);
+            if (!(on >> k & 1)) continue;
+            const T r = P[k].dR * (pair_red(P[k]) - P[k].uR);
+            if (tid + k * nt < np) m.r.at(tid + k * nt).st(r);
         }
         __syncthreads();
         mid_restrict<T, true>(m, d);
@@ -480,9 +522,10 @@ __device__ __forceinline__ void mid_pre(const MidItem<T>& m, int d, int nu1, boo
         for (int k = tid; k < (g.ng << (d + 2)); k += nt) {
             const int p = g.plo + (k >> (d + 2)), cell = k & ((4 << d) - 1), nx = 1 << p;
             if ((cell & (nx - 1)) == 0 || cell < nx) continue;
-            const T aw = g.ax[k - 1], ae = g.ax[k], as = g.ay[k - nx], an = g.ay[k];
-            m.r[k] = g.b[k] - ((aw + ae + as + an) * g.u[k] - (aw * g.u[k - 1] + ae * g.u[k + 1]) -
-                               (as * g.u[k - nx] + an * g.u[k + nx]));
+            const Sm<T> x = g.ax.at(k), y = g.ay.at(k), u = g.u.at(k);
+            const T aw = x.at(-1).ld(), ae = x.ld(), as = y.at(-nx).ld(), an = y.ld();
+            m.r.at(k).st(g.b.at(k).ld() - ((aw + ae + as + an) * u.ld() - (aw * u.at(-1).ld() + ae * u.at(1).ld()) -
+                                           (as * u.at(-nx).ld() + an * u.at(nx).ld())));
         }
         __syncthreads();
         mid_restrict<T, false>(m, d);
@@ -497,60 +540,50 @@ template <class T, int NP>
 __device__ __forceinline__ void mid_post(const MidItem<T>& m, int d, int nu2, T omega)
 {
     const MidDiag<T> g = mid_diag(m, d);
-    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x;
+    const int np = g.ng << (d + 1), tid = threadIdx.x, nt = blockDim.x, dump = 2 * np + (1 << (g.plo + g.ng - 1));
+    const uint32_t on = pairs_of_warp<NP>(np);
     const int plo = mid_plo(d - 1, m.qic);
-    const T* cu = d == m.lo && m.lo > 0 ? m.u3 : mid_diag(m, d - 1).u;
-    Pair<T> P[NP];
+    const bool op = d == m.lo && m.lo > 0;
+    const Sm<T> cu{op ? m.u3.a : m.u.at(m.at[op ? d : d - 1].y).a};
+    Pair<T> P[NP] = {};
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int mm = tid + k * nt;
         Pair<T>& a = P[k];
-        pair_load(a, g, d, mm, mm < np);
-        if (a.nx == 0) continue;
+        if (!(on >> k & 1)) continue;
+        pair_load(a, g, d, mm, np, dump);
+        if (a.w == 0) continue;
         const int p = g.plo + (mm >> (d + 1)), q = d + 2 - p, cell = (2 * mm) & ((4 << d) - 1);
-        const int i = cell & (a.nx - 1), j = cell >> p;
-        const bool hx = p > 1, hy = q > 1;
-        T xA = T(0), xB = T(0), yA = T(0), yB = T(0);
-        if (hx) {  // grid (p-1, q): row j, columns i/2 and i/2 + 1
-            const T* c = cu + ((p - 1 - plo) << (d + 1)) + (j << (p - 1)) + (i >> 1);
-            xA = c[0];
-            xB = T(0.5) * (xA + c[1]);
-        }
-        if (hy) {  // grid (p, q-1): rows j/2 and, between two of them, j/2 + 1
-            const T* c = cu + ((p - plo) << (d + 1)) + ((j >> 1) << p) + i;
-            const auto c0 = ld2(c);
-            yA = c0.x;
-            yB = c0.y;
-            if (j & 1) {
-                const auto c1 = ld2(c + a.nx);
-                yA = T(0.5) * (yA + c1.x);
-                yB = T(0.5) * (yB + c1.y);
+        const int nx = 1 << p, i = cell & (nx - 1), j = cell >> p;
+        const bool hx = p > 1, hy = q > 1, redB = j & 1;
+        const Sm<T> cx = cu.at(((p - 1 - plo) << (d + 1)) + (j << (p - 1)) + (i >> 1));  // grid (p-1, q): row j, from column i/2
+        const Sm<T> cy = cu.at(((p - plo) << (d + 1)) + ((j >> 1) << p) + i);            // grid (p, q-1): from row j/2
+        // correction at node A (B = 0) or B (B = 1) from the scaled coefficients
+        auto corr = [&](int B, T h0, T h1, T v0, T v1) {
+            T x = T(0), y = T(0);
+            if (hx) {
+                x = cx.ld();
+                if (B) x = T(0.5) * (x + cx.at(1).ld());
             }
-        }
-        const bool redB = a.eR > 0;
-        if (a.vK) {
-            const T x = redB ? xA : xB, y = redB ? yA : yB;
-            T e = hx ? x : y;
-            if (hx && hy) {
-                const T cx = a.pK + a.oK, cy = a.sK + a.nK, x2 = cx * cx, y2 = cy * cy, w = rcp_of(x2 + y2);
-                e = (x2 * w) * x + (y2 * w) * y;
+            if (hy) {
+                y = cy.at(B).ld();
+                if (redB) y = T(0.5) * (y + cy.at(nx + B).ld());
             }
-            a.uK += omega * e;
-            g.u[a.cR - a.eR] = a.uK;
+            if (!(hx && hy)) return hx ? x : y;
+            const T c1 = h0 + h1, c2 = v0 + v1, x2 = c1 * c1, y2 = c2 * c2, w = rcp_of(x2 + y2);
+            return (x2 * w) * x + (y2 * w) * y;
+        };
+        if (!redB || i > 0) {
+            a.uK += omega * corr(redB ? 0 : 1, a.pK, a.oK, a.sK, a.nK);
+            Sm<T>{a.aR - a.e}.st(a.uK);
         }
-        if (nu2 == 0 && a.vR) {
-            const T x = redB ? xB : xA, y = redB ? yB : yA;
-            T e = hx ? x : y;
-            if (hx && hy) {
-                const T cx = a.pR + a.oR, cy = a.sR + a.nR, x2 = cx * cx, y2 = cy * cy, w = rcp_of(x2 + y2);
-                e = (x2 * w) * x + (y2 * w) * y;
-            }
-            a.uR += omega * e;
-            g.u[a.cR] = a.uR;
+        if (nu2 == 0 && (redB || i > 0)) {
+            a.uR += omega * corr(redB ? 1 : 0, a.pR, a.oR, a.sR, a.nR);
+            Sm<T>{a.aR}.st(a.uR);
         }
     }
     __syncthreads();
-    mid_sweeps<T, NP>(P, g.u, nu2, false);
+    mid_sweeps<T, NP>(P, on, nu2, false);
 }
 
 // u3 = M b3: two threads a row.
@@ -562,10 +595,9 @@ __device__ __forceinline__ void mid_matrix(const MidItem<T>& m)
         const int t = t2 >> 1, h = t2 & 1;
         T s0 = T(0), s1 = T(0), s2 = T(0), s3 = T(0);
         if (t < m.n3) {
-            const T* row = m.M + t * m.ld3 + h * half;
-            const T* v = m.b3 + h * half;
+            const Sm<T> row = m.M.at(t * m.ld3 + h * half), v = m.b3.at(h * half);
             for (int k = 0; k < half; k += 4) {
-                const auto a = ld2(row + k), b = ld2(row + k + 2), x = ld2(v + k), y = ld2(v + k + 2);
+                const auto a = row.at(k).ld2(), b = row.at(k + 2).ld2(), x = v.at(k).ld2(), y = v.at(k + 2).ld2();
                 s0 += a.x * x.x;
                 s1 += a.y * x.y;
                 s2 += b.x * y.x;
@@ -584,7 +616,7 @@ __device__ __forceinline__ void mid_matrix(const MidItem<T>& m)
                 o -= nn;
             }
             const int nx1 = (1 << p) - 1, j = 1 + o / nx1, i = 1 + o - (j - 1) * nx1;
-            m.u3[((p - plo) << (kOpD + 2)) + (j << p) + i] = s;
+            m.u3.at(((p - plo) << (kOpD + 2)) + (j << p) + i).st(s);
         }
     }
     __syncthreads();
@@ -650,24 +682,29 @@ __device__ __forceinline__ void mid_fill(const MidItem<T>& m, const SampleInfo& 
     const int tid = threadIdx.x, nt = blockDim.x;
     const MidWords w = mid_words(m.pic, m.qic, m.lo, m.hi, 1);
     int c0 = 0;
-    for (int d = m.lo; d <= m.hi; ++d) {
-        const int nc = mid_cells(d, m.pic, m.qic), plo = mid_plo(d, m.qic);
-        for (int k = tid; k < nc; k += nt) {
-            const int p = plo + (k >> (d + 2)), cell = k & ((4 << d) - 1);
-            const int i = cell & ((1 << p) - 1), j = cell >> p;
-            const int64_t o = S.node_off + grid_offset(p, d + 2 - p, S.Q) + j * ((1 << p) + 1) + i;
-            m.ax[c0 + k] = ax[o];
-            m.ay[c0 + k] = ay[o];
+    for (int d = m.lo; d <= m.hi; ++d)
+        for (int p = mid_plo(d, m.qic); p <= mid_phi(d, m.pic); ++p) {
+            const T* gx = ax + S.node_off + grid_offset(p, d + 2 - p, S.Q);
+            const T* gy = ay + (gx - ax);
+#pragma unroll 2
+            for (int k = tid; k < 4 << d; k += nt) {  // cell (i, j) is node (i, j) of rows of 2^p + 1
+                const int o = k + (k >> p);
+                const T x = gx[o], y = gy[o];
+                m.ax.at(c0 + k).st(x);
+                m.ay.at(c0 + k).st(y);
+            }
+            c0 += 4 << d;
         }
-        c0 += nc;
-    }
-    for (int k = tid; k < w.cells + w.pads; k += nt) m.u[k] = T(0);
+    for (int k = tid; k < w.cells; k += nt) m.b.at(k).st(T(0));  // boundary nodes read it (with zero coefficients)
+    for (int k = tid; k < w.cells + w.pads; k += nt) m.u.at(k).st(T(0));
     if (m.lo > 0) {
         const T* M = op + S.op_off + op_offset(m.pic < 4 ? m.pic : 4, m.qic < 4 ? m.qic : 4, S.P, S.Q);
-        for (int k = 2 * tid; k < m.n3 * m.ld3; k += 2 * nt)
-            *reinterpret_cast<typename Vec2<T>::V*>(m.M + k) = ld2(M + k);
-        for (int k = tid; k < kOpN; k += nt) m.b3[k] = T(0);
-        for (int k = tid; k < kU3; k += nt) m.u3[k] = T(0);
+        for (int k = 2 * tid; k < m.n3 * m.ld3; k += 2 * nt) {
+            const auto v = *reinterpret_cast<const typename Vec2<T>::V*>(M + k);
+            m.M.at(k).st2(v.x, v.y);
+        }
+        for (int k = tid; k < kOpN; k += nt) m.b3.at(k).st(T(0));
+        for (int k = tid; k < kU3; k += nt) m.u3.at(k).st(T(0));
     }
 }
 
@@ -685,25 +722,26 @@ __global__ void __launch_bounds__(kMidThreads, sizeof(T) == 4 ? 3 : 1)
     mid_fill(m, S, ax, ay, op);
     __syncthreads();
     const MidDiag<T> g = mid_diag(m, kMidD);
-    const int nc = g.ng << (kMidD + 2), tid = threadIdx.x, nt = blockDim.x;
-    for (int k = tid; k < nc; k += nt) {
-        const int p = g.plo + (k >> (kMidD + 2)), q = kMidD + 2 - p, cell = k & ((4 << kMidD) - 1);
-        const int i = cell & ((1 << p) - 1), j = cell >> p;
-        if (i == 0 || j == 0) continue;
-        const int64_t o = t.scr + grid_offset(p, q, qi) + j * ((1 << p) + 1) + i;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    for (int p = g.plo; p < g.plo + g.ng; ++p) {
+        const int q = kMidD + 2 - p;
+        const int64_t so = t.scr + grid_offset(p, q, qi);
         const bool hx = p < pi, hy = q < qi;
-        g.b[k] = (hx && hy) ? T(0.5) * sbx[o] + T(0.5) * sby[o] : (hx ? sbx[o] : sby[o]);
+        for (int k = tid; k < 4 << kMidD; k += nt) {
+            const int64_t o = so + k + (k >> p);
+            const T v = (hx && hy) ? T(0.5) * sbx[o] + T(0.5) * sby[o] : (hx ? sbx[o] : sby[o]);
+            if (k >> p && k & ((1 << p) - 1)) g.b.at(((p - g.plo) << (kMidD + 2)) + k).st(v);
+        }
     }
     __syncthreads();
     for (int call = 0; call < cp.mu; ++call) mid_cycle(m, cp.mu, cp.nu1, cp.nu2, (T)cp.omega, call == 0);
     for (int p = g.plo; p < g.plo + g.ng; ++p) {
-        const int q = kMidD + 2 - p, nx = 1 << p, W = nx + 1, n = W * ((1 << q) + 1);
+        const int q = kMidD + 2 - p, nx = 1 << p;
         T* dst = su + t.scr + grid_offset(p, q, qi);
-        const T* src = g.u + ((p - g.plo) << (kMidD + 2));
-        for (int v = tid; v < n; v += nt) {
-            const int j = v / W, i = v - j * W;
-            dst[v] = src[j * nx + i];  // boundary nodes are zeros of the layout
-        }
+        for (int k = tid; k < 4 << kMidD; k += nt)  // column 0 and row 0 are zeros of the layout
+            dst[k + (k >> p)] = g.u.at(((p - g.plo) << (kMidD + 2)) + k).ld();
+        for (int k = tid; k <= 1 << q; k += nt) dst[k * (nx + 1) + nx] = T(0);
+        for (int k = tid; k <= nx; k += nt) dst[(nx + 1) * (1 << q) + k] = T(0);
     }
 }
 
@@ -735,14 +773,15 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, 
     for (int step = 0;; ++step) {
         __syncthreads();
         double acc = 0.0;
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            const int i = 1 + k % (nx - 1), j = 1 + k / (nx - 1), c = j * W + i;
+        for (int k = nx + threadIdx.x; k < nx * ny; k += blockDim.x) {
+            const int i = k & (nx - 1), j = k >> p, c = j * W + i;
+            if (i == 0) continue;
             const double aw = fx[c - 1], ae = fx[c], as = fy[c - W], an = fy[c];
             const double Au = (aw + ae + as + an) * u[c] - (aw * u[c - 1] + ae * u[c + 1]) - (as * u[c - W] + an * u[c + W]);
             const double r = 1.0 - Au;
             acc += r * r;
-            g.b[(j << p) + i] = (T)r;
-            g.u[(j << p) + i] = T(0);
+            g.b.at(k).st((T)r);
+            g.u.at(k).st(T(0));
         }
         const double ss = block_sum(acc);
         if (threadIdx.x == 0) {
@@ -764,9 +803,9 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, 
         __syncthreads();
         if (!s_act) return;
         mid_cycle(m, cp.mu, cp.nu1, cp.nu2, (T)cp.omega, true);
-        for (int k = threadIdx.x; k < n; k += blockDim.x) {
-            const int i = 1 + k % (nx - 1), j = 1 + k / (nx - 1);
-            u[j * W + i] += (double)g.u[(j << p) + i];
+        for (int k = nx + threadIdx.x; k < nx * ny; k += blockDim.x) {
+            const int i = k & (nx - 1), j = k >> p;
+            if (i > 0) u[j * W + i] += (double)g.u.at(k).ld();
         }
     }
 }

@@ -69,6 +69,10 @@ struct Segment {
     int64_t list_off;   // the segment's samples are slist[list_off .. list_off+count)
     int64_t scr_slot;   // offset of the item's hierarchy inside the sample's stage scratch
     int64_t stage_base; // item-level lists: index of (group, item) in the stage's flag array
+    // set by visit_offsets for the visit lists: the hierarchy of the group's sample 0 and the
+    // stride between samples; the task grid and its children in a hierarchy, the grid in a rectangle
+    int64_t scr0, scr_per;
+    int so, cxo, cyo, co;
 };
 
 struct Group {
@@ -77,6 +81,16 @@ struct Group {
     int64_t scr_start;      // start of the group's stage scratch
     int64_t scr_per_sample; // stage scratch per sample of the group
 };
+
+inline void visit_offsets(Segment& s, const Group& G)
+{
+    s.scr0 = G.scr_start + s.scr_slot;
+    s.scr_per = G.scr_per_sample;
+    s.so = (int)grid_offset(s.p, s.q, s.qi);
+    s.cxo = s.p > 1 ? (int)grid_offset(s.p - 1, s.q, s.qi) : 0;
+    s.cyo = s.q > 1 ? (int)grid_offset(s.p, s.q - 1, s.qi) : 0;
+    s.co = (int)grid_offset(s.p, s.q, G.Q);
+}
 
 struct DevCtx {
     const SampleInfo* samples;
@@ -1585,6 +1599,7 @@ __global__ void k_qoi(DevCtx cx, const double* u64, const double* Z, int qoi, do
 }  // namespace msg
 
 #include "mid.cuh"
+#include "visit.cuh"
 
 namespace msg {
 
@@ -1820,6 +1835,37 @@ static std::vector<uint2> low_resolve(const msg_params& prm, std::vector<LowDesc
     return rp;
 }
 
+// Node entries and phase programs (one call on diagonal kOpD) of the classes whose
+// matrices k_lowop builds; desc[c] is class c of mid.cuh.
+struct OpTables {
+    LowDesc desc[kOpClasses];
+    std::vector<uint4> ent;
+    std::vector<uint2> prog;
+    int ecap, pcap;  // entries and program words of the largest class (words: even)
+};
+
+static OpTables op_tables(const msg_params& prm)
+{
+    OpTables t;
+    const LowPlanes& lp = low_tables().planes[kOpD];
+    const std::vector<int> words = low_program(kOpD, prm, false);
+    t.ecap = t.pcap = 0;
+    for (int c = 0; c < kOpClasses; ++c) {
+        LowDesc& D = t.desc[c];
+        low_build_class(op_pic(c), op_qic(c), kOpD, lp, D, t.ent);
+        D.prog = (int)t.prog.size();
+        for (int w : words) {
+            const int kind = w & 7, d = w >> 3, cnt = D.cnt[d][kind];
+            if (cnt == 0 || (kind == LK_RESID && D.cnt[d][LK_RESTRICT] == 0)) continue;
+            t.prog.push_back(make_uint2((uint32_t)kind | (uint32_t)cnt << 3, (uint32_t)(D.off[d][kind] - D.e0)));
+        }
+        D.nops = (int)t.prog.size() - D.prog;
+        t.ecap = std::max(t.ecap, D.e1 - D.e0);
+        t.pcap = std::max(t.pcap, (D.nops + 1) & ~1);
+    }
+    return t;
+}
+
 constexpr size_t kSmemMax = 227 * 1024;  // dynamic shared memory of one CTA
 // Launch shape and cut of the low-diagonal kernel for these parameters.
 struct LowShape {
@@ -1946,8 +1992,10 @@ int validate(const int32_t* PQ, int64_t S, const msg_params* prm)
         set_error("tune_visit_smem must be in [0, 227] (KB)");
         return MSG_ERR_INVALID;
     }
-    const LowShape ls = low_shape(*prm);
-    if (ls.smem[ls.cut] > kSmemMax) {
+    // (with the defaults the cut drops until the phase kernel fits, so only a caller's shape can fail)
+    const bool shaped = prm->tune_low_cut || prm->tune_low_items || prm->tune_low_warps;
+    const LowShape ls = shaped ? low_shape(*prm) : LowShape{};
+    if (shaped && ls.smem[ls.cut] > kSmemMax) {
         set_error("tune_low_warps x tune_low_items items of the low-diagonal kernel do not fit the shared memory of one CTA");
         return MSG_ERR_INVALID;
     }
@@ -2052,21 +2100,21 @@ void build_plan(const int32_t* PQ, int64_t S, Plan& pl)
 // The cycles run on chip (mid.cuh) unless the caller sets the cut of the
 // low-diagonal kernel: that keeps the recursion below the cut as phases.
 bool on_chip(const msg_params& prm) { return prm.tune_low_cut == 0; }
+// planes of the face images: those of the matrices, or of the phase kernel's highest cut
+const LowPlanes& img_planes(const msg_params& prm) { return low_tables().planes[on_chip(prm) ? kOpD : kLowMax]; }
 // highest stage solved by k_item (-1: none)
 int item_stages(const msg_params& prm) { return !on_chip(prm) ? -1 : prm.precision == MSG_PREC_MIXED ? kItemL32 : kItemL64; }
-// shared memory of the largest item of a stage, and of k_mid
-size_t item_smem(int L, const msg_params& prm)
+// shared memory of the largest item of a stage, and of k_mid, with cycles in T
+// (the convergence study runs in FP64 whatever prm.precision says)
+template <class T>
+size_t item_smem(int L, int nu1)
 {
-    const size_t es = prm.precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
     int most = 0;
-    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, L, prm.nu1));
-    return es * most;
+    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, L, nu1));
+    return sizeof(T) * most;
 }
-size_t mid_smem(const msg_params& prm)
-{
-    const size_t es = prm.precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
-    return es * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kMidD, prm.nu1);
-}
+template <class T>
+size_t mid_smem(int nu1) { return sizeof(T) * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kMidD, nu1); }
 
 struct WsLayout {
     size_t op;  // low-diagonal matrices (mid.cuh)
@@ -2091,16 +2139,21 @@ WsLayout layout_of(const Plan& pl, const msg_params& prm)
     w.gpos = take(sizeof(int) * pl.S);
     w.groups = take(sizeof(Group) * pl.groups.size() * (pl.Lmax + 2));
     w.allsegs = take(sizeof(Segment) * pl.all_segs.size());
-    {
+    const size_t es = precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
+    if (on_chip(prm)) {
+        const OpTables t = op_tables(prm);
+        w.low_desc = take(sizeof(t.desc));
+        w.low_ent = take(sizeof(uint4) * t.ent.size());
+        w.low_prog = take(sizeof(uint2) * t.prog.size());
+    } else {
         std::vector<LowDesc> desc;
         w.low_desc = take(sizeof(LowDesc) * kLowClassesMax);
         w.low_ent = take(sizeof(uint4) * low_tables().ent.size());
-        w.low_prog = take(sizeof(uint2) * low_resolve(prm, desc, !on_chip(prm)).size());
+        w.low_prog = take(sizeof(uint2) * low_resolve(prm, desc).size());
     }
     {
-        const LowPlanes& lp = low_tables().planes[kLowMax];
-        const size_t es_img = precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
-        w.low_img = take(es_img * (size_t)pl.S * (lp.nfx + lp.nfy));
+        const LowPlanes& lp = img_planes(prm);
+        w.low_img = take(es * (size_t)pl.S * (lp.nfx + lp.nfy));
     }
     w.nstep = take(sizeof(int) * pl.total_q);
     w.cycles_i = take(sizeof(int) * pl.total_q);
@@ -2108,7 +2161,6 @@ WsLayout layout_of(const Plan& pl, const msg_params& prm)
     w.u64 = take(sizeof(double) * pl.total_nodes);
     w.ax64 = take(sizeof(double) * pl.total_nodes);
     w.ay64 = take(sizeof(double) * pl.total_nodes);
-    const size_t es = precision == MSG_PREC_MIXED ? sizeof(float) : sizeof(double);
     if (precision == MSG_PREC_MIXED) {
         w.ax32 = take(sizeof(float) * pl.total_nodes);
         w.ay32 = take(sizeof(float) * pl.total_nodes);
@@ -2191,14 +2243,194 @@ struct SolveCtx {
     const LowDesc* low_desc;
     const uint4* low_ent;
     const uint2* low_prog;  // resolved programs of all classes
-    int op_pcap;            // program words of the longest class of diagonal kOpD, even
 };
+
+// Does k_visit take grid (p, q) of diagonal d?  It has pairs for a whole CTA of
+// at least a warp, its smallest cluster holds visit_threads_max x kVisitPairs pairs per
+// CTA, and a slab needs two rows.  Depends on the grid alone, so a sample's path does
+// not depend on its batch.
+template <class T>
+static int visit_cluster(int d) { return (int)std::max<int64_t>(1, (int64_t(1) << (d + 1)) / (visit_threads_max<T>() * kVisitPairs)); }
+template <class T>
+static bool visit_takes(int d, int q)
+{
+    return d >= 5 && visit_cluster<T>(d) <= kVisitClusterMax && (int64_t(1) << q) >= 2 * visit_cluster<T>(d);
+}
+
+// One visit half of diagonal d for the segments segs[0 .. c.nseg) (host copy).
+// Launch shape: see the rule below; `block` (threads per CTA) overrides it.
+template <class T>
+static cudaError_t launch_visit(const DevCtx& c, const Segment* segs, int d, T* su, T* sbx, T* sby, const T* ax,
+                                const T* ay, int pre, int zero, int nu, T omega, int block, cudaStream_t st)
+{
+    const int np = 1 << (d + 1);  // pairs of a grid
+    int64_t tasks = 0, maxc = 0;
+    int qmin = 30;
+    double bytes = 0;
+    for (int k = 0; k < c.nseg; ++k) {
+        tasks += segs[k].count;
+        maxc = std::max<int64_t>(maxc, segs[k].count);
+        qmin = std::min(qmin, segs[k].q);
+        const double b = (segs[k].p < segs[k].pi && segs[k].q < segs[k].qi) ? 2.0 : 1.0;
+        const double ch = (segs[k].p > 1 ? 0.5 : 0.0) + (segs[k].q > 1 ? 0.5 : 0.0);
+        bytes += (double)segs[k].count * pts(segs[k].p, segs[k].q) * (b + 2 + (pre ? 1 : 2) + ch) * sizeof(T);
+    }
+    // as few CTAs per grid as hold it: a cluster barrier costs a CTA barrier several times over.
+    // `block`: that many threads per CTA at most, where the slabs of the shortest grid allow it
+    int C = visit_cluster<T>(d);
+    if (block)
+        while (np / (kVisitPairs * C) > std::max(block, 32) && 2 * C <= kVisitClusterMax && (1 << qmin) >= 4 * C) C *= 2;
+    const int nt = np / (kVisitPairs * C);
+    int words = 0;
+    for (int k = 0; k < c.nseg; ++k) words = std::max(words, visit_words(segs[k].p, segs[k].q, C));
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(maxc * C), (unsigned)c.nseg);
+    cfg.blockDim = dim3(nt);
+    cfg.dynamicSmemBytes = sizeof(T) * words;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = C;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    auto go = [&](auto k) {
+        return cudaLaunchKernelEx(&cfg, k, c, su, sbx, sby, ax, ay, pre, zero, nu, omega, C);
+    };
+    prof_begin(pre ? K_PRE : K_POST, st);
+    cudaError_t e;
+    if (C == 1) e = go(k_visit<T, kVisitPairs, false>);
+    else e = go(k_visit<T, kVisitPairs, true>);
+    prof_end(pre ? K_PRE : K_POST, st, bytes, 0.0, d);
+    return e;
+}
+
+// Attributes of the k_visit variants (idempotent).
+template <class T>
+static int visit_attributes()
+{
+    auto set = [](auto k) {
+        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+        return e == cudaSuccess ? cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
+    };
+    MSG_CUDA_TRY(set(k_visit<T, kVisitPairs, false>));
+    MSG_CUDA_TRY(set(k_visit<T, kVisitPairs, true>));
+    return MSG_OK;
+}
 
 // Threads per CTA of k_item: a thread holds at most four pairs of a diagonal.
 template <class T>
 static int item_threads(int L)
 {
     return L <= 2 ? 32 : L <= 4 ? 64 : L <= 6 ? 128 : 256;
+}
+
+// The grids of one diagonal in a cycle's launches: segments (host copy and context of
+// the device copy), k_visit's first, from `fall` those it does not take.
+struct VisitList {
+    DevCtx cx;
+    const Segment* host = nullptr;
+    size_t n = 0, fall = 0;
+    double bytes_pre = 0, bytes_post = 0;  // words
+    DevCtx ctx(size_t a, size_t b) const
+    {
+        DevCtx c = cx;
+        c.segs += a;
+        c.nseg = (int)(b - a);
+        return c;
+    }
+};
+
+// One visit half (pre: 1 PRE, 0 POST) of diagonal d: k_visit, and for the grids it does
+// not take (or with no sweeps, or on request) the one-CTA kernels.  True on a launch error.
+template <class T>
+static bool visit_half(const VisitList& v, int d, int pre, int zi, T* su, T* sbx, T* sby, const T* ax, const T* ay,
+                       const msg_params& prm, int block, size_t visit_smem, cudaStream_t st)
+{
+    if (v.n == 0) return false;
+    const int nu = pre ? prm.nu1 : prm.nu2;
+    size_t seg0 = 0, seg1 = v.n;
+    if (nu > 0 && visit_smem <= kVisitSmemKB * 1024 && v.fall > seg0) {
+        bool launch_err = launch_visit<T>(v.ctx(seg0, v.fall), v.host + seg0, d, su, sbx, sby, ax, ay,
+                                      pre, zi, nu, (T)prm.omega, prm.tune_block, st) != cudaSuccess;
+        seg0 = v.fall;
+        if (launch_err || seg0 == seg1) return launch_err;
+    }
+    DevCtx c = v.ctx(seg0, seg1);
+    prof_begin(pre ? K_PRE : K_POST, st);
+    int64_t maxc = 0;
+    for (size_t k = seg0; k < seg1; ++k) maxc = std::max<int64_t>(maxc, v.host[k].count);
+    const dim3 g2((unsigned)maxc, (unsigned)(seg1 - seg0));  // x: sample in segment, y: segment
+    // threads per CTA: every grid of diagonal d has 2^(d+2) cells, 2^(d+1) points per
+    // colour; small grids get no idle warps, the big ones (d >= 10) twice the block
+    const int vb = d >= 10 ? std::min(2 * block, 1024) : std::min(block, std::max(32, 1 << (d + 1)));
+    // register-cached visit when every grid of the launch has at most
+    // kRegThreadsMax x NPT nodes of a colour and its shared planes (u; PRE also r)
+    // fit the limit; else the global-memory visit
+    int64_t nodes = 0, nslot = 0;
+    for (size_t k = seg0; k < seg1; ++k) {
+        const int sp = v.host[k].p, sq = v.host[k].q;
+        nodes = std::max<int64_t>(nodes, (int64_t)((1 << sp) + 1) * ((1 << sq) + 1));
+        nslot = std::max<int64_t>(nslot, (int64_t)((1 << sq) - 1) << (sp - 1));
+    }
+    const int nptmax = sizeof(T) == 4 ? 4 : 2;  // FP64 nodes take twice the registers
+    int npt = 1;
+    while (npt < nptmax && (nslot + npt - 1) / npt > block) npt *= 2;
+    const int vr = (int)std::max<int64_t>(32, ((nslot + npt - 1) / npt + 31) / 32 * 32);
+    const size_t rsm = (pre ? 2 : 1) * (size_t)nodes * sizeof(T);
+    if (vr <= kRegThreadsMax && rsm <= visit_smem) {
+        const double om = prm.omega;
+        if (npt == 1) k_visit_reg<T, 1><<<g2, vr, rsm, st>>>(c, su, sbx, sby, ax, ay, pre, zi, nu, om);
+        else if (npt == 2) k_visit_reg<T, 2><<<g2, vr, rsm, st>>>(c, su, sbx, sby, ax, ay, pre, zi, nu, om);
+        else if constexpr (sizeof(T) == 4)
+            k_visit_reg<T, 4><<<g2, vr, rsm, st>>>(c, su, sbx, sby, ax, ay, pre, zi, nu, om);
+    } else if (pre) {
+        // residual band of the restriction: the whole grid when it has at most
+        // kBandNodes nodes, else bands of at least 3 rows
+        int band = 0;
+        for (size_t k = seg0; k < seg1; ++k) {
+            const int W = (1 << v.host[k].p) + 1, n = W * ((1 << v.host[k].q) + 1);
+            band = std::max(band, std::min(n, std::max(kBandNodes, 3 * W)));
+        }
+        k_pre<T><<<g2, vb, sizeof(T) * band, st>>>(c, su, sbx, sby, ax, ay, zi, prm.nu1, band);
+    } else {
+        k_post<T><<<g2, vb, 0, st>>>(c, su, sbx, sby, ax, ay, prm.nu2, prm.omega);
+    }
+    prof_end(pre ? K_PRE : K_POST, st, (pre ? v.bytes_pre : v.bytes_post) * sizeof(T), 0.0, d);
+    return cudaGetLastError() != cudaSuccess;
+}
+
+// The launches of one mu-cycle on diagonal L (Algorithm 1, the recursion unrolled on the
+// host): half(d, pre, zero) above the cut, low() for the mu calls at the cut.
+template <class Half, class Low>
+static void cycle_launches(int L, int cut, int mu, bool zero, Half half, Low low)
+{
+    struct Frame { int d, k, zi, phase; };
+    std::vector<Frame> stack;
+    stack.push_back({L, 0, zero, 0});
+    while (!stack.empty()) {
+        Frame& f = stack.back();
+        if (f.phase == 0) {
+            half(f.d, 1, f.zi);
+            f.phase = 1;
+            if (f.d - 1 <= cut) {
+                low(f.d - 1, mu);
+                f.phase = 2;
+            }
+            continue;
+        }
+        if (f.phase == 1) {
+            if (f.k < mu) {
+                const int zi = (f.k == 0);
+                f.k += 1;
+                stack.push_back({f.d - 1, 0, zi, 0});
+                continue;
+            }
+            f.phase = 2;
+        }
+        half(f.d, 0, 0);
+        stack.pop_back();
+    }
 }
 
 // Stage L of FMSG for the samples handed over by stage L-1: cubic
@@ -2250,7 +2482,7 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
 
     std::vector<std::vector<int>> active(its.size()), fresh(its.size());
     size_t item_nseg = 0;
-    std::vector<size_t> dseg0(L + 1, 0), dnseg(L + 1, 0);
+    std::vector<size_t> dseg0(L + 1, 0), dnseg(L + 1, 0), dfall(L + 1, 0);  // k_visit's segments, then the others from dfall
     std::vector<double> dpre(L + 1, 0), dpost(L + 1, 0);
     int64_t nitems = 0;
     double item_pts = 0, low_bytes = 0, low_flops = 0;
@@ -2305,13 +2537,17 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
                 dseg0[d] = ns;
                 b = 0;
                 dpre[d] = dpost[d] = 0;
+                // the grids k_visit takes first, then those it cannot slice
+                for (int part = 0; part < 2; ++part, dfall[d] = part == 1 ? ns : dfall[d])
                 for (size_t k = 0; k < its.size(); ++k) {
                     if (lists[k].empty()) continue;
                     const ItemType& it = its[k];
                     for (int pp = std::max(1, d + 2 - it.qi); pp <= std::min(it.pi, d + 1); ++pp) {
                         const int qq = d + 2 - pp;
-                        h_segs[ns++] = Segment{it.g, it.pi, it.qi, pp, qq, b, (int64_t)lists[k].size(), loff[k],
-                                               it.scr_slot, it.stage_base};
+                        if (visit_takes<T>(d, qq) != (part == 0)) continue;
+                        h_segs[ns] = Segment{it.g, it.pi, it.qi, pp, qq, b, (int64_t)lists[k].size(), loff[k],
+                                             it.scr_slot, it.stage_base};
+                        visit_offsets(h_segs[ns++], hsg[it.g]);
                         b += (int64_t)lists[k].size();
                         const double n = (double)lists[k].size() * pts(pp, qq);
                         const double bw = (pp < it.pi && qq < it.qi) ? 2.0 : 1.0;
@@ -2453,7 +2689,7 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
         auto launch_low = [&](int d, int calls) {
             if (chip) {
                 prof_begin(K_LOW, st);
-                k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem(C.prm), st>>>(
+                k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem<T>(C.prm.nu1), st>>>(
                     ic, su, sbx, sby, C.ax, C.ay, (const T*)(C.ws + wl.op), C.cp);
                 prof_end(K_LOW, st, low_bytes, 0.0, d);
                 launch_err |= cudaGetLastError() != cudaSuccess;
@@ -2486,81 +2722,17 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
             launch_err |= cudaGetLastError() != cudaSuccess;
         };
         auto launch_half = [&](int d, int pre, int zi) {
-            if (dnseg[d] == 0) return;
-            DevCtx c = ctx_of(dseg0[d], dnseg[d]);
-            prof_begin(pre ? K_PRE : K_POST, st);
-            int64_t maxc = 0;
-            for (size_t k = dseg0[d]; k < dseg0[d] + dnseg[d]; ++k) maxc = std::max<int64_t>(maxc, h_segs[k].count);
-            const dim3 g2((unsigned)maxc, (unsigned)dnseg[d]);  // x: sample in segment, y: segment
-            // threads per CTA: every grid of diagonal d has 2^(d+2) cells, 2^(d+1) points per
-            // colour; small grids get no idle warps, the big ones (d >= 10) twice the block
-            const int vb = d >= 10 ? std::min(2 * C.block, 1024) : std::min(C.block, std::max(32, 1 << (d + 1)));
-            // register-cached visit when every grid of the launch has at most
-            // kRegThreadsMax x NPT nodes of a colour and its shared planes (u; PRE also r)
-            // fit the limit; else the global-memory visit
-            const int nu = pre ? C.prm.nu1 : C.prm.nu2;
-            int64_t nodes = 0, nslot = 0;
-            for (size_t k = dseg0[d]; k < dseg0[d] + dnseg[d]; ++k) {
-                const int sp = h_segs[k].p, sq = h_segs[k].q;
-                nodes = std::max<int64_t>(nodes, (int64_t)((1 << sp) + 1) * ((1 << sq) + 1));
-                nslot = std::max<int64_t>(nslot, (int64_t)((1 << sq) - 1) << (sp - 1));
-            }
-            const int nptmax = sizeof(T) == 4 ? 4 : 2;  // FP64 nodes take twice the registers
-            int npt = 1;
-            while (npt < nptmax && (nslot + npt - 1) / npt > C.block) npt *= 2;
-            const int vr = (int)std::max<int64_t>(32, ((nslot + npt - 1) / npt + 31) / 32 * 32);
-            const size_t rsm = (pre ? 2 : 1) * (size_t)nodes * sizeof(T);
-            if (vr <= kRegThreadsMax && rsm <= C.visit_smem) {
-                const double om = C.prm.omega;
-                if (npt == 1) k_visit_reg<T, 1><<<g2, vr, rsm, st>>>(c, su, sbx, sby, C.ax, C.ay, pre, zi, nu, om);
-                else if (npt == 2) k_visit_reg<T, 2><<<g2, vr, rsm, st>>>(c, su, sbx, sby, C.ax, C.ay, pre, zi, nu, om);
-                else if constexpr (sizeof(T) == 4)
-                    k_visit_reg<T, 4><<<g2, vr, rsm, st>>>(c, su, sbx, sby, C.ax, C.ay, pre, zi, nu, om);
-            } else if (pre) {
-                // residual band of the restriction: the whole grid when it has at most
-                // kBandNodes nodes, else bands of at least 3 rows
-                int band = 0;
-                for (size_t k = dseg0[d]; k < dseg0[d] + dnseg[d]; ++k) {
-                    const int W = (1 << h_segs[k].p) + 1, n = W * ((1 << h_segs[k].q) + 1);
-                    band = std::max(band, std::min(n, std::max(kBandNodes, 3 * W)));
-                }
-                k_pre<T><<<g2, vb, sizeof(T) * band, st>>>(c, su, sbx, sby, C.ax, C.ay, zi, C.prm.nu1, band);
-            } else {
-                k_post<T><<<g2, vb, 0, st>>>(c, su, sbx, sby, C.ax, C.ay, C.prm.nu2, C.prm.omega);
-            }
-            prof_end(pre ? K_PRE : K_POST, st, (pre ? dpre[d] : dpost[d]) * es, 0.0, d);
-            launch_err |= cudaGetLastError() != cudaSuccess;
+            VisitList v;
+            v.cx = ctx_of(dseg0[d], dnseg[d]);
+            v.host = h_segs + dseg0[d];
+            v.n = dnseg[d];
+            v.fall = dfall[d] - dseg0[d];
+            v.bytes_pre = dpre[d];
+            v.bytes_post = dpost[d];
+            launch_err |= visit_half<T>(v, d, pre, zi, su, sbx, sby, C.ax, C.ay, C.prm, C.block, C.visit_smem, st);
         };
-        if (L <= cut) {
-            launch_low(L, 1);
-        } else {
-            struct Frame { int d, k, zi, phase; };
-            std::vector<Frame> stack;
-            stack.push_back({L, 0, 1, 0});
-            while (!stack.empty()) {
-                Frame& f = stack.back();
-                if (f.phase == 0) {
-                    launch_half(f.d, 1, f.zi);
-                    f.phase = 1;
-                    if (f.d - 1 <= cut) {
-                        launch_low(f.d - 1, C.prm.mu);
-                        f.phase = 2;
-                    }
-                    continue;
-                }
-                if (f.phase == 1) {
-                    if (f.k < C.prm.mu) {
-                        const int zi = (f.k == 0);
-                        f.k += 1;
-                        stack.push_back({f.d - 1, 0, zi, 0});
-                        continue;
-                    }
-                    f.phase = 2;
-                }
-                launch_half(f.d, 0, 0);
-                stack.pop_back();
-            }
-        }
+        if (L <= cut) launch_low(L, 1);
+        else cycle_launches(L, cut, C.prm.mu, true, launch_half, launch_low);
         if (launch_err) { set_error("kernel launch failed in the cycle schedule"); return finish(MSG_ERR_CUDA); }
         prof_begin(K_UPDATE, st);
         k_update<T><<<(unsigned)nitems, kThreads, 0, st>>>(ic, C.u64, su);
@@ -2571,30 +2743,36 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
     return finish(MSG_OK);
 }
 
-// Matrices of the low diagonals, then stages 0 .. nlow-1, each one launch of
-// k_item over the stage's items of every sample.
+// The matrices of every sample, one launch per class that some group has.
+template <class T>
+static int matrices(const OpTables& ot, const std::vector<Group>& groups, const SampleInfo* samples, int S, const T* img,
+                    const LowDesc* desc, const uint4* ent, const uint2* prog, const msg_params& prm, T* op, cudaStream_t st)
+{
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    const LowPlanes& lp = low_tables().planes[kOpD];
+    for (int c = 0; c < kOpClasses; ++c) {
+        const int pic = op_pic(c), qic = op_qic(c), n = op_n(pic, qic);
+        bool any = false;
+        for (const Group& g : groups) any |= op_has(pic, qic, g.P, g.Q);
+        if (!any) continue;
+        const dim3 blk((n + 31) / 32 * 32, 768 / ((n + 31) / 32 * 32));
+        const size_t smem = sizeof(uint4) * ot.ecap + sizeof(uint2) * ot.pcap +
+                            sizeof(T) * (lp.nfx + lp.nfy + (size_t)(2 * lp.nu + lp.nr) * n);
+        prof_begin(K_COEFFS, st);
+        k_lowop<T><<<(unsigned)S, blk, smem, st>>>(samples, pic, qic, img, lp.nfx + lp.nfy, lp.nfx, desc + c, ent, prog, lp,
+                                                  prm.mu, (T)prm.omega, op);
+        prof_end(K_COEFFS, st, 0.0, 0.0);
+        MSG_CHECK_LAUNCH();
+    }
+    return MSG_OK;
+}
+
+// Stages 0 .. nlow-1, each one launch of k_item over the stage's items of every sample.
 template <class T>
 static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
 {
     const Plan& pl = C.pl;
     T* op = (T*)(C.ws + C.wl.op);
-    for (int c = 0; c < kOpClasses; ++c) {
-        const int pic = op_pic(c), qic = op_qic(c), n = op_n(pic, qic);
-        bool any = false;
-        for (const Group& g : pl.groups) any |= op_has(pic, qic, g.P, g.Q);
-        if (!any) continue;
-        const LowPlanes& lp = low_tables().planes[kOpD];
-        const LowPlanes& lpm = low_tables().planes[kLowMax];
-        const dim3 blk((n + 31) / 32 * 32, 768 / ((n + 31) / 32 * 32));
-        const size_t smem = sizeof(uint4) * C.low.ecap[kOpD] + sizeof(uint2) * C.op_pcap +
-                            sizeof(T) * (lp.nfx + lp.nfy + (size_t)(2 * lp.nu + lp.nr) * n);
-        prof_begin(K_COEFFS, st);
-        k_lowop<T><<<(unsigned)pl.S, blk, smem, st>>>(C.base.samples, pic, qic, (const T*)(C.ws + C.wl.low_img),
-                                                     lpm.nfx + lpm.nfy, lpm.nfx, C.low_desc, C.low_ent, C.low_prog, lp,
-                                                     C.prm.mu, (T)C.prm.omega, op);
-        prof_end(K_COEFFS, st, 0.0, 0.0);
-        MSG_CHECK_LAUNCH();
-    }
     for (int L = 0; L < nlow; ++L) {
         std::vector<Segment> segs;
         int64_t b = 0;
@@ -2613,12 +2791,35 @@ static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
         c.segs = (const Segment*)(C.ws + C.wl.segs[L]);
         c.nseg = (int)segs.size();
         prof_begin(K_LOW, st);
-        k_item<T><<<(unsigned)b, item_threads<T>(L), item_smem(L, C.prm), st>>>(
+        k_item<T><<<(unsigned)b, item_threads<T>(L), item_smem<T>(L, C.prm.nu1), st>>>(
             c, L, C.u64, C.ax64, C.ay64, C.ax, C.ay, op, C.cp, C.prm.max_cycles, C.prm.eps, C.cyc, C.rel, C.stat);
         prof_end(K_LOW, st, work * 40.0, 0.0, L);
         MSG_CHECK_LAUNCH();
         MSG_CUDA_TRY(cudaStreamSynchronize(st));
     }
+    return MSG_OK;
+}
+
+// Shared-memory limits of the cycles' kernels (idempotent).
+template <class T>
+static int cycle_attributes()
+{
+    // the residual band: 3 rows of a 2^12-cell-wide grid at most
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_pre<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)(sizeof(T) * std::max(kBandNodes, 3 * ((1 << 12) + 1)))));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    if constexpr (sizeof(T) == 4)
+        MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    int rc = visit_attributes<T>();
+    if (rc != MSG_OK) return rc;
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_item<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
     return MSG_OK;
 }
 
@@ -2640,8 +2841,9 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
                   (const double*)(ws + wl.ax64), (const double*)(ws + wl.ay64), nullptr, nullptr,
                   (int*)(ws + wl.nstep), (int*)(ws + wl.cycles_i), (double*)(ws + wl.relres_i),
                   CycleParams{prm.mu, prm.nu1, prm.nu2, prm.omega}, prm.tune_block ? prm.tune_block : kVisitThreads,
-                  (size_t)(prm.tune_visit_smem ? prm.tune_visit_smem : kVisitSmemKB) * 1024, low_shape(prm), (const LowDesc*)(ws + wl.low_desc), (const uint4*)(ws + wl.low_ent),
-                  (const uint2*)(ws + wl.low_prog), 0};
+                  (size_t)(prm.tune_visit_smem ? prm.tune_visit_smem : kVisitSmemKB) * 1024,
+                  on_chip(prm) ? LowShape{} : low_shape(prm), (const LowDesc*)(ws + wl.low_desc), (const uint4*)(ws + wl.low_ent),
+                  (const uint2*)(ws + wl.low_prog)};
     float* ax32 = mixed ? (float*)(ws + wl.ax32) : nullptr;
     float* ay32 = mixed ? (float*)(ws + wl.ay32) : nullptr;
     C.ax = mixed ? (const T*)ax32 : (const T*)(ws + wl.ax64);
@@ -2666,7 +2868,7 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
                                                    ax32, ay32);
         prof_end(K_COEFFS, st, nodes * (16.0 + 16.0 + (mixed ? 8.0 : 0.0)), 0.0);
         MSG_CHECK_LAUNCH();
-        const LowPlanes& lp = low_tables().planes[kLowMax];
+        const LowPlanes& lp = img_planes(prm);
         prof_begin(K_COEFFS, st);
         k_lowimg<T><<<(unsigned)pl.S, kThreads, 0, st>>>(C.base.samples, C.ax, C.ay, lp, (T*)(ws + wl.low_img),
                                                           (int64_t)(lp.nfx + lp.nfy), lp.nfx);
@@ -2674,36 +2876,35 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
         MSG_CHECK_LAUNCH();
     }
     {
-        // tables of the low-diagonal program: class descriptors, node entries, programs
+        // tables of the low diagonals: class descriptors, node entries, programs
         const LowTables& lt = low_tables();
         std::vector<LowDesc> desc;
-        const std::vector<uint2> rp = low_resolve(prm, desc, !on_chip(prm));
-        MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_desc, desc.data(), sizeof(LowDesc) * desc.size(),
-                                     cudaMemcpyHostToDevice, st));
-        MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_ent, lt.ent.data(), sizeof(uint4) * lt.ent.size(),
-                                     cudaMemcpyHostToDevice, st));
-        MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.low_prog, rp.data(), sizeof(uint2) * rp.size(),
-                                     cudaMemcpyHostToDevice, st));
-        for (const LowDesc& D : desc)
-            if (D.dl == kOpD) C.op_pcap = std::max(C.op_pcap, (D.nops + 1) & ~1);
+        std::vector<uint2> rp;
+        OpTables ot;
+        if (on_chip(prm)) ot = op_tables(prm);
+        else rp = low_resolve(prm, desc);
+        auto up = [&](size_t at, const void* p, size_t bytes) {
+            return cudaMemcpyAsync(ws + at, p, bytes, cudaMemcpyHostToDevice, st);
+        };
+        if (on_chip(prm)) {
+            MSG_CUDA_TRY(up(wl.low_desc, ot.desc, sizeof(ot.desc)));
+            MSG_CUDA_TRY(up(wl.low_ent, ot.ent.data(), sizeof(uint4) * ot.ent.size()));
+            MSG_CUDA_TRY(up(wl.low_prog, ot.prog.data(), sizeof(uint2) * ot.prog.size()));
+            int rc = matrices<T>(ot, pl.groups, C.base.samples, pl.S, (const T*)(ws + wl.low_img), C.low_desc, C.low_ent,
+                                 C.low_prog, prm, (T*)(ws + wl.op), st);
+            if (rc != MSG_OK) return rc;
+        } else {
+            MSG_CUDA_TRY(up(wl.low_desc, desc.data(), sizeof(LowDesc) * desc.size()));
+            MSG_CUDA_TRY(up(wl.low_ent, lt.ent.data(), sizeof(uint4) * lt.ent.size()));
+            MSG_CUDA_TRY(up(wl.low_prog, rp.data(), sizeof(uint2) * rp.size()));
+        }
         // the sources are host vectors: finish the copies before they go out of scope
         MSG_CUDA_TRY(cudaStreamSynchronize(st));
     }
-    // the residual band: 3 rows of a 2^12-cell-wide grid at most
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_pre<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(sizeof(T) * std::max(kBandNodes, 3 * ((1 << 12) + 1)))));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    if constexpr (sizeof(T) == 4)
-        MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_item<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
+    {
+        int rc = cycle_attributes<T>();
+        if (rc != MSG_OK) return rc;
+    }
     MSG_CUDA_TRY(cudaStreamSynchronize(st));
 
     // ---- low stages on chip, one launch each (the stream orders a stage after its children's)
@@ -2931,7 +3132,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
     std::vector<SampleInfo> samples(S);
     std::vector<int> ids(S);
     for (int64_t s = 0; s < S; ++s) {
-        samples[s] = SampleInfo{P, Q, s * R, s * nf, 0};
+        samples[s] = SampleInfo{P, Q, s * R, s * nf, 0, 0};
         ids[s] = (int)s;
     }
     const Group grp{P, Q, 0, (int)S, 0, R};
