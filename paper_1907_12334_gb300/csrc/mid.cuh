@@ -810,4 +810,68 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, 
     }
 }
 
+// Convergence study on hierarchies that fit one CTA: residual history of MSG cycles
+// on (u, b = 1) from u = 0, FP64, one CTA per sample.
+__global__ void __launch_bounds__(256) k_history_chip(DevCtx cx, int L, const double* ax, const double* ay, const double* op,
+                                                      CycleParams cp, int ncycles, double* hist)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int2 at[kMidMax + 1];
+    const TaskRef t = resolve(cx);
+    const SampleInfo& S = cx.samples[t.s];
+    const int p = t.seg->pi, q = t.seg->qi, nx = 1 << p, ny = 1 << q;
+    const MidItem<double> m = mid_item<double>((double*)smem_raw, at, p, q, L > kOpD ? kOpD + 1 : 0, L, cp.nu1);
+    mid_fill(m, S, ax, ay, op);
+    __syncthreads();
+    const MidDiag<double> g = mid_diag(m, L);
+    for (int k = nx + threadIdx.x; k < nx * ny; k += blockDim.x)
+        if (k & (nx - 1)) g.b.at(k).st(1.0);
+    const double nb = sqrt((double)(nx - 1) * (ny - 1));
+    for (int cyc = 0; cyc <= ncycles; ++cyc) {
+        __syncthreads();
+        if (cyc > 0) mid_cycle(m, cp.mu, cp.nu1, cp.nu2, cp.omega, cyc == 1);
+        double acc = 0.0;
+        for (int k = nx + threadIdx.x; k < nx * ny; k += blockDim.x) {
+            if ((k & (nx - 1)) == 0) continue;
+            const Sm<double> x = g.ax.at(k), y = g.ay.at(k), u = g.u.at(k);
+            const double aw = x.at(-1).ld(), ae = x.ld(), as = y.at(-nx).ld(), an = y.ld();
+            const double r = 1.0 - ((aw + ae + as + an) * u.ld() - (aw * u.at(-1).ld() + ae * u.at(1).ld()) -
+                                    (as * u.at(-nx).ld() + an * u.at(nx).ld()));
+            acc += r * r;
+        }
+        const double ss = block_sum(acc);
+        if (threadIdx.x == 0) hist[(int64_t)t.s * (ncycles + 1) + cyc] = sqrt(ss) / nb;
+    }
+}
+
+// The same on larger hierarchies, between the launches of the cycles (b in sbx, u in su
+// of each sample's scratch): start values of the top grid, and one entry of the history.
+__global__ void k_history_start(int P, int Q, int64_t R, double* su, double* sbx)
+{
+    const int W = (1 << P) + 1, n = W * ((1 << Q) + 1);
+    const int64_t o = (int64_t)blockIdx.y * R + grid_offset(P, Q, Q);
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        su[o + k] = 0.0;
+        sbx[o + k] = 1.0;  // (the boundary's is not read)
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_history_norm(int P, int Q, int64_t R, const double* su, const double* ax,
+                                                       const double* ay, double* hist, int stride)
+{
+    const int nx = 1 << P, ny = 1 << Q, W = nx + 1;
+    const int64_t o = (int64_t)blockIdx.x * R + grid_offset(P, Q, Q);
+    const double *u = su + o, *x = ax + o, *y = ay + o;
+    double acc = 0.0;
+    for (int k = nx + threadIdx.x; k < nx * ny; k += blockDim.x) {
+        const int i = k & (nx - 1), c = k + (k >> P);
+        if (i == 0) continue;
+        const double aw = x[c - 1], ae = x[c], as = y[c - W], an = y[c];
+        const double r = 1.0 - ((aw + ae + as + an) * u[c] - (aw * u[c - 1] + ae * u[c + 1]) - (as * u[c - W] + an * u[c + W]));
+        acc += r * r;
+    }
+    const double ss = block_sum(acc);
+    if (threadIdx.x == 0) hist[(int64_t)blockIdx.x * stride] = sqrt(ss) / sqrt((double)(nx - 1) * (ny - 1));
+}
+
 }  // namespace msg

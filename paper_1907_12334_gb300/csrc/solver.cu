@@ -436,9 +436,9 @@ __global__ void k_post(DevCtx cx, T* su, T* sbx, T* sby, const T* ax, const T* a
 // ------------------------------------------------------ convergence study --
 //
 // Residual history of plain cycles from a zero initial guess on each sample's
-// finest grid, b = 1 (Sec. 2, numerical experiments): MSG cycles (Algorithm 1
-// over the whole hierarchy, by the visit halves above), or multigrid with
-// standard coarsening on the diagonal grids (P-k, Q-k) of the same hierarchy:
+// finest grid, b = 1 (Sec. 2, numerical experiments).  MSG cycles run on the
+// solver's own kernels (mid.cuh, visit.cuh) in FP64.  Multigrid with standard
+// coarsening runs on the diagonal grids (P-k, Q-k) of the same hierarchy:
 // full weighting (the tensor product of 1/4 [1 2 1]), bilinear interpolation,
 // the same red-black smoother, coefficients and damping, and an exact solve
 // of the first grid with a single interior line (p = 1 or q = 1).  The paper
@@ -446,7 +446,7 @@ __global__ void k_post(DevCtx cx, T* su, T* sbx, T* sby, const T* ax, const T* a
 // for vertex-centred grids.  One CTA per sample runs a host-built program of
 // the cycle's operations, in FP64.
 
-enum HistOp { H_PRE = 0, H_POST, H_STD_PRE, H_STD_POST, H_STD_LINE };
+enum HistOp { H_STD_PRE = 0, H_STD_POST, H_STD_LINE };
 
 // nu1 sweeps, r = b - A u into the grid's by plane (free in this method), full
 // weighting into the child's bx, child u = 0.
@@ -535,13 +535,12 @@ __device__ void cta_std_line(const G& grp, const Hier<T>& h, int p, int q)
     grp.sync();
 }
 
-// hist[s][k] = ||1 - A u_k||_h / ||1||_h on the sample's finest grid, k = 0..ncycles.
-// prog: one cycle, op.x = kind | (p or diagonal) << 4 | q << 12, op.y = zero-init.
+// Standard coarsening: hist[s][k] = ||1 - A u_k||_h / ||1||_h on the sample's finest grid,
+// k = 0..ncycles.  prog: one cycle, words kind | p << 4 | q << 12.
 template <class T>
-__global__ void k_cycle_history(DevCtx cx, T* su, T* sbx, T* sby, const T* ax, const T* ay, const int2* prog,
-                                int nops, int ncycles, CycleParams cp, int band, double* hist)
+__global__ void k_cycle_history(DevCtx cx, T* su, T* sbx, T* sby, const T* ax, const T* ay, const int* prog,
+                                int nops, int ncycles, CycleParams cp, double* hist)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];  // `band` residual nodes of the MSG restriction
     __shared__ double red[32];
     TaskRef t;
     if (!resolve_2d(cx, t)) return;
@@ -562,20 +561,10 @@ __global__ void k_cycle_history(DevCtx cx, T* su, T* sbx, T* sby, const T* ax, c
     for (int cyc = 0; cyc <= ncycles; ++cyc) {
         if (cyc > 0)
             for (int o = 0; o < nops; ++o) {
-                const int2 op = prog[o];
-                const int kind = op.x & 15, a = (op.x >> 4) & 255, b = (op.x >> 12) & 255;
-                if (kind == H_PRE || kind == H_POST) {
-                    for (int p = max(1, a + 2 - Q); p <= min(P, a + 1); ++p) {
-                        if (kind == H_PRE) visit_pre(grp, h, p, a + 2 - p, op.y, cp.nu1, (T*)smem_raw, band);
-                        else visit_post(grp, h, p, a + 2 - p, cp.nu2, (T)cp.omega);
-                    }
-                } else if (kind == H_STD_PRE) {
-                    cta_std_pre(grp, h, a, b, cp.nu1);
-                } else if (kind == H_STD_POST) {
-                    cta_std_post(grp, h, a, b, cp.nu2, (T)cp.omega);
-                } else {
-                    cta_std_line(grp, h, a, b);
-                }
+                const int op = prog[o], kind = op & 15, a = (op >> 4) & 255, b = (op >> 12) & 255;
+                if (kind == H_STD_PRE) cta_std_pre(grp, h, a, b, cp.nu1);
+                else if (kind == H_STD_POST) cta_std_post(grp, h, a, b, cp.nu2, (T)cp.omega);
+                else cta_std_line(grp, h, a, b);
             }
         double s = 0.0;
         for (int k = grp.tid; k < (top.ny - 1) * W; k += grp.n) {
@@ -2962,40 +2951,26 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
 // ------------------------------------------------- convergence study (host) --
 namespace {
 
-void hist_prog_msg(int s, int zi, int mu, std::vector<int2>& prog)
-{
-    prog.push_back(make_int2(H_PRE | s << 4, zi));
-    if (s == 0) return;
-    for (int k = 0; k < mu; ++k) hist_prog_msg(s - 1, k == 0, mu, prog);
-    prog.push_back(make_int2(H_POST | s << 4, 0));
-}
-
-void hist_prog_std(int p, int q, int mu, std::vector<int2>& prog)
+void hist_prog_std(int p, int q, int mu, std::vector<int>& prog)
 {
     if (p == 1 || q == 1) {
-        prog.push_back(make_int2(H_STD_LINE | p << 4 | q << 12, 0));
+        prog.push_back(H_STD_LINE | p << 4 | q << 12);
         return;
     }
-    prog.push_back(make_int2(H_STD_PRE | p << 4 | q << 12, 0));
+    prog.push_back(H_STD_PRE | p << 4 | q << 12);
     for (int k = 0; k < mu; ++k) hist_prog_std(p - 1, q - 1, mu, prog);
-    prog.push_back(make_int2(H_STD_POST | p << 4 | q << 12, 0));
-}
-
-std::vector<int2> hist_prog(int P, int Q, int method, int mu)
-{
-    std::vector<int2> prog;
-    if (method == 0) hist_prog_msg(P + Q - 2, 0, mu, prog);  // the top keeps its iterate
-    else hist_prog_std(P, Q, mu, prog);
-    return prog;
+    prog.push_back(H_STD_POST | p << 4 | q << 12);
 }
 
 struct HistLayout {
-    size_t samples, gpos, slist, groups, segs, prog, ax, ay, su, sbx, sby, total;
+    size_t samples, gpos, slist, groups, segs, prog, ax, ay, su, sbx, sby;
+    size_t low_desc, low_ent, low_prog, low_img, op;  // MSG: matrices of the low diagonals and their tables
+    size_t total;
 };
 
-HistLayout hist_layout(int P, int Q, int64_t S, size_t nprog)
+HistLayout hist_layout(int P, int Q, int64_t S, const msg_params& prm, int method)
 {
-    HistLayout w;
+    HistLayout w{};
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += (b + 255) / 256 * 256; return o; };
     const size_t R = (size_t)rect_nodes(P, Q) * (size_t)S;
@@ -3003,8 +2978,20 @@ HistLayout hist_layout(int P, int Q, int64_t S, size_t nprog)
     w.gpos = take(sizeof(int) * S);
     w.slist = take(sizeof(int) * S);
     w.groups = take(sizeof(Group));
-    w.segs = take(sizeof(Segment) * (P * Q + 1));
-    w.prog = take(sizeof(int2) * nprog);
+    w.segs = take(sizeof(Segment) * (2 * P * Q + 1));
+    if (method == MSG_HIST_STANDARD) {
+        std::vector<int> prog;
+        hist_prog_std(P, Q, prm.mu, prog);
+        w.prog = take(sizeof(int) * prog.size());
+    } else {
+        const OpTables t = op_tables(prm);
+        const LowPlanes& lp = low_tables().planes[kOpD];
+        w.low_desc = take(sizeof(t.desc));
+        w.low_ent = take(sizeof(uint4) * t.ent.size());
+        w.low_prog = take(sizeof(uint2) * t.prog.size());
+        w.low_img = take(sizeof(double) * (lp.nfx + lp.nfy) * S);
+        w.op = take(sizeof(double) * op_offset(0, 0, P, Q) * S);
+    }
     w.ax = take(sizeof(double) * R);
     w.ay = take(sizeof(double) * R);
     w.su = take(sizeof(double) * R);
@@ -3106,7 +3093,7 @@ extern "C" size_t msg_history_workspace_bytes(int32_t P, int32_t Q, int64_t S, c
 {
     clear_error();
     if (hist_check(P, Q, S, prm, method, 1) != MSG_OK) return 0;
-    return hist_layout(P, Q, S, hist_prog(P, Q, method, prm->mu).size()).total;
+    return hist_layout(P, Q, S, *prm, method).total;
 }
 
 extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_params* prm, int32_t method,
@@ -3119,8 +3106,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
     if (S == 0) return MSG_OK;
     if (!Z || !hist || !workspace) { set_error("Z, hist or workspace is NULL"); return MSG_ERR_INVALID; }
     if ((uintptr_t)workspace % 256) { set_error("workspace must be 256-byte aligned"); return MSG_ERR_INVALID; }
-    const std::vector<int2> prog = hist_prog(P, Q, method, prm->mu);
-    const HistLayout w = hist_layout(P, Q, S, prog.size());
+    const HistLayout w = hist_layout(P, Q, S, *prm, method);
     if (ws_bytes < w.total) {
         set_error("workspace too small: need " + std::to_string(w.total) + " bytes");
         return MSG_ERR_WORKSPACE;
@@ -3132,7 +3118,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
     std::vector<SampleInfo> samples(S);
     std::vector<int> ids(S);
     for (int64_t s = 0; s < S; ++s) {
-        samples[s] = SampleInfo{P, Q, s * R, s * nf, 0, 0};
+        samples[s] = SampleInfo{P, Q, s * R, s * nf, 0, s * op_offset(0, 0, P, Q)};
         ids[s] = (int)s;
     }
     const Group grp{P, Q, 0, (int)S, 0, R};
@@ -3141,12 +3127,30 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
         for (int q = 1; q <= Q; ++q)
             segs.push_back(Segment{0, P, Q, p, q, (int64_t)segs.size() * S, S, 0, 0, 0});
     segs.push_back(Segment{0, P, Q, P, Q, 0, S, 0, 0, 0});
+    // MSG on a hierarchy larger than a CTA: the grids of each diagonal above the cut
+    const int L = P + Q - 2;
+    std::vector<VisitList> lists(L + 1);
+    std::vector<size_t> first(L + 1, 0);
+    if (method == MSG_HIST_MSG && L > kItemL64)
+        for (int d = kMidD + 1; d <= L; ++d) {
+            first[d] = segs.size();
+            for (int part = 0; part < 2; ++part) {
+                for (int p = std::max(1, d + 2 - Q); p <= std::min(P, d + 1); ++p) {
+                    const int q = d + 2 - p;
+                    if (visit_takes<double>(d, q) != (part == 0)) continue;
+                    Segment sg{0, P, Q, p, q, 0, S, 0, 0, 0};
+                    visit_offsets(sg, grp);
+                    segs.push_back(sg);
+                }
+                if (part == 0) lists[d].fall = segs.size() - first[d];
+            }
+            lists[d].n = segs.size() - first[d];
+        }
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.samples, samples.data(), sizeof(SampleInfo) * S, cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.gpos, ids.data(), sizeof(int) * S, cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.slist, ids.data(), sizeof(int) * S, cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.groups, &grp, sizeof(Group), cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.segs, segs.data(), sizeof(Segment) * segs.size(), cudaMemcpyHostToDevice, st));
-    MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.prog, prog.data(), sizeof(int2) * prog.size(), cudaMemcpyHostToDevice, st));
     DevCtx cx;
     cx.samples = (const SampleInfo*)(ws + w.samples);
     cx.gpos = (const int*)(ws + w.gpos);
@@ -3163,14 +3167,76 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
     DevCtx ch = cx;
     ch.segs = cx.segs + P * Q;
     ch.nseg = 1;
-    const int band = std::max(kBandNodes, 3 * ((1 << P) + 1));
+    double* su = (double*)(ws + w.su);
+    double* sbx = (double*)(ws + w.sbx);
+    double* sby = (double*)(ws + w.sby);
     const CycleParams cp{prm->mu, prm->nu1, prm->nu2, prm->omega};
-    prof_begin(K_PRE, st);
-    k_cycle_history<double><<<dim3((unsigned)S, 1), 256, sizeof(double) * band, st>>>(
-        ch, (double*)(ws + w.su), (double*)(ws + w.sbx), (double*)(ws + w.sby), ax, ay,
-        (const int2*)(ws + w.prog), (int)prog.size(), ncycles, cp, band, hist);
-    prof_end(K_PRE, st, 0.0, 0.0);
+    if (method == MSG_HIST_STANDARD) {
+        std::vector<int> prog;
+        hist_prog_std(P, Q, prm->mu, prog);
+        MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.prog, prog.data(), sizeof(int) * prog.size(), cudaMemcpyHostToDevice, st));
+        prof_begin(K_PRE, st);
+        k_cycle_history<double><<<dim3((unsigned)S, 1), 256, 0, st>>>(ch, su, sbx, sby, ax, ay, (const int*)(ws + w.prog),
+                                                                     (int)prog.size(), ncycles, cp, hist);
+        prof_end(K_PRE, st, 0.0, 0.0);
+        MSG_CHECK_LAUNCH();
+        MSG_CUDA_TRY(cudaStreamSynchronize(st));  // prog is read by its copy
+        return MSG_OK;
+    }
+    const OpTables ot = op_tables(*prm);
+    const LowPlanes& lp = low_tables().planes[kOpD];
+    MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.low_desc, ot.desc, sizeof(ot.desc), cudaMemcpyHostToDevice, st));
+    MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.low_ent, ot.ent.data(), sizeof(uint4) * ot.ent.size(), cudaMemcpyHostToDevice, st));
+    MSG_CUDA_TRY(cudaMemcpyAsync(ws + w.low_prog, ot.prog.data(), sizeof(uint2) * ot.prog.size(), cudaMemcpyHostToDevice, st));
+    prof_begin(K_COEFFS, st);
+    k_lowimg<double><<<(unsigned)S, kThreads, 0, st>>>(cx.samples, ax, ay, lp, (double*)(ws + w.low_img),
+                                                       (int64_t)(lp.nfx + lp.nfy), lp.nfx);
+    prof_end(K_COEFFS, st, (double)S * (lp.nfx + lp.nfy) * 16.0, 0.0);
     MSG_CHECK_LAUNCH();
+    double* op = (double*)(ws + w.op);
+    rc = matrices<double>(ot, std::vector<Group>{grp}, cx.samples, (int)S, (const double*)(ws + w.low_img),
+                          (const LowDesc*)(ws + w.low_desc), (const uint4*)(ws + w.low_ent), (const uint2*)(ws + w.low_prog),
+                          *prm, op, st);
+    if (rc != MSG_OK) return rc;
+    if (L <= kItemL64) {
+        const size_t sm = sizeof(double) * mid_total(P, Q, L > kOpD ? kOpD + 1 : 0, L, prm->nu1);
+        MSG_CUDA_TRY(cudaFuncSetAttribute(k_history_chip, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
+        prof_begin(K_LOW, st);
+        k_history_chip<<<(unsigned)S, item_threads<double>(L), sm, st>>>(ch, L, ax, ay, op, cp, ncycles, hist);
+        prof_end(K_LOW, st, 0.0, 0.0, L);
+        MSG_CHECK_LAUNCH();
+    } else {
+        rc = cycle_attributes<double>();
+        if (rc != MSG_OK) return rc;
+        for (int d = kMidD + 1; d <= L; ++d) {
+            lists[d].cx = cx;
+            lists[d].cx.segs = cx.segs + first[d];
+            lists[d].host = segs.data() + first[d];
+        }
+        const int n = ((1 << P) + 1) * ((1 << Q) + 1);
+        k_history_start<<<dim3((unsigned)((n + 255) / 256), (unsigned)S), 256, 0, st>>>(P, Q, R, su, sbx);
+        MSG_CHECK_LAUNCH();
+        bool bad = false;
+        for (int cyc = 0; cyc <= ncycles && !bad; ++cyc) {
+            if (cyc > 0)
+                cycle_launches(
+                    L, kMidD, prm->mu, false,
+                    [&](int d, int pre, int zi) {
+                        bad |= visit_half<double>(lists[d], d, pre, zi, su, sbx, sby, ax, ay, *prm, kVisitThreads, kVisitSmemKB * 1024, st);
+                    },
+                    [&](int, int) {
+                        prof_begin(K_LOW, st);
+                        k_mid<double><<<(unsigned)S, kMidThreads, mid_smem<double>(prm->nu1), st>>>(ch, su, sbx, sby, ax, ay, op, cp);
+                        prof_end(K_LOW, st, 0.0, 0.0, kMidD);
+                        bad |= cudaGetLastError() != cudaSuccess;
+                    });
+            prof_begin(K_RESIDUAL, st);
+            k_history_norm<<<(unsigned)S, 1024, 0, st>>>(P, Q, R, su, ax, ay, hist + cyc, ncycles + 1);
+            prof_end(K_RESIDUAL, st, (double)S * n * 24.0, 0.0);
+            bad |= cudaGetLastError() != cudaSuccess;
+        }
+        if (bad) { set_error("kernel launch failed in the cycle schedule"); return MSG_ERR_CUDA; }
+    }
     // the host tables above are read by the copies: finish before they go out of scope
     MSG_CUDA_TRY(cudaStreamSynchronize(st));
     return MSG_OK;

@@ -12,6 +12,7 @@ the floor is 2^-52 |A| |u| with |A| <= 2 a_max (4^p + 4^q) and |u| <= 1 / (8 a_m
 import numpy as np
 import pytest
 
+import oracle
 from paper_1907_12334_gb300 import inputs
 
 pytestmark = pytest.mark.gpu
@@ -46,3 +47,22 @@ def test_on_chip_cycles_match_the_phase_kernels(mu, nu1, nu2, precision):
                 floor = 2.0 ** -52 * 2 * contrast * (4.0 ** p + 4.0 ** q) / 8
                 assert floor > kw["eps"] or abs(int(a[2][k]) - int(b[2][k])) <= 1, (P, Q, p, q)
                 k += 1
+
+
+@pytest.mark.parametrize("P,Q,kw", [(5, 6, {}), (7, 4, dict(nu1=1, nu2=3)), (9, 2, {}), (2, 9, dict(mu=1)), (6, 6, dict(nu1=0)),
+                                    (1, 10, {})])
+def test_history_beyond_one_cta_matches_oracle(P, Q, kw):
+    """Residual histories on hierarchies that run on launches of visits and k_mid: both
+    sides in FP64, so they agree to 1e-8 relative down to the residual's rounding floor
+    (as above, four times: two sides, and rounding of u beside that of the residual)."""
+    from paper_1907_12334_gb300 import build, msg
+
+    build.build()
+    n, Z = 6, inputs.smooth_field(P, Q, 1.0)
+    h = msg.msg_cycle_history(P, Q, 2, msg.SolverParams(**kw), 0, torch.from_numpy(np.concatenate([Z, -Z])).to(DEV), n)
+    floor = 2.0 ** -52 * 2 * np.exp(np.ptp(Z)) * (4.0 ** P + 4.0 ** Q) / 8
+    prm = msg.SolverParams(**kw)
+    op = oracle.SolverParams(mu=prm.mu, nu1=prm.nu1, nu2=prm.nu2, omega=prm.omega)
+    for k, z in enumerate((Z, -Z)):
+        ho = oracle.Hierarchy(P, Q, Z=z, prm=op).cycle_history(0, n)
+        np.testing.assert_allclose(h[k].cpu().numpy(), ho, rtol=1e-8, atol=4 * floor)
