@@ -2,6 +2,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -111,6 +112,34 @@ int staging_release(int token, cudaStream_t st)
     s.pending = true;
     s.held = false;
     return MSG_OK;
+}
+
+cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st)
+{
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    cudaMemPool_t pool = nullptr;
+    if (e == cudaSuccess) {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = pools.find(dev);
+        if (it != pools.end()) {
+            pool = it->second;
+        } else {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            e = cudaMemPoolCreate(&pool, &props);
+            uint64_t keep = kTempKeep;
+            if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e == cudaSuccess) pools[dev] = pool;
+        }
+    }
+    if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 
 void set_error(const std::string& what) { g_last_error = what; }

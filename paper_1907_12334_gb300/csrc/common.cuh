@@ -40,6 +40,51 @@ void clear_error();
 int staging_acquire(size_t bytes, void** ptr, int* token);
 int staging_release(int token, cudaStream_t st);
 
+// Stream-ordered temporary (freed with cudaFreeAsync on the same stream) from a pool of
+// this library's own, one per device, made on first use.  It keeps up to kTempKeep bytes
+// between calls: the device's default pool gives everything back at each
+// synchronisation, and mapping it again cost a call 200 us.  Returns the CUDA error, and
+// leaves none pending.
+constexpr uint64_t kTempKeep = uint64_t(64) << 20;
+cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st);
+
+// (TZ)x of FP32 results, exact.  The conversion instruction to FP64 runs at the FP64
+// pipe's rate (two a clock and SM), a limit of its own for kernels that write FP64 fields
+// from FP32 sums; a normal number is widened by moving its IEEE-754 fields instead: the
+// exponent's bias grows by 1023 - 127 = 896, the 23-bit fraction moves to the top of 52 bits.
+__device__ __forceinline__ bool widens(float x)  // neither zero, subnormal, infinite nor NaN
+{
+    return (__float_as_uint(x) & 0x7fffffffu) - 0x00800000u < 0x7f000000u;
+}
+__device__ __forceinline__ double widen_normal(float x)
+{
+    const uint32_t u = __float_as_uint(x);
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (896u << 20))), (int)(u << 29));
+}
+// N results at p, p + stride, ..; one test for all of them keeps the stores free of branches
+template <int N>
+__device__ __forceinline__ void store_wide(float* p, int64_t stride, const float (&v)[N], int n)
+{
+#pragma unroll
+    for (int k = 0; k < N; ++k, p += stride)
+        if (k < n) *p = v[k];
+}
+template <int N>
+__device__ __forceinline__ void store_wide(double* p, int64_t stride, const float (&v)[N], int n)
+{
+    bool all = n >= N;
+#pragma unroll
+    for (int k = 0; k < N; ++k) all &= widens(v[k]);
+    if (all) {
+#pragma unroll
+        for (int k = 0; k < N; ++k, p += stride) *p = widen_normal(v[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < N; ++k, p += stride)
+            if (k < n) *p = (double)v[k];
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Hierarchy layout.
 //

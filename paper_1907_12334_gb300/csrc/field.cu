@@ -42,34 +42,181 @@ __global__ void k_normals(uint64_t seed, uint64_t s0, int64_t S, int M, double* 
 }
 
 // ---------------------------------------------------------------- SIMT GEMM --
-// Z[s][x] = sum_m Phi[x][m] * (sqrt_lambda[m] * xi[s][m]); 64x64 tile per CTA,
-// 16-deep K slices staged in shared memory, 4x4 outputs per thread.
-template <class TP, class TA, class TZ>
-__global__ void __launch_bounds__(256) k_kl_simt(const TP* __restrict__ Phi, const double* __restrict__ sl,
+// Z[s][x] = sum_m Phi[x][m] * A[s][m], A = sqrt_lambda[m] * xi[s][m], terms in
+// increasing m, one fused multiply-add each: every kernel here gives the same bits.
+
+// A rounded to FP32 once per call, rows padded to a multiple of four terms with zeros.
+// (The product is taken in FP64, whose rate is 1/64 of FP32's here: formed again in every
+// tile, as k_kl_simt does, it costs as much as the contraction.)
+__global__ void k_kl_a32(const double* __restrict__ sl, const double* __restrict__ xi, int64_t S, int M, int Mp, float* A)
+{
+    const int64_t n = S * Mp;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t s = e / Mp;
+        const int m = (int)(e - s * Mp);
+        A[e] = m < M ? (float)(sl[m] * xi[s * M + m]) : 0.f;
+    }
+}
+
+// FP32: a tile of 16 TR samples x 128 points per CTA, TR x 8 outputs per thread (samples
+// ty TR .. + TR - 1, points tx + 16 b: the half warps of a store write 16 consecutive
+// points).  Bound by the FMA pipe: 8 TR FMAs for 8 + TR / 4 shared loads a term; the next
+// 16 terms travel to registers meanwhile.  Sample tiles are the fastest grid index, so the
+// CTAs that read one tile of Phi run together and find it in L2.  513 x 513 points, 400
+// terms, 512 samples: 5.25 ms with the 64 x 64
+// tiles of k_kl_simt, 2.35 ms here (46 TFLOP/s).
+template <int TR, class TZ>
+__global__ void __launch_bounds__(256, 2) k_kl_f32(const float* __restrict__ Phi, const float* __restrict__ A, int64_t npts,
+                                                   int M, int Mp, int64_t S, int64_t stiles, int vec, TZ* __restrict__ Z)
+{
+    constexpr int TS = 16 * TR, TX = 128, BK = 16, LA = TS + 4, LB = TX + 4;
+    __shared__ __align__(16) float sA[2][BK * LA], sB[2][BK * LB];
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int64_t s0 = (int64_t)(blockIdx.x % stiles) * TS, x0 = (int64_t)(blockIdx.x / stiles) * TX;
+    // loads: four consecutive terms of a row each (rows past the end: the last row, not stored)
+    constexpr int NA = (TS * 4 + 255) / 256, NB = TX * 4 / 256;
+    const int kq = 4 * (tid & 3), row = tid >> 2;
+    // vec: every row of Phi starts on 16 bytes
+    float4 ra[NA], rb[NB];
+    // this thread's rows relative to the tiles, at its first terms
+    const float *tA = A + s0 * Mp, *tB = Phi + x0 * M;
+    int oa[NA], ob[NB];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) oa[i] = (int)min((int64_t)(row + 64 * i), S - 1 - s0) * Mp + kq;
+#pragma unroll
+    for (int i = 0; i < NB; ++i) ob[i] = (int)min((int64_t)(row + 64 * i), npts - 1 - x0) * M + kq;
+    const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto fetch = [&](int k0) {
+        const int k = k0 + kq;
+#pragma unroll
+        for (int i = 0; i < NA; ++i)
+            ra[i] = (k < Mp && row + 64 * i < TS) ? *reinterpret_cast<const float4*>(tA + oa[i] + k0) : none;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const float* p = tB + ob[i] + k0;
+            if (vec) rb[i] = k < M ? *reinterpret_cast<const float4*>(p) : none;
+            else
+                rb[i] = make_float4(k < M ? p[0] : 0.f, k + 1 < M ? p[1] : 0.f, k + 2 < M ? p[2] : 0.f, k + 3 < M ? p[3] : 0.f);
+        }
+    };
+    auto store = [&](int h) {
+#pragma unroll
+        for (int i = 0; i < NA; ++i) {
+            float* d = &sA[h][kq * LA + row + 64 * i];
+            if (row + 64 * i >= TS) continue;
+            d[0] = ra[i].x; d[LA] = ra[i].y; d[2 * LA] = ra[i].z; d[3 * LA] = ra[i].w;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            float* d = &sB[h][kq * LB + row + 64 * i];
+            d[0] = rb[i].x; d[LB] = rb[i].y; d[2 * LB] = rb[i].z; d[3 * LB] = rb[i].w;
+        }
+    };
+    float acc[TR][8];
+#pragma unroll
+    for (int a = 0; a < TR; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+    fetch(0);
+    store(0);
+    __syncthreads();
+    for (int k0 = 0, h = 0; k0 < Mp; k0 += BK, h ^= 1) {
+        if (k0 + BK < Mp) fetch(k0 + BK);
+        const float *a0 = sA[h] + ty * TR, *b0 = sB[h] + tx;
+#pragma unroll 8
+        for (int k = 0; k < BK; ++k) {
+            float av[TR], bv[8];
+#pragma unroll
+            for (int a = 0; a < TR; a += TR < 4 ? TR : 4) {
+                if constexpr (TR < 4) {
+                    const float2 v = *reinterpret_cast<const float2*>(a0 + k * LA);
+                    av[0] = v.x; av[1] = v.y;
+                } else {
+                    const float4 v = *reinterpret_cast<const float4*>(a0 + k * LA + a);
+                    av[a] = v.x; av[a + 1] = v.y; av[a + 2] = v.z; av[a + 3] = v.w;
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < 8; ++b) bv[b] = b0[k * LB + 16 * b];
+#pragma unroll
+            for (int a = 0; a < TR; ++a)
+#pragma unroll
+                for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+        }
+        if (k0 + BK < Mp) store(h ^ 1);  // the other buffer was read before the last barrier
+        __syncthreads();
+    }
+#pragma unroll
+    for (int a = 0; a < TR; ++a) {
+        const int64_t s = s0 + ty * TR + a;
+        if (s >= S) continue;
+        const int64_t left = npts - x0 - tx;  // points from this thread's first on
+        store_wide<8>(Z + s * npts + x0 + tx, 16, acc[a], (int)min((left + 15) >> 4, (int64_t)8));
+    }
+}
+
+// FP64: a tile of 8 samples x 32 points per CTA, one output per thread.  Bound by the FP64
+// pipe (two FMAs a clock and SM), so what counts is work done for padding and an even
+// spread over the SMs: small tiles, with a warp's points consecutive.  129 x 65 points, 64
+// terms, 24 samples: 71.8 us with 64 x 64 tiles, 28.7 us here (23 us at
+// the FP64 rate).
+template <class TZ>
+__global__ void __launch_bounds__(256) k_kl_f64(const double* __restrict__ Phi, const double* __restrict__ sl,
+                                                const double* __restrict__ xi, int64_t npts, int M, int64_t S, int64_t xtiles,
+                                                TZ* __restrict__ Z)
+{
+    constexpr int BK = 64;
+    __shared__ double sA[8][BK], sB[BK][33];
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int64_t x0 = (int64_t)(blockIdx.x % xtiles) * 32, s0 = (int64_t)(blockIdx.x / xtiles) * 8;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < M; k0 += BK) {
+        const int nk = min(BK, M - k0);
+        for (int e = tid; e < 8 * BK; e += 256) {
+            const int r = e >> 6, k = e & 63;
+            if (k < nk) sA[r][k] = s0 + r < S ? sl[k0 + k] * xi[(s0 + r) * M + k0 + k] : 0.0;
+        }
+        for (int e = tid; e < 32 * BK; e += 256) {
+            const int r = e >> 6, k = e & 63;
+            if (k < nk) sB[k][r] = Phi[min(x0 + r, npts - 1) * M + k0 + k];
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int k = 0; k < nk; ++k) acc = fma(sA[ty][k], sB[k][tx], acc);
+        __syncthreads();
+    }
+    const int64_t x = x0 + tx, s = s0 + ty;
+    if (x < npts && s < S) Z[s * npts + x] = (TZ)acc;
+}
+
+// FP32 without a temporary for A (when none can be had): 64x64 tile per CTA, 16-deep K
+// slices staged in shared memory, 4x4 outputs per thread.
+template <class TZ>
+__global__ void __launch_bounds__(256) k_kl_simt(const float* __restrict__ Phi, const double* __restrict__ sl,
                                                  const double* __restrict__ xi, int64_t npts, int M, int64_t S,
                                                  TZ* __restrict__ Z)
 {
-    __shared__ TA sA[16][64 + 1];  // [k][s]
-    __shared__ TA sB[16][64 + 1];  // [k][x]
+    __shared__ float sA[16][64 + 1];  // [k][s]
+    __shared__ float sB[16][64 + 1];  // [k][x]
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int64_t s0 = (int64_t)blockIdx.y * 64, x0 = (int64_t)blockIdx.x * 64;
-    TA acc[4][4];
+    float acc[4][4];
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = TA(0);
+        for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
     for (int k0 = 0; k0 < M; k0 += 16) {
         for (int e = threadIdx.x; e < 64 * 16; e += 256) {
             int r = e / 16, k = e % 16;
             int64_t s = s0 + r, x = x0 + r;
             int m = k0 + k;
-            sA[k][r] = (s < S && m < M) ? (TA)(sl[m] * xi[s * M + m]) : TA(0);
-            sB[k][r] = (x < npts && m < M) ? (TA)Phi[x * M + m] : TA(0);
+            sA[k][r] = (s < S && m < M) ? (float)(sl[m] * xi[s * M + m]) : 0.f;
+            sB[k][r] = (x < npts && m < M) ? Phi[x * M + m] : 0.f;
         }
         __syncthreads();
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-            TA av[4], bv[4];
+            float av[4], bv[4];
 #pragma unroll
             for (int a = 0; a < 4; ++a) av[a] = sA[k][ty * 4 + a];
 #pragma unroll
@@ -77,7 +224,7 @@ __global__ void __launch_bounds__(256) k_kl_simt(const TP* __restrict__ Phi, con
 #pragma unroll
             for (int a = 0; a < 4; ++a)
 #pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
+                for (int b = 0; b < 4; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
         }
         __syncthreads();
     }
@@ -121,6 +268,29 @@ extern "C" int32_t msg_normals(uint64_t seed, uint64_t s0, int64_t S, int32_t M,
 namespace {
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 }
+
+namespace {
+// The sample tile that pads S least; a temporary for A, or the kernel that needs none.
+template <class TZ>
+void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts, int M, int64_t S, TZ* Z, cudaStream_t st)
+{
+    const int Mp = (M + 3) & ~3, TR = S <= 32 ? 2 : S <= 64 ? 4 : 8;
+    const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = stiles * ((npts + 127) / 128);
+    void* A = nullptr;
+    if (tiles > 0x7fffffffLL || temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) {
+        const dim3 grid((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
+        k_kl_simt<TZ><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
+        return;
+    }
+    k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);
+    const unsigned g = (unsigned)tiles;
+    const int vec = M == Mp && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
+    if (TR == 2) k_kl_f32<2, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
+    else if (TR == 4) k_kl_f32<4, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
+    else k_kl_f32<8, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
+    cudaFreeAsync(A, st);
+}
+}  // namespace
 
 extern "C" size_t kl_prepared_bytes(int64_t npts, int32_t M, int32_t mode)
 {
@@ -180,23 +350,25 @@ extern "C" int32_t sample_field(const void* prepared, int64_t npts, int32_t M, i
         return kl_tc_sample(prepared, npts, M, mode, xi, S, Z, z_fp32, st);
     }
     if (S > 65535LL * 64) { set_error("sample_field: too many samples for one call"); return MSG_ERR_INVALID; }
-    dim3 grid((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
     const char* base = (const char*)prepared;
     const double pe = mode == MSG_GEMM_FP64 ? 8.0 : 4.0, ze = z_fp32 ? 4.0 : 8.0;
+    if (mode != MSG_GEMM_FP64 && mode != MSG_GEMM_FP32) {
+        set_error("sample_field: unknown mode");
+        return MSG_ERR_INVALID;
+    }
     prof_begin(K_KL, st);
     if (mode == MSG_GEMM_FP64) {
         const double* Phi = (const double*)base;
         const double* sl = (const double*)(base + align256(sizeof(double) * npts * M));
-        if (z_fp32) k_kl_simt<double, double, float><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, (float*)Z);
-        else k_kl_simt<double, double, double><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, (double*)Z);
-    } else if (mode == MSG_GEMM_FP32) {
+        const int64_t xt = (npts + 31) / 32, tiles = xt * ((S + 7) / 8);
+        if (tiles > 0x7fffffffLL) { set_error("sample_field: too many points and samples for one call"); return MSG_ERR_INVALID; }
+        if (z_fp32) k_kl_f64<float><<<(unsigned)tiles, 256, 0, st>>>(Phi, sl, xi, npts, M, S, xt, (float*)Z);
+        else k_kl_f64<double><<<(unsigned)tiles, 256, 0, st>>>(Phi, sl, xi, npts, M, S, xt, (double*)Z);
+    } else {
         const float* Phi = (const float*)base;
         const double* sl = (const double*)(base + align256(sizeof(float) * npts * M));
-        if (z_fp32) k_kl_simt<float, float, float><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, (float*)Z);
-        else k_kl_simt<float, float, double><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, (double*)Z);
-    } else {
-        set_error("sample_field: unknown mode");
-        return MSG_ERR_INVALID;
+        if (z_fp32) kl_fp32<float>(Phi, sl, xi, npts, M, S, (float*)Z, st);
+        else kl_fp32<double>(Phi, sl, xi, npts, M, S, (double*)Z, st);
     }
     prof_end(K_KL, st, pe * npts * M + 8.0 * S * M + ze * S * npts, 2.0 * npts * M * S);
     MSG_CHECK_LAUNCH();

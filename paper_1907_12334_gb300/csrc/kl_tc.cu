@@ -376,7 +376,7 @@ int tc_launch(const TcLayout& L, const char* b, int64_t npts, int32_t M, const d
     const size_t apart = (size_t)Sp * L.Kp * sizeof(E), apart_al = (apart + 255) / 256 * 256;
     // the converted A lives in a stream-ordered temporary, freed after the contraction
     char* abuf = nullptr;
-    MSG_CUDA_TRY(cudaMallocAsync((void**)&abuf, parts * apart_al, st));
+    MSG_CUDA_TRY(temp_alloc((void**)&abuf, parts * apart_al, st));
     E* A0 = (E*)abuf;
     E* A1 = parts == 2 ? (E*)(abuf + apart_al) : nullptr;
     k_prep_a<MODE><<<152 * 4, 256, 0, st>>>((const double*)(b + L.sl), xi, S, M, L.Kp, Sp, A0, A1);

@@ -86,7 +86,7 @@ extern "C" int32_t mimc_differences(const int32_t* L, int64_t S, int32_t p0, int
     }
     if (ptau) memcpy((char*)hp + tb_al, ptau, pb);
     char* dbuf = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&dbuf, tb_al + pb + 256, st);
+    cudaError_t e = temp_alloc((void**)&dbuf, tb_al + pb + 256, st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dbuf, hp, tb_al + pb, cudaMemcpyHostToDevice, st);
     const int rel = staging_release(token, st);
     if (e != cudaSuccess) {
