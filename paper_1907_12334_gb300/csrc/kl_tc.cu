@@ -10,20 +10,34 @@
 // and the bench.
 //
 // Z[s][x] = sum_m A[s][m] B[x][m] with A = sqrt(lambda) * xi (samples x terms)
-// and B = Phi (points x terms).  One CTA computes a 128 (samples) x 256 (points)
-// tile of Z: accumulators in 256 TMEM columns, K in 128-byte chunks (64 bf16 or
-// 32 TF32 terms) staged through shared memory in the 128-byte-swizzled K-major
-// layout the UMMA descriptors expect.  A is converted from FP64
-// xi and sqrt(lambda) once per call into a stream-ordered temporary; B is
-// converted once per basis by kl_tc_prepare; both are zero-padded [rows][Kp] part
-// arrays whose tiles arrive by 16-byte asynchronous copies (cp.async) through a
-// ring of stages (2 for BF16X3, 4 for TF32) filled ahead of the MMAs that read
-// them.  One elected thread issues the
-// MMAs and commits them to an mbarrier per stage; every wait is bounded and a
-// timeout sets a device flag (read by msg_device_status) instead of hanging.  The
-// epilogue moves each warp's 32 x 32 accumulator blocks through shared memory so
-// that every global store of a warp writes 32 consecutive points of one sample.
+// and B = Phi (points x terms), as zero-padded [rows][Kp] part arrays: B's are made
+// once per basis by kl_tc_prepare, A's once per call in a stream-ordered temporary.
+//
+// k_kl_tc is persistent, one CTA per SM over tiles of 128 samples x 256 points, with
+// a role per warp:
+//   warp 0   loads: TMA tiles of both operands, 32 terms a stage (64 bytes of a row in
+//            bf16, 128 in TF32) in the swizzled K-major layout the UMMA descriptors
+//            expect, through a ring of 4 stages of 48 KB (with 2 stages of 64 terms one
+//            load at a time was in flight: 2.11 ms for the BF16X3 size below);
+//   warp 1   issues the MMAs of a stage and commits them to its "empty" barrier, and the
+//            last of a tile to the accumulator's "full" barrier;
+//   warps 4-11  epilogue: 32 x 32 accumulator blocks through a padded shared tile, so that
+//            every global store of a warp writes 32 consecutive points of one sample.
+// Two accumulators of 256 TMEM columns alternate, so the loads and MMAs of the next tile
+// run under the stores of the last.  Bound by the tensor pipe (BF16X3: three products a
+// term) and by the Z stores; with the three steps of a tile one after the other in
+// 152 x 54 CTAs it took 3.58 ms for 1024 x 1024 points, 400 terms, 1024 samples in
+// BF16X3, now 1.90 ms; 257 x 129 points, 300 terms, 777
+// samples, FP64 fields in TF32: 113 -> 76 us.
+// Sample tiles are the fastest tile index: the CTAs that read one Phi tile run together
+// and find it in L2 (A is small and stays there).  Every wait is bounded; one that runs
+// out sets a device flag (read by msg_device_status), ends every role and leaves
+// the rest of the output unwritten.
+#include <cuda.h>
+
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "kl_tc.cuh"
@@ -35,10 +49,8 @@ namespace {
 
 constexpr int kTM = 128;  // samples per tile (UMMA M)
 constexpr int kTN = 256;  // points per tile (UMMA N)
-constexpr int kThreadsTC = 256;
-constexpr int kRowBytes = 128;                        // one swizzled K row
-constexpr int kAbytes = kTM * kRowBytes;              // 16 KB per A part and stage
-constexpr int kBbytes = kTN * kRowBytes;              // 32 KB per B part and stage
+constexpr int kThreadsTC = 384;
+constexpr int kStages = 4;                            // of 48 KB
 constexpr long long kSpinLimit = 1ll << 22;           // bounded mbarrier waits (seconds)
 
 // Operand modes of the tensor-core kernel.
@@ -47,35 +59,37 @@ template <int MODE> struct TcCfg;
 template <> struct TcCfg<TC_BF16X3> {
     typedef __nv_bfloat16 E;
     static constexpr int parts = 2;   // hi, lo
-    static constexpr int TK = 64;     // terms per 128-byte row
-    static constexpr int stages = 2;  // 96 KB each
+    static constexpr int TK = 32;        // terms a stage
+    static constexpr int row_bytes = 64; // one swizzled K row of a stage
+    static constexpr int pad = 64;       // rows of the part arrays are padded to this many terms
 };
 template <> struct TcCfg<TC_TF32> {
     typedef float E;
     static constexpr int parts = 1;
     static constexpr int TK = 32;
-    static constexpr int stages = 4;  // 48 KB each
+    static constexpr int row_bytes = 128;
+    static constexpr int pad = 32;
 };
-template <int MODE> constexpr int stage_bytes() { return TcCfg<MODE>::parts * (kAbytes + kBbytes); }
-template <int MODE> constexpr int smem_bytes() { return TcCfg<MODE>::stages * stage_bytes<MODE>() + 1024; }  // + alignment slack
+template <int MODE> constexpr int a_bytes() { return kTM * TcCfg<MODE>::row_bytes; }  // per part and stage
+template <int MODE> constexpr int b_bytes() { return kTN * TcCfg<MODE>::row_bytes; }
+template <int MODE> constexpr int stage_bytes() { return TcCfg<MODE>::parts * (a_bytes<MODE>() + b_bytes<MODE>()); }
+constexpr int kEpiBytes = 8 * 32 * 33 * 4;  // a padded 32 x 32 block per epilogue warp
+template <int MODE> constexpr int smem_bytes() { return kStages * stage_bytes<MODE>() + kEpiBytes + 1024; }  // + alignment slack
 
 __host__ __device__ inline int64_t round_up(int64_t a, int64_t b) { return (a + b - 1) / b * b; }
 
 __device__ int g_tc_error;  // set by a kernel whose mbarrier wait ran out (sticky until msg_device_status)
 
-// Byte offset of 16-byte chunk `chunk` (0..7) of row r in a K-major tile with the
-// 128-byte swizzle: 8-row atoms of 1024 bytes, chunk c of row rr stored at
-// chunk position c ^ rr.
-__device__ __forceinline__ uint32_t sw128(int r, int chunk) { return (r >> 3) * 1024 + (r & 7) * 128 + ((chunk ^ (r & 7)) << 4); }
-
 // tcgen05 shared-memory matrix descriptor: start address >> 4 in bits 0-13,
 // leading byte offset >> 4 in 16-29 (unused by swizzled K-major tiles),
-// stride byte offset >> 4 in 32-45 (1024: next 8-row atom), descriptor
-// version 1 in bits 46-47, swizzle mode 2 (128-byte) in bits 61-63.
+// stride byte offset >> 4 in 32-45 (the next atom of 8 rows), descriptor
+// version 1 in bits 46-47, swizzle mode in bits 61-63 (2: 128-byte, 4: 64-byte).
+template <int MODE>
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr)
 {
-    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(16 >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) |
-           (1ull << 46) | (2ull << 61);
+    constexpr int row = TcCfg<MODE>::row_bytes;
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(16 >> 4) << 16) | ((uint64_t)(8 * row >> 4) << 32) | (1ull << 46) |
+           ((row == 128 ? 2ull : 4ull) << 61);
 }
 
 // Instruction descriptor: D = F32 (bits 4-5 = 1); A and B formats in bits 7-9
@@ -95,8 +109,9 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
 
-// Wait until the mbarrier phase with the given parity has completed; false on timeout.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
+// Wait until the mbarrier phase with the given parity has completed; false when the
+// limit runs out or another role gave up (*dead, which is then set).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* dead)
 {
     const uint32_t a = smem_u32(bar);
     for (long long it = 0; it < kSpinLimit; ++it) {
@@ -109,8 +124,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
             : "r"(a), "r"(parity)
             : "memory");
         if (done) return true;
+        if ((it & 15) == 15 && *dead) return false;
     }
+    *dead = 1;
     return false;
+}
+
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// The box of `map` at element x (a multiple of 64 bytes) and row y into shared memory.
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar)
+{
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+                 "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
+                 : "memory");
 }
 
 template <int MODE>
@@ -196,15 +230,16 @@ __global__ void k_tf32_phi(const double* Phi, int64_t npts, int M, int64_t Kp, i
 }
 
 // A = sqrt(lambda) * xi converted once per call into zero-padded [Sp][Kp] part
-// arrays in the operand format (the main loop then only copies).
+// arrays in the operand format (the main loop then only copies); a warp per row.
 template <int MODE>
-__global__ void k_prep_a(const double* sl, const double* xi, int64_t S, int M, int64_t Kp, int64_t Sp,
+__global__ void k_prep_a(const double* sl, const double* xi, int64_t S, int M, int Kp, int64_t Sp,
                          typename TcCfg<MODE>::E* A0, typename TcCfg<MODE>::E* A1)
 {
-    const int64_t n = Sp * Kp;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = e / Kp, m = e % Kp;
+    const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (s >= Sp) return;
+    for (int m = threadIdx.x & 31; m < Kp; m += 32) {
         const double v = (s < S && m < M) ? sl[m] * xi[s * M + m] : 0.0;
+        const int64_t e = s * Kp + m;
         if constexpr (MODE == TC_TF32) {
             A0[e] = to_tf32(v);
         } else {
@@ -216,133 +251,144 @@ __global__ void k_prep_a(const double* sl, const double* xi, int64_t S, int M, i
     }
 }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-
+// tile t: samples 128 (t mod stiles) .., points 256 (t / stiles) ..
 template <int MODE, class TZ>
 __global__ void __launch_bounds__(kThreadsTC, 1)
-    k_kl_tc(const typename TcCfg<MODE>::E* __restrict__ A0, const typename TcCfg<MODE>::E* __restrict__ A1,
-            const typename TcCfg<MODE>::E* __restrict__ B0, const typename TcCfg<MODE>::E* __restrict__ B1,
-            int64_t npts, int64_t Kp, int64_t S, TZ* __restrict__ Z)
+    k_kl_tc(const __grid_constant__ CUtensorMap mA0, const __grid_constant__ CUtensorMap mA1,
+            const __grid_constant__ CUtensorMap mB0, const __grid_constant__ CUtensorMap mB1, int64_t npts, int nchunks,
+            int64_t S, int stiles, int ntiles, TZ* __restrict__ Z)
 {
-    typedef typename TcCfg<MODE>::E E;
-    constexpr int parts = TcCfg<MODE>::parts, TK = TcCfg<MODE>::TK, NST = TcCfg<MODE>::stages;
-    constexpr int EPC = 16 / (int)sizeof(E);  // terms per 16-byte chunk
+    constexpr int parts = TcCfg<MODE>::parts, TK = TcCfg<MODE>::TK, NST = kStages, kAbytes = a_bytes<MODE>(), kBbytes = b_bytes<MODE>();
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[NST];
+    __shared__ __align__(8) uint64_t full[NST], empty[NST], acc_full[2], acc_empty[2];
     __shared__ uint32_t tmem_base_slot;
+    __shared__ volatile int dead;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // 1024-aligned stage buffers (swizzle atoms must start on 1024 bytes)
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char* base = smem_raw + (((raw + 1023) & ~1023u) - raw);
-    // blockIdx.x runs over the sample tiles: the CTAs that read one Phi tile are
-    // launched next to each other and find it in L2 (A is small and stays there)
-    const int64_t s0 = (int64_t)blockIdx.x * kTM, x0 = (int64_t)blockIdx.y * kTN;
 
-    if (warp == 0) {  // TMEM: 128 lanes x 256 FP32 columns
+    if (warp == 0) {  // TMEM: 128 lanes x 512 FP32 columns, two accumulators
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                     "r"(kTN)
+                     "r"(2 * kTN)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int k = 0; k < NST; ++k) mbar_init(&bars[k], 1);
+        for (int k = 0; k < NST; ++k) {
+            mbar_init(&full[k], 1);
+            mbar_init(&empty[k], 1);
+        }
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(&acc_full[k], 1);
+            mbar_init(&acc_empty[k], 8);
+        }
+        dead = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = tmem_base_slot;
+    auto stage = [&](int n) { return smem_u32(base + (n % NST) * stage_bytes<MODE>()); };  // A parts, then B parts
 
-    const int nchunks = (int)(Kp / TK);
-    // one chunk of A (128 rows) and B (256 rows) into its stage by 16-byte asynchronous copies
-    auto load_chunk = [&](int kc) {
-        unsigned char* sA = base + (kc % NST) * stage_bytes<MODE>();  // A parts, then B parts
-        unsigned char* sB = sA + parts * kAbytes;
-        for (int t = tid; t < kTM * 8; t += kThreadsTC) {
-            const int r = t >> 3, c = t & 7;
-            const int64_t g = (s0 + r) * Kp + (int64_t)kc * TK + c * EPC;
-            const uint32_t off = sw128(r, c);
-            cp_async16(smem_u32(sA + off), A0 + g);
-            if constexpr (parts == 2) cp_async16(smem_u32(sA + kAbytes + off), A1 + g);
+    if (warp == 0 && lane == 0) {  // ---- loads
+        int n = 0;  // stages filled
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+            const int s0 = (t % stiles) * kTM, x0 = (t / stiles) * kTN;
+            for (int kc = 0; kc < nchunks; ++kc, ++n) {
+                if (n >= NST && !(ok = mbar_wait(&empty[n % NST], ((n / NST) - 1) & 1, &dead))) break;
+                uint64_t* bar = &full[n % NST];
+                const uint32_t d = stage(n);
+                mbar_expect(bar, stage_bytes<MODE>());
+                tma_load(d, &mA0, kc * TK, s0, bar);
+                if constexpr (parts == 2) tma_load(d + kAbytes, &mA1, kc * TK, s0, bar);
+                tma_load(d + parts * kAbytes, &mB0, kc * TK, x0, bar);
+                if constexpr (parts == 2) tma_load(d + parts * kAbytes + kBbytes, &mB1, kc * TK, x0, bar);
+            }
         }
-        for (int t = tid; t < kTN * 8; t += kThreadsTC) {
-            const int r = t >> 3, c = t & 7;
-            const int64_t g = (x0 + r) * Kp + (int64_t)kc * TK + c * EPC;
-            const uint32_t off = sw128(r, c);
-            cp_async16(smem_u32(sB + off), B0 + g);
-            if constexpr (parts == 2) cp_async16(smem_u32(sB + kBbytes + off), B1 + g);
+        // copies in flight end before the CTA does (normally the MMAs have waited for them)
+        for (int k = n > NST ? n - NST : 0; k < n; ++k) {
+            int none = 0;
+            mbar_wait(&full[k % NST], (k / NST) & 1, &none);
         }
-    };
-    // prologue: the first NST-1 chunks in flight (one commit group per chunk, empty past the end)
-    for (int kc = 0; kc < NST - 1; ++kc) {
-        if (kc < nchunks) load_chunk(kc);
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    bool ok = true;
-    for (int kc = 0; kc < nchunks; ++kc) {
-        // chunk kc has landed once at most NST-2 newer groups are pending
-        asm volatile("cp.async.wait_group %0;" ::"n"(NST - 2) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // make the copies visible to the tensor cores
-        __syncthreads();
-        if (tid == 0) {
+    } else if (warp == 1 && lane == 0) {  // ---- MMAs
+        int n = 0, w = 0;  // stages read, tiles done
+        bool ok = true;
+        for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++w) {
+            const uint32_t acc = tmem + (uint32_t)((w & 1) * kTN);
+            if (w >= 2 && !(ok = mbar_wait(&acc_empty[w & 1], ((w >> 1) - 1) & 1, &dead))) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_u32(base + (kc % NST) * stage_bytes<MODE>());
-            const uint32_t b0 = a0 + parts * kAbytes;
+            for (int kc = 0; kc < nchunks; ++kc, ++n) {
+                if (!(ok = mbar_wait(&full[n % NST], (n / NST) & 1, &dead))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                const uint32_t a0 = stage(n), b0 = a0 + parts * kAbytes;
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {  // 4 MMA K steps of 32 bytes per 128-byte row
-                const uint32_t ko = ks * 32;
-                const uint32_t first = (kc == 0 && ks == 0) ? 0u : 1u;
-                mma<MODE>(tmem, smem_desc(a0 + ko), smem_desc(b0 + ko), first);
-                if constexpr (MODE == TC_BF16X3) {
-                    mma<MODE>(tmem, smem_desc(a0 + ko), smem_desc(b0 + kBbytes + ko), 1u);  // hi * lo
-                    mma<MODE>(tmem, smem_desc(a0 + kAbytes + ko), smem_desc(b0 + ko), 1u);  // lo * hi
+                for (int ks = 0; ks < TcCfg<MODE>::row_bytes / 32; ++ks) {  // MMA K steps of 32 bytes
+                    const uint32_t ko = ks * 32;
+                    const uint32_t first = (kc == 0 && ks == 0) ? 0u : 1u;
+                    mma<MODE>(acc, smem_desc<MODE>(a0 + ko), smem_desc<MODE>(b0 + ko), first);
+                    if constexpr (MODE == TC_BF16X3) {
+                        mma<MODE>(acc, smem_desc<MODE>(a0 + ko), smem_desc<MODE>(b0 + kBbytes + ko), 1u);  // hi * lo
+                        mma<MODE>(acc, smem_desc<MODE>(a0 + kAbytes + ko), smem_desc<MODE>(b0 + ko), 1u);  // lo * hi
+                    }
                 }
+                mma_commit(&empty[n % NST]);
             }
-            mma_commit(&bars[kc % NST]);
+            if (ok) mma_commit(&acc_full[w & 1]);
         }
-        // refill: chunk kc+NST-1 goes into the stage chunk kc-1 used, once its MMAs are done
-        const int nk = kc + NST - 1;
-        if (nk < nchunks) {
-            if (kc >= 1) ok &= mbar_wait(&bars[(kc - 1) % NST], ((kc - 1) / NST) & 1);
-            load_chunk(nk);
+        // MMAs in flight end before the memory they use is given back (normally the epilogue
+        // has waited for them)
+        if (!ok && n > 0) {
+            int none = 0;
+            mbar_wait(&empty[(n - 1) % NST], ((n - 1) / NST) & 1, &none);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
-    }
-    // the last commit completes after every MMA of the CTA
-    if (nchunks >= 1) ok &= mbar_wait(&bars[(nchunks - 1) % NST], ((nchunks - 1) / NST) & 1);
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    // every thread took part in the same waits; make the decision CTA-wide
-    const int all_ok = __syncthreads_and(ok ? 1 : 0);
-    if (!all_ok) {
-        if (tid == 0) atomicExch(&g_tc_error, 1);
-    } else {
-        // epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (samples), columns 128 (w / 4) .. +127
-        // (points); each 32 x 32 block goes through a padded shared tile so that the stores of a
-        // warp cover 32 consecutive points of one sample
-        const int lane_base = 32 * (warp & 3), col_base = 128 * (warp >> 2);
-        float* tile = reinterpret_cast<float*>(base) + warp * 32 * 33;  // the stages are free now
-        for (int cb = 0; cb < 128; cb += 32) {
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)lane_base << 16) + (uint32_t)(col_base + cb), v);
+    } else if (warp >= 4) {  // ---- epilogue
+        // warp w reads TMEM lanes 32 (w % 4) .. + 31 (samples), columns 128 ((w - 4) / 4) .. + 127 (points)
+        const int lane_base = 32 * (warp & 3), col_base = 128 * ((warp - 4) >> 2);
+        const uint32_t tile = smem_u32(base + NST * stage_bytes<MODE>()) + (warp - 4) * 32 * 33 * 4;
+        const uint32_t mine = tile + lane * 33 * 4, column = tile + lane * 4;
+        int w = 0;
+        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++w) {
+            const int64_t s0 = (int64_t)(t % stiles) * kTM + lane_base, x0 = (int64_t)(t / stiles) * kTN + col_base;
+            if (!mbar_wait(&acc_full[w & 1], (w >> 1) & 1, &dead)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t acc = tmem + ((uint32_t)lane_base << 16) + (uint32_t)((w & 1) * kTN + col_base);
+            const int rows = (int)min((int64_t)32, S - s0);  // may be <= 0
+            for (int cb = 0; cb < 128; cb += 32) {
+                float v[32];
+                tmem_ld32(acc + (uint32_t)cb, v);
+                if (cb == 96) {  // the accumulator is in registers: the MMAs may have it back
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[w & 1]);
+                }
 #pragma unroll
-            for (int k = 0; k < 32; ++k) tile[lane * 33 + k] = v[k];
-            __syncwarp();
-            const int64_t x = x0 + col_base + cb + lane;
-            for (int rr = 0; rr < 32; ++rr) {
-                const int64_t s = s0 + lane_base + rr;
-                if (s < S && x < npts) Z[s * npts + x] = (TZ)tile[rr * 33 + lane];
+                for (int k = 0; k < 32; ++k) asm volatile("st.shared.f32 [%0], %1;" ::"r"(mine + 4 * k), "f"(v[k]) : "memory");
+                __syncwarp();
+                const int64_t x = x0 + cb + lane;
+                TZ* z = Z + s0 * npts + x;
+                if (x < npts) {
+#pragma unroll
+                    for (int r0 = 0; r0 < 32; r0 += 16) {  // 16 loads in flight, then their stores
+                        float o[16];
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o[k]) : "r"(column + (r0 + k) * 33 * 4) : "memory");
+                        store_wide<16>(z + r0 * npts, npts, o, rows - r0);
+                    }
+                }
+                __syncwarp();
             }
-            __syncwarp();
         }
     }
+    __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (tid == 0 && dead) atomicExch(&g_tc_error, 1);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTN) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kTN) : "memory");
 }
 
 struct TcLayout {
@@ -354,7 +400,7 @@ TcLayout tc_layout(int64_t npts, int32_t M, int mode)
 {
     TcLayout L{};
     const bool tf = mode == TC_TF32;
-    L.Kp = round_up(M, tf ? TcCfg<TC_TF32>::TK : TcCfg<TC_BF16X3>::TK);
+    L.Kp = round_up(M, tf ? TcCfg<TC_TF32>::pad : TcCfg<TC_BF16X3>::pad);
     L.Np = round_up(npts, kTN);
     const size_t part = (size_t)L.Np * L.Kp * (tf ? sizeof(float) : sizeof(__nv_bfloat16));
     L.p0 = 0;
@@ -366,28 +412,72 @@ TcLayout tc_layout(int64_t npts, int32_t M, int mode)
 
 int tc_mode(int32_t gemm_mode) { return gemm_mode == MSG_GEMM_TF32 ? TC_TF32 : TC_BF16X3; }
 
+// cuTensorMapEncodeTiled through the runtime (no link against the driver library).
+typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                             const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                             CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeFn encode_fn()
+{
+    static const EncodeFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return (EncodeFn)p;
+    }();
+    return fn;
+}
+
+// Map of a [rows][Kp] part array in boxes of one stage's terms x box_rows.
+template <int MODE>
+bool part_map(CUtensorMap* m, const void* p, int64_t rows, int64_t Kp, int box_rows)
+{
+    typedef typename TcCfg<MODE>::E E;
+    const cuuint64_t dim[2] = {(cuuint64_t)Kp, (cuuint64_t)rows}, stride[1] = {(cuuint64_t)(Kp * sizeof(E))};
+    const cuuint32_t box[2] = {(cuuint32_t)TcCfg<MODE>::TK, (cuuint32_t)box_rows}, es[2] = {1, 1};
+    return encode_fn()(m, MODE == TC_TF32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                       const_cast<void*>(p), dim, stride, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       TcCfg<MODE>::row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int MODE, class TZ>
 int tc_launch(const TcLayout& L, const char* b, int64_t npts, int32_t M, const double* xi, int64_t S, void* Z,
               cudaStream_t st)
 {
     typedef typename TcCfg<MODE>::E E;
     constexpr int parts = TcCfg<MODE>::parts;
-    const int64_t Sp = round_up(S, kTM);
+    const int64_t Sp = round_up(S, kTM), stiles = Sp / kTM, ntiles = stiles * (L.Np / kTN);
+    if (ntiles > 0x7fffffffLL || Sp > 0x7fffffffLL) { set_error("sample_field: too many samples for one call"); return MSG_ERR_INVALID; }
     const size_t apart = (size_t)Sp * L.Kp * sizeof(E), apart_al = (apart + 255) / 256 * 256;
+    if (!encode_fn()) { set_error("cuTensorMapEncodeTiled is not available"); return MSG_ERR_UNSUPPORTED; }
     // the converted A lives in a stream-ordered temporary, freed after the contraction
     char* abuf = nullptr;
     MSG_CUDA_TRY(temp_alloc((void**)&abuf, parts * apart_al, st));
     E* A0 = (E*)abuf;
-    E* A1 = parts == 2 ? (E*)(abuf + apart_al) : nullptr;
-    k_prep_a<MODE><<<152 * 4, 256, 0, st>>>((const double*)(b + L.sl), xi, S, M, L.Kp, Sp, A0, A1);
-    MSG_CHECK_LAUNCH();
-    dim3 grid((unsigned)(Sp / kTM), (unsigned)(L.Np / kTN));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_kl_tc<MODE, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<MODE>()));
-    k_kl_tc<MODE, TZ><<<grid, kThreadsTC, smem_bytes<MODE>(), st>>>(A0, A1 ? A1 : A0, (const E*)(b + L.p0),
-                                                                     (const E*)(b + (parts == 2 ? L.p1 : L.p0)), npts,
-                                                                     L.Kp, S, (TZ*)Z);
-    MSG_CHECK_LAUNCH();
-    MSG_CUDA_TRY(cudaFreeAsync(abuf, st));
+    E* A1 = parts == 2 ? (E*)(abuf + apart_al) : A0;
+    CUtensorMap mA0, mA1, mB0, mB1;
+    const bool mapped = part_map<MODE>(&mA0, A0, Sp, L.Kp, kTM) && part_map<MODE>(&mA1, A1, Sp, L.Kp, kTM) &&
+                        part_map<MODE>(&mB0, b + L.p0, L.Np, L.Kp, kTN) &&
+                        part_map<MODE>(&mB1, b + (parts == 2 ? L.p1 : L.p0), L.Np, L.Kp, kTN);
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = mapped ? cudaSuccess : cudaErrorInvalidValue;
+    if (e == cudaSuccess) {
+        k_prep_a<MODE><<<(unsigned)((Sp + 7) / 8), 256, 0, st>>>((const double*)(b + L.sl), xi, S, M, (int)L.Kp, Sp, A0, A1);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_kl_tc<MODE, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<MODE>());
+    if (e == cudaSuccess) {
+        k_kl_tc<MODE, TZ><<<(unsigned)std::min<int64_t>(ntiles, std::max(sms, 1)), kThreadsTC, smem_bytes<MODE>(), st>>>(
+            mA0, mA1, mB0, mB1, npts, (M + TcCfg<MODE>::TK - 1) / TcCfg<MODE>::TK, S, (int)stiles, (int)ntiles, (TZ*)Z);
+        e = cudaGetLastError();
+    }
+    cudaFreeAsync(abuf, st);
+    if (e != cudaSuccess) { set_error(std::string("sample_field: ") + cudaGetErrorString(e)); return MSG_ERR_CUDA; }
     return MSG_OK;
 }
 
