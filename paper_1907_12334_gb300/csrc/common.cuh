@@ -101,6 +101,12 @@ __host__ __device__ __forceinline__ int64_t grid_offset(int p, int q, int Qtop)
 {
     return tsum(p - 1) * tsum(Qtop) + (int64_t)((1 << p) + 1) * tsum(q - 1);
 }
+// the same in 32 bits (a rectangle holds at most T(12)^2 < 2^27 nodes)
+__host__ __device__ __forceinline__ int grid_offset32(int p, int q, int Qtop)
+{
+    auto t = [](int n) { return (2 << n) - 2 + n; };
+    return t(p - 1) * t(Qtop) + ((1 << p) + 1) * t(q - 1);
+}
 __host__ __device__ __forceinline__ int64_t rect_nodes(int P, int Q) { return tsum(P) * tsum(Q); }
 __host__ __device__ __forceinline__ int64_t field_nodes(int P, int Q)
 {

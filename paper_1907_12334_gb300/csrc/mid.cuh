@@ -237,7 +237,7 @@ struct MidItem {
     Sm<T> b3;  // its right-hand side, compact
     Sm<T> u3;  // its result: the cells of diagonal kOpD
     const int2* at;  // first word of each diagonal in b, ax, ay (x) and in u (y)
-    int pic, qic, lo, hi;
+    int pic, qic, lo, klo, hi;
     int n3, ld3;
 };
 
@@ -250,24 +250,26 @@ __host__ __device__ __forceinline__ int mid_cells(int d, int pic, int qic)
 }
 __host__ __device__ __forceinline__ int mid_pad(int d, int pic) { return 4 + (1 << mid_phi(d, pic)); }
 
-// words of the arrays of an item: cells of diagonals lo..hi, their pads, the residual
-struct MidWords { int cells, pads, r; };
-__host__ __device__ __forceinline__ MidWords mid_words(int pic, int qic, int lo, int hi, int nu1)
+// words of the arrays of an item: cells of the diagonals whose coefficients and b are
+// stored (klo..hi; the ones below are kept in registers), cells of all, their pads, the residual
+struct MidWords { int cells, ucells, pads, r; };
+__host__ __device__ __forceinline__ MidWords mid_words(int pic, int qic, int lo, int klo, int hi, int nu1)
 {
-    MidWords w{0, 0, 0};
+    MidWords w{0, 0, 0, 0};
     for (int d = lo; d <= hi; ++d) {
         const int c = mid_cells(d, pic, qic), r = nu1 == 0 ? c : c >> 1;
-        w.cells += c;
+        w.cells += d >= klo ? c : 0;
+        w.ucells += c;
         w.pads += mid_pad(d, pic);
         w.r = r > w.r ? r : w.r;
     }
     return w;
 }
 constexpr int kU3 = 4 * 32 + 20;  // cells of diagonal kOpD and their pad
-__host__ __device__ __forceinline__ int mid_total(int pic, int qic, int lo, int hi, int nu1)
+__host__ __device__ __forceinline__ int mid_total(int pic, int qic, int lo, int klo, int hi, int nu1)
 {
-    const MidWords w = mid_words(pic, qic, lo, hi, nu1);
-    int t = 4 * w.cells + w.pads + w.r;
+    const MidWords w = mid_words(pic, qic, lo, klo, hi, nu1);
+    int t = 3 * w.cells + w.ucells + w.pads + w.r;
     if (lo > 0) {
         const int n = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
         t += n * op_ld(n) + kOpN + kU3;
@@ -278,11 +280,11 @@ __host__ __device__ __forceinline__ int mid_total(int pic, int qic, int lo, int 
 // The pointers of an item whose words start at sm (16-byte aligned), and the table
 // of its diagonals (written by thread 0; a CTA barrier comes before its first use).
 template <class T>
-__device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic, int lo, int hi, int nu1)
+__device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic, int lo, int klo, int hi, int nu1)
 {
     MidItem<T> m;
-    const MidWords w = mid_words(pic, qic, lo, hi, nu1);
-    m.pic = pic; m.qic = qic; m.lo = lo; m.hi = hi;
+    const MidWords w = mid_words(pic, qic, lo, klo, hi, nu1);
+    m.pic = pic; m.qic = qic; m.lo = lo; m.klo = klo; m.hi = hi;
     m.n3 = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
     m.ld3 = op_ld(m.n3);
     m.M = Sm<T>{(uint32_t)__cvta_generic_to_shared(sm)};
@@ -295,11 +297,12 @@ __device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic
     m.u = m.r.at(w.r);
     m.at = at;
     if (threadIdx.x == 0) {
-        int c = 0, pad = 0;
+        int c = 0, u = 0;
         for (int d = lo; d <= hi; ++d) {
-            at[d] = make_int2(c, c + pad);
-            c += mid_cells(d, pic, qic);
-            pad += mid_pad(d, pic);
+            at[d] = make_int2(c, u);
+            const int n = mid_cells(d, pic, qic);
+            c += d >= klo ? n : 0;
+            u += n + mid_pad(d, pic);
         }
     }
     return m;
@@ -344,14 +347,17 @@ struct Pair {
 
 // From the faces and values of nodes A (even column, u at address aA) and B: aw, am,
 // ae the faces west of A, between, east of B; s, n the south and north ones.  ok: a row
-// of nodes; hasA: A is not the west boundary; redB: B is the red node.
+// of nodes; hasA: A is not the west boundary; redB: B is the red node.  iR, iK: what the
+// nodes' values were scaled with.
 template <class T>
 __device__ __forceinline__ void pair_set(Pair<T>& P, uint32_t aA, int nx, bool ok, bool hasA, bool redB, T aw, T am, T ae,
-                                         T sA, T sB, T nA, T nB, T bA, T bB, T uA, T uB)
+                                         T sA, T sB, T nA, T nB, T bA, T bB, T uA, T uB, T& iR, T& iK)
 {
     constexpr uint32_t es = sizeof(T);
     const T dA = aw + am + sA + nA, dB = am + ae + sB + nB;
-    const T iA = hasA ? rcp_of(dA) : T(0), iB = ok ? rcp_of(dB) : T(0), iR = redB ? iB : iA, iK = redB ? iA : iB;
+    const T iA = hasA ? rcp_of(dA) : T(0), iB = ok ? rcp_of(dB) : T(0);
+    iR = redB ? iB : iA;
+    iK = redB ? iA : iB;
     P.w = ok ? nx * es : 0u;
     P.aR = aA + (ok && redB ? es : 0u);
     P.e = ok ? (redB ? es : 0u - es) : 0u;
@@ -376,8 +382,9 @@ __device__ __forceinline__ void pair_load(Pair<T>& P, const MidDiag<T>& g, int d
     const Sm<T> x = g.ax.at(c), y = g.ay.at(c);
     const T aw = x.at(-1).ld();
     const auto ae = x.ld2(), an = y.ld2(), as = y.at(ok ? -nx : 0).ld2(), bb = g.b.at(c).ld2(), uu = g.u.at(c).ld2();
+    T iR, iK;
     pair_set(P, g.u.at(cA).a, nx, ok, hasA, redB, aw, ae.x, ae.y, as.x, as.y, an.x, an.y, bb.x, bb.y, ok ? uu.x : T(0),
-             ok ? uu.y : T(0));
+             ok ? uu.y : T(0), iR, iK);
 }
 
 // b + sum a u of the red / black node
@@ -493,7 +500,7 @@ __device__ __forceinline__ void mid_restrict(const MidItem<T>& m, int d)
 // diagonal d-1 (whose correction restarts from zero).  After a black half sweep
 // the residual of a black node is zero up to the rounding of its own update, so
 // only the red nodes' is formed.
-template <class T, int NP>
+template <class T, int NP, bool RESTRICT = true>
 __device__ __forceinline__ void mid_pre(const MidItem<T>& m, int d, int nu1, bool zero)
 {
     const MidDiag<T> g = mid_diag(m, d);
@@ -517,6 +524,7 @@ __device__ __forceinline__ void mid_pre(const MidItem<T>& m, int d, int nu1, boo
             if (tid + k * nt < np) m.r.at(tid + k * nt).st(r);
         }
         __syncthreads();
+        if (!RESTRICT) return;
         mid_restrict<T, true>(m, d);
     } else {
         for (int k = tid; k < (g.ng << (d + 2)); k += nt) {
@@ -680,23 +688,23 @@ template <class T>
 __device__ __forceinline__ void mid_fill(const MidItem<T>& m, const SampleInfo& S, const T* ax, const T* ay, const T* op)
 {
     const int tid = threadIdx.x, nt = blockDim.x;
-    const MidWords w = mid_words(m.pic, m.qic, m.lo, m.hi, 1);
+    const MidWords w = mid_words(m.pic, m.qic, m.lo, m.klo, m.hi, 1);
+    const T *gx = ax + S.node_off, *gy = ay + S.node_off;
     int c0 = 0;
-    for (int d = m.lo; d <= m.hi; ++d)
-        for (int p = mid_plo(d, m.qic); p <= mid_phi(d, m.pic); ++p) {
-            const T* gx = ax + S.node_off + grid_offset(p, d + 2 - p, S.Q);
-            const T* gy = ay + (gx - ax);
+    for (int d = m.klo; d <= m.hi; ++d) {
+        const int nc = mid_cells(d, m.pic, m.qic), plo = mid_plo(d, m.qic);
 #pragma unroll 2
-            for (int k = tid; k < 4 << d; k += nt) {  // cell (i, j) is node (i, j) of rows of 2^p + 1
-                const int o = k + (k >> p);
-                const T x = gx[o], y = gy[o];
-                m.ax.at(c0 + k).st(x);
-                m.ay.at(c0 + k).st(y);
-            }
-            c0 += 4 << d;
+        for (int k = tid; k < nc; k += nt) {  // cell (i, j) is node (i, j) of rows of 2^p + 1
+            const int p = plo + (k >> (d + 2)), cell = k & ((4 << d) - 1);
+            const int o = grid_offset32(p, d + 2 - p, S.Q) + cell + (cell >> p);
+            const T x = gx[o], y = gy[o];
+            m.ax.at(c0 + k).st(x);
+            m.ay.at(c0 + k).st(y);
         }
+        c0 += nc;
+    }
     for (int k = tid; k < w.cells; k += nt) m.b.at(k).st(T(0));  // boundary nodes read it (with zero coefficients)
-    for (int k = tid; k < w.cells + w.pads; k += nt) m.u.at(k).st(T(0));
+    for (int k = tid; k < w.ucells + w.pads; k += nt) m.u.at(k).st(T(0));
     if (m.lo > 0) {
         const T* M = op + S.op_off + op_offset(m.pic < 4 ? m.pic : 4, m.qic < 4 ? m.qic : 4, S.P, S.Q);
         for (int k = 2 * tid; k < m.n3 * m.ld3; k += 2 * nt) {
@@ -705,6 +713,39 @@ __device__ __forceinline__ void mid_fill(const MidItem<T>& m, const SampleInfo& 
         }
         for (int k = tid; k < kOpN; k += nt) m.b3.at(k).st(T(0));
         for (int k = tid; k < kU3; k += nt) m.u3.at(k).st(T(0));
+    }
+}
+
+// b of diagonal kMidD from the restrictions its parents left in the item's scratch, and u
+// back to it.
+template <class T>
+__device__ __forceinline__ void mid_take(const MidItem<T>& m, int64_t scr, int pi, int qi, const T* sbx, const T* sby)
+{
+    const MidDiag<T> g = mid_diag(m, kMidD);
+    const T *bx = sbx + scr, *by = sby + scr;
+#pragma unroll 2
+    for (int k = threadIdx.x; k < g.ng << (kMidD + 2); k += blockDim.x) {
+        const int p = g.plo + (k >> (kMidD + 2)), q = kMidD + 2 - p, cell = k & ((4 << kMidD) - 1);
+        const int o = grid_offset32(p, q, qi) + cell + (cell >> p);
+        const bool hx = p < pi, hy = q < qi;
+        const T v = (hx && hy) ? T(0.5) * bx[o] + T(0.5) * by[o] : (hx ? bx[o] : by[o]);
+        if (cell >> p && cell & ((1 << p) - 1)) g.b.at(k).st(v);
+    }
+}
+template <class T>
+__device__ __forceinline__ void mid_give(const MidItem<T>& m, int64_t scr, int qi, T* su)
+{
+    const MidDiag<T> g = mid_diag(m, kMidD);
+    T* dst = su + scr;
+    for (int k = threadIdx.x; k < g.ng << (kMidD + 2); k += blockDim.x) {  // column 0 and row 0 are zeros of the layout
+        const int p = g.plo + (k >> (kMidD + 2)), q = kMidD + 2 - p, cell = k & ((4 << kMidD) - 1);
+        const int o = grid_offset32(p, q, qi) + cell + (cell >> p);
+        dst[o] = g.u.at(k).ld();
+        if ((cell & ((1 << p) - 1)) == (1 << p) - 1) dst[o + 1] = T(0);  // the other two sides
+        if (cell >> p == (1 << q) - 1) {
+            dst[o + (1 << p) + 1] = T(0);
+            if ((cell & ((1 << p) - 1)) == (1 << p) - 1) dst[o + (1 << p) + 2] = T(0);
+        }
     }
 }
 
@@ -718,36 +759,38 @@ __global__ void __launch_bounds__(kMidThreads, sizeof(T) == 4 ? 3 : 1)
     const SampleInfo& S = cx.samples[t.s];
     const int pi = t.seg->pi, qi = t.seg->qi;
     __shared__ int2 at[kMidMax + 1];
-    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, min(pi, kMidD + 1), min(qi, kMidD + 1), kOpD + 1, kMidD, cp.nu1);
+    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, min(pi, kMidD + 1), min(qi, kMidD + 1), kOpD + 1, kOpD + 1, kMidD, cp.nu1);
     mid_fill(m, S, ax, ay, op);
     __syncthreads();
-    const MidDiag<T> g = mid_diag(m, kMidD);
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int p = g.plo; p < g.plo + g.ng; ++p) {
-        const int q = kMidD + 2 - p;
-        const int64_t so = t.scr + grid_offset(p, q, qi);
-        const bool hx = p < pi, hy = q < qi;
-        for (int k = tid; k < 4 << kMidD; k += nt) {
-            const int64_t o = so + k + (k >> p);
-            const T v = (hx && hy) ? T(0.5) * sbx[o] + T(0.5) * sby[o] : (hx ? sbx[o] : sby[o]);
-            if (k >> p && k & ((1 << p) - 1)) g.b.at(((p - g.plo) << (kMidD + 2)) + k).st(v);
-        }
-    }
+    mid_take(m, t.scr, pi, qi, sbx, sby);
     __syncthreads();
     for (int call = 0; call < cp.mu; ++call) mid_cycle(m, cp.mu, cp.nu1, cp.nu2, (T)cp.omega, call == 0);
-    for (int p = g.plo; p < g.plo + g.ng; ++p) {
-        const int q = kMidD + 2 - p, nx = 1 << p;
-        T* dst = su + t.scr + grid_offset(p, q, qi);
-        for (int k = tid; k < 4 << kMidD; k += nt)  // column 0 and row 0 are zeros of the layout
-            dst[k + (k >> p)] = g.u.at(((p - g.plo) << (kMidD + 2)) + k).ld();
-        for (int k = tid; k <= 1 << q; k += nt) dst[k * (nx + 1) + nx] = T(0);
-        for (int k = tid; k <= nx; k += nt) dst[(nx + 1) * (1 << q) + k] = T(0);
+    mid_give(m, t.scr, qi, su);
+}
+
+// The decision of k_residual: does the item take another cycle?  first: its relative
+// residual before the first one (set at step 0).
+__device__ __forceinline__ int item_goes_on(int step, double rr, double& first, int max_cycles, double eps, int* status)
+{
+    if (step == 0) {
+        first = rr;
+        return 1;
     }
+    if (!(rr == rr) || isinf(rr)) {
+        atomicOr(status, MSG_SAMPLE_NONFINITE);
+        return 0;
+    }
+    if (rr <= eps) return 0;
+    if (step >= max_cycles || (rr > 1.0 && rr > first)) {
+        atomicOr(status, MSG_SAMPLE_NOT_CONVERGED);
+        return 0;
+    }
+    return 1;
 }
 
 // An item of a low stage, solved whole: Algorithm 2's initial guess, then
 // defect-correction cycles until the residual meets eps (or the item stops), the
-// decision of k_residual word for word.
+// decision of k_residual.
 template <class T>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, int L, double* u64, const double* ax64, const double* ay64,
                                                           const T* ax, const T* ay, const T* op, CycleParams cp, int max_cycles,
@@ -763,7 +806,8 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, 
     const double* fx = ax64 + off;
     const double* fy = ay64 + off;
     __shared__ int2 at[kMidMax + 1];
-    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, p, q, L > kOpD ? kOpD + 1 : 0, L, cp.nu1);
+    const int lo = L > kOpD ? kOpD + 1 : 0;
+    const MidItem<T> m = mid_item<T>((T*)smem_raw, at, p, q, lo, lo, L, cp.nu1);
     mid_fill(m, S, ax, ay, op);
     item_guess(S, p, q, u64, ax64, ay64);
     __syncthreads();
@@ -786,14 +830,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 512 : 256) k_item(DevCtx cx, 
         const double ss = block_sum(acc);
         if (threadIdx.x == 0) {
             const double rr = sqrt(ss / (double)n);
-            int act = 1;
-            if (step == 0) first = rr;
-            else if (!(rr == rr) || isinf(rr)) { act = 0; atomicOr(&status[t.s], MSG_SAMPLE_NONFINITE); }
-            else if (rr <= eps) act = 0;
-            else if (step >= max_cycles || (rr > 1.0 && rr > first)) {
-                act = 0;
-                atomicOr(&status[t.s], MSG_SAMPLE_NOT_CONVERGED);
-            }
+            const int act = item_goes_on(step, rr, first, max_cycles, eps, &status[t.s]);
             s_act = act;
             if (!act) {
                 cycles[t.item] = step;
@@ -820,7 +857,8 @@ __global__ void __launch_bounds__(256) k_history_chip(DevCtx cx, int L, const do
     const TaskRef t = resolve(cx);
     const SampleInfo& S = cx.samples[t.s];
     const int p = t.seg->pi, q = t.seg->qi, nx = 1 << p, ny = 1 << q;
-    const MidItem<double> m = mid_item<double>((double*)smem_raw, at, p, q, L > kOpD ? kOpD + 1 : 0, L, cp.nu1);
+    const int lo = L > kOpD ? kOpD + 1 : 0;
+    const MidItem<double> m = mid_item<double>((double*)smem_raw, at, p, q, lo, lo, L, cp.nu1);
     mid_fill(m, S, ax, ay, op);
     __syncthreads();
     const MidDiag<double> g = mid_diag(m, L);

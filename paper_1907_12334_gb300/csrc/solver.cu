@@ -1588,6 +1588,7 @@ __global__ void k_qoi(DevCtx cx, const double* u64, const double* Z, int qoi, do
 }  // namespace msg
 
 #include "mid.cuh"
+#include "kept.cuh"
 #include "visit.cuh"
 
 namespace msg {
@@ -2099,11 +2100,23 @@ template <class T>
 size_t item_smem(int L, int nu1)
 {
     int most = 0;
-    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, L, nu1));
+    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, 0, L, nu1));
     return sizeof(T) * most;
 }
 template <class T>
-size_t mid_smem(int nu1) { return sizeof(T) * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kMidD, nu1); }
+size_t mid_smem(int nu1) { return sizeof(T) * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kOpD + 1, kMidD, nu1); }
+
+// The kept forms of both: FP32 cycles with sweeps on both sides.
+template <class T>
+bool kept(const msg_params& prm) { return sizeof(T) == 4 && prm.nu1 > 0 && prm.nu2 > 0; }
+size_t kept_item_smem(int L, int nu1)
+{
+    int most = 0;
+    for (int p = 1; p <= L + 1; ++p)
+        most = std::max(most, L > kOpD ? kept_total(p, L + 2 - p, kOpD + 1, kKeepItem, L, nu1) : kept_total(p, L + 2 - p, 0, kKeepLow, L, nu1));
+    return sizeof(float) * most;
+}
+size_t kept_mid_smem(int nu1) { return sizeof(float) * kept_total(kMidD + 1, kMidD + 1, kOpD + 1, kKeepMid, kMidD, nu1); }
 
 struct WsLayout {
     size_t op;  // low-diagonal matrices (mid.cuh)
@@ -2305,6 +2318,13 @@ static int visit_attributes()
     MSG_CUDA_TRY(set(k_visit<T, kVisitPairs, false>));
     MSG_CUDA_TRY(set(k_visit<T, kVisitPairs, true>));
     return MSG_OK;
+}
+
+// Threads per CTA of k_item_kept: a thread per pair of every kept diagonal of the stage's
+// items, and half as many as pairs on diagonals 7 to 9.
+static int kept_item_threads(int L)
+{
+    return L <= 2 ? 32 : L <= 5 ? 64 : L == 6 ? 128 : L == 7 ? 256 : 512;
 }
 
 // Threads per CTA of k_item: a thread holds at most four pairs of a diagonal.
@@ -2678,8 +2698,14 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
         auto launch_low = [&](int d, int calls) {
             if (chip) {
                 prof_begin(K_LOW, st);
-                k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem<T>(C.prm.nu1), st>>>(
-                    ic, su, sbx, sby, C.ax, C.ay, (const T*)(C.ws + wl.op), C.cp);
+                const T* op = (const T*)(C.ws + wl.op);
+                bool done = false;
+                if constexpr (sizeof(T) == 4)
+                    if ((done = kept<T>(C.prm)))
+                        k_mid_kept<T><<<(unsigned)nitems, kKeptThreads, kept_mid_smem(C.prm.nu1), st>>>(ic, su, sbx, sby, C.ax, C.ay,
+                                                                                                      op, C.cp);
+                if (!done)
+                    k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem<T>(C.prm.nu1), st>>>(ic, su, sbx, sby, C.ax, C.ay, op, C.cp);
                 prof_end(K_LOW, st, low_bytes, 0.0, d);
                 launch_err |= cudaGetLastError() != cudaSuccess;
                 return;
@@ -2780,8 +2806,18 @@ static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
         c.segs = (const Segment*)(C.ws + C.wl.segs[L]);
         c.nseg = (int)segs.size();
         prof_begin(K_LOW, st);
-        k_item<T><<<(unsigned)b, item_threads<T>(L), item_smem<T>(L, C.prm.nu1), st>>>(
-            c, L, C.u64, C.ax64, C.ay64, C.ax, C.ay, op, C.cp, C.prm.max_cycles, C.prm.eps, C.cyc, C.rel, C.stat);
+        auto go = [&](auto kernel, int threads, size_t smem) {
+            kernel<<<(unsigned)b, threads, smem, st>>>(c, L, C.u64, C.ax64, C.ay64, C.ax, C.ay, op, C.cp, C.prm.max_cycles,
+                                                       C.prm.eps, C.cyc, C.rel, C.stat);
+        };
+        bool done = false;
+        if constexpr (sizeof(T) == 4)
+            if ((done = kept<T>(C.prm))) {
+                const size_t sm = kept_item_smem(L, C.prm.nu1);
+                if (L < kOpD + 1 + kKeepItem) go(k_item_kept<T, true>, kept_item_threads(L), sm);
+                else go(k_item_kept<T, false>, kept_item_threads(L), sm);
+            }
+        if (!done) go(k_item<T>, item_threads<T>(L), item_smem<T>(L, C.prm.nu1));
         prof_end(K_LOW, st, work * 40.0, 0.0, L);
         MSG_CHECK_LAUNCH();
         MSG_CUDA_TRY(cudaStreamSynchronize(st));
@@ -2807,6 +2843,12 @@ static int cycle_attributes()
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     int rc = visit_attributes<T>();
     if (rc != MSG_OK) return rc;
+    if constexpr (sizeof(T) == 4) {
+        const int most = (int)kSmemMax - 1024;
+        MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid_kept<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        MSG_CUDA_TRY(cudaFuncSetAttribute(k_item_kept<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+        MSG_CUDA_TRY(cudaFuncSetAttribute(k_item_kept<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    }
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
     MSG_CUDA_TRY(cudaFuncSetAttribute(k_item<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
     return MSG_OK;
@@ -3199,7 +3241,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
                           *prm, op, st);
     if (rc != MSG_OK) return rc;
     if (L <= kItemL64) {
-        const size_t sm = sizeof(double) * mid_total(P, Q, L > kOpD ? kOpD + 1 : 0, L, prm->nu1);
+        const size_t sm = sizeof(double) * mid_total(P, Q, L > kOpD ? kOpD + 1 : 0, 0, L, prm->nu1);
         MSG_CUDA_TRY(cudaFuncSetAttribute(k_history_chip, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
         prof_begin(K_LOW, st);
         k_history_chip<<<(unsigned)S, item_threads<double>(L), sm, st>>>(ch, L, ax, ay, op, cp, ncycles, hist);

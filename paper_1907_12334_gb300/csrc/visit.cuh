@@ -91,8 +91,9 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
             uB = gu[o + 1];
         }
         // b and u at boundary nodes are whatever the scratch held: not used
+        T iR, iK;
         pair_set(P[k], U.at(cA).a, nx, ok, hasA, redB, aw, am, ae, sA, sB, nA, nB, hasA ? bA : T(0), ok ? bB : T(0),
-                 hasA ? uA : T(0), ok ? uB : T(0));
+                 hasA ? uA : T(0), ok ? uB : T(0), iR, iK);
     }
     if (!pre) {  // Eq. (2.4) at the black nodes (the first red half sweep overwrites the red ones)
         const T* ucx = su + scr + sg->cxo + j0 * (hx2 + 1);
