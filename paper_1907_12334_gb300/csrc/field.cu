@@ -65,9 +65,10 @@ __global__ void k_kl_a32(const double* __restrict__ sl, const double* __restrict
 // CTAs that read one tile of Phi run together and find it in L2.  513 x 513 points, 400
 // terms, 512 samples: 5.25 ms with the 64 x 64
 // tiles of k_kl_simt, 2.35 ms here (46 TFLOP/s).
-template <int TR, class TZ>
-__global__ void __launch_bounds__(256, 2) k_kl_f32(const float* __restrict__ Phi, const float* __restrict__ A, int64_t npts,
-                                                   int M, int Mp, int64_t S, int64_t stiles, int vec, TZ* __restrict__ Z)
+template <int TR, bool DIRECT, class TZ>
+__global__ void __launch_bounds__(256, 2) k_kl_f32(const float* __restrict__ Phi, const float* __restrict__ A,
+                                                   const double* __restrict__ sl, const double* __restrict__ xi,
+                                                   int64_t npts, int M, int Mp, int64_t S, int64_t stiles, int vec, TZ* __restrict__ Z)
 {
     constexpr int TS = 16 * TR, TX = 128, BK = 16, LA = TS + 4, LB = TX + 4;
     __shared__ __align__(16) float sA[2][BK * LA], sB[2][BK * LB];
@@ -79,18 +80,31 @@ __global__ void __launch_bounds__(256, 2) k_kl_f32(const float* __restrict__ Phi
     // vec: every row of Phi starts on 16 bytes
     float4 ra[NA], rb[NB];
     // this thread's rows relative to the tiles, at its first terms
-    const float *tA = A + s0 * Mp, *tB = Phi + x0 * M;
+    const float *tA = DIRECT ? nullptr : A + s0 * Mp, *tB = Phi + x0 * M;
+    const double* tX = DIRECT ? xi + s0 * M : nullptr;
     int oa[NA], ob[NB];
 #pragma unroll
-    for (int i = 0; i < NA; ++i) oa[i] = (int)min((int64_t)(row + 64 * i), S - 1 - s0) * Mp + kq;
+    for (int i = 0; i < NA; ++i) oa[i] = (int)min((int64_t)(row + 64 * i), S - 1 - s0) * (DIRECT ? M : Mp) + kq;
 #pragma unroll
     for (int i = 0; i < NB; ++i) ob[i] = (int)min((int64_t)(row + 64 * i), npts - 1 - x0) * M + kq;
     const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
     auto fetch = [&](int k0) {
         const int k = k0 + kq;
 #pragma unroll
-        for (int i = 0; i < NA; ++i)
-            ra[i] = (k < Mp && row + 64 * i < TS) ? *reinterpret_cast<const float4*>(tA + oa[i] + k0) : none;
+        for (int i = 0; i < NA; ++i) {
+            if constexpr (DIRECT) {  // A's elements formed here
+                ra[i] = none;
+                if (row + 64 * i < TS) {
+                    const double* x = tX + oa[i] + k0;
+                    if (k < M) ra[i].x = (float)(sl[k] * x[0]);
+                    if (k + 1 < M) ra[i].y = (float)(sl[k + 1] * x[1]);
+                    if (k + 2 < M) ra[i].z = (float)(sl[k + 2] * x[2]);
+                    if (k + 3 < M) ra[i].w = (float)(sl[k + 3] * x[3]);
+                }
+            } else {
+                ra[i] = (k < Mp && row + 64 * i < TS) ? *reinterpret_cast<const float4*>(tA + oa[i] + k0) : none;
+            }
+        }
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const float* p = tB + ob[i] + k0;
@@ -276,6 +290,18 @@ void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts,
 {
     const int Mp = (M + 3) & ~3, TR = S <= 32 ? 2 : S <= 64 ? 4 : 8;
     const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = stiles * ((npts + 127) / 128);
+    const unsigned g = (unsigned)tiles;
+    const int vec = M == (M & ~3) && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
+    // Few tiles with few coefficients each: forming them in the tile costs the FP64 pipe less
+    // (16 TR M / 2 clocks a tile and SM) than a launch and a temporary cost the call: 9 x 9
+    // points, 20 terms, 8 samples 10.8 -> 8.2 us, 250 x 200, 60, 20 16.4 us (the sums are the
+    // same bits).  The line is at 15000 clocks, 7 us; 200 x 100, 300, 60 lies above it with 47 us.
+    if (16LL * TR * M * ((tiles + 151) / 152) <= 15000) {
+        if (TR == 2) k_kl_f32<2, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+        else if (TR == 4) k_kl_f32<4, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+        else k_kl_f32<8, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+        return;
+    }
     void* A = nullptr;
     if (tiles > 0x7fffffffLL || temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) {
         const dim3 grid((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
@@ -283,11 +309,9 @@ void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts,
         return;
     }
     k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);
-    const unsigned g = (unsigned)tiles;
-    const int vec = M == Mp && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
-    if (TR == 2) k_kl_f32<2, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
-    else if (TR == 4) k_kl_f32<4, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
-    else k_kl_f32<8, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, npts, M, Mp, S, stiles, vec, Z);
+    if (TR == 2) k_kl_f32<2, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+    else if (TR == 4) k_kl_f32<4, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+    else k_kl_f32<8, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
     cudaFreeAsync(A, st);
 }
 }  // namespace
