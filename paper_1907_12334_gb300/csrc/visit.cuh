@@ -130,9 +130,10 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
     }
     // halo rows: zeros at the grid's boundary and in column 0; with neighbours, PRE from a
     // nonzero u takes their black nodes from memory (the only ones read before the
-    // neighbour has written its red ones)
+    // neighbour has written its red ones).  The red node in the last column of row -1 lies
+    // before column 0 of row 0, which reads it with weight zero: it must be a number.
     for (int i = threadIdx.x; i < nx; i += nt) {
-        if (!below || i == 0) U.at(i - nx).st(T(0));
+        if (!below || i == 0 || i == nx - 1) U.at(i - nx).st(T(0));
         else if (pre && !zero && ((i + j0 - 1) & 1)) U.at(i - nx).st(gu[i - W]);
         if (!above || i == 0) U.at(R * nx + i).st(T(0));
         else if (pre && !zero && ((i + j0 + R) & 1)) U.at(R * nx + i).st(gu[R * W + i]);

@@ -66,3 +66,26 @@ def test_history_beyond_one_cta_matches_oracle(P, Q, kw):
     for k, z in enumerate((Z, -Z)):
         ho = oracle.Hierarchy(P, Q, Z=z, prm=op).cycle_history(0, n)
         np.testing.assert_allclose(h[k].cpu().numpy(), ho, rtol=1e-8, atol=4 * floor)
+
+
+@pytest.mark.parametrize("P,Q,S,precision", [(8, 8, 160, "MIXED"), (6, 9, 40, "MIXED"), (7, 6, 40, "FP64"), (5, 5, 8, "MIXED")])
+def test_workspace_contents_do_not_matter(P, Q, S, precision):
+    """A workspace full of NaN gives the bits that one full of zeros gives (nothing is read
+    before it is written, also with weight zero)."""
+    from paper_1907_12334_gb300 import build, msg
+
+    build.build()
+    pq = np.array([(P, Q)] * S, dtype=np.int32)
+    z = torch.from_numpy(inputs.smooth_field(P, Q, 1.5)).to(DEV)
+    Z = (z[None] * torch.linspace(-1, 1, S, dtype=torch.float64, device=DEV)[:, None]).reshape(-1).contiguous()
+    prm = msg.SolverParams(eps=1e-9, max_cycles=60, precision=getattr(msg, f"MSG_PREC_{precision}"))
+    n, _ = msg.packed_sizes(pq)
+    out = []
+    for fill in (0, 255, 255):
+        ws = torch.full((msg.msg_workspace_bytes(pq, prm),), fill, dtype=torch.uint8, device=DEV)
+        Q_, st = torch.empty(n, dtype=torch.float64, device=DEV), torch.empty(S, dtype=torch.int32, device=DEV)
+        msg.msg_solve_batch(pq, prm, Z, Q_, st, workspace=ws)
+        out.append((Q_.cpu(), st.cpu()))
+    assert int(out[0][1].abs().max()) == 0
+    for q, st in out[1:]:
+        assert torch.equal(q, out[0][0]) and torch.equal(st, out[0][1])
