@@ -374,6 +374,7 @@ template <class T>
 __global__ void __launch_bounds__(kKeptThreads, 2)
     k_mid_kept(DevCtx cx, T* su, const T* sbx, const T* sby, const T* ax, const T* ay, const T* op, CycleParams cp)
 {
+    launch_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int2 at[kMidMax + 1];
     const TaskRef t = resolve(cx);
@@ -385,6 +386,7 @@ __global__ void __launch_bounds__(kKeptThreads, 2)
     mid_fill(m, S, ax, ay, op);
     for (int x = 0; x < kKeepMid; ++x) kept_load(m, tb, kOpD + 1 + x, S, ax, ay);
     kept_op(m, tb);
+    wait_previous();
     __syncthreads();
     mid_take(m, t.scr, pi, qi, sbx, sby);
     __syncthreads();

@@ -224,6 +224,15 @@ struct Sm {
     }
 };
 
+// The launches of a cycle are a chain of short dependent kernels.  Each lets the next one
+// start at once and waits for the one before it only when it has read what does not
+// change during a solve (lists, coefficients, matrices): what follows launch_next in a
+// kernel up to wait_previous runs under its predecessor.  A kernel that waits waits for the
+// end of the whole previous kernel, hence of all before it.  Measured with FP32 cycles:
+// 180 samples of 4 to 128 cells a side 32.0 -> 26.4 ms, 192 of 256 x 256 327 -> 308 ms.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One item's hierarchy (pic, qic: its top grid clipped to the diagonals held)
 // on chip: diagonals lo..hi; below lo (when lo = kOpD + 1) the matrix.
 template <class T>

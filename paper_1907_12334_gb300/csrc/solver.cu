@@ -2259,6 +2259,31 @@ static bool visit_takes(int d, int q)
     return d >= 5 && visit_cluster<T>(d) <= kVisitClusterMax && (int64_t(1) << q) >= 2 * visit_cluster<T>(d);
 }
 
+// Launch attribute of a kernel that calls wait_previous (mid.cuh) before it touches what the
+// kernel before it on the stream reads or writes.  FP32 cycles only: in FP64, where a CTA fills
+// its SM and its arithmetic is what bounds it, the early start costs more than it hides
+// (12 cycles of 32 samples of 64 x 64: 27.4 ms, chained 28.8 ms).
+static cudaLaunchAttribute chained()
+{
+    cudaLaunchAttribute a{};
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+template <class K, class... A>
+static cudaError_t launch_chained(K k, unsigned grid, int threads, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at = chained();
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // One visit half of diagonal d for the segments segs[0 .. c.nseg) (host copy).
 // Launch shape: see the rule below; `block` (threads per CTA) overrides it.
 template <class T>
@@ -2290,12 +2315,18 @@ static cudaError_t launch_visit(const DevCtx& c, const Segment* segs, int d, T* 
     cfg.blockDim = dim3(nt);
     cfg.dynamicSmemBytes = sizeof(T) * words;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    int na = 0;
+    // the first launch of a cycle comes after the copies of its lists: not chained
+    if (sizeof(T) == 4 && !(pre && segs[0].p == segs[0].pi && segs[0].q == segs[0].qi)) at[na++] = chained();
+    if (C > 1) {
+        at[na].id = cudaLaunchAttributeClusterDimension;
+        at[na].val.clusterDim.x = C;
+        at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+        ++na;
+    }
     cfg.attrs = at;
-    cfg.numAttrs = C > 1 ? 1 : 0;
+    cfg.numAttrs = na;
     auto go = [&](auto k) {
         return cudaLaunchKernelEx(&cfg, k, c, su, sbx, sby, ax, ay, pre, zero, nu, omega, C);
     };
@@ -2702,8 +2733,8 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
                 bool done = false;
                 if constexpr (sizeof(T) == 4)
                     if ((done = kept<T>(C.prm)))
-                        k_mid_kept<T><<<(unsigned)nitems, kKeptThreads, kept_mid_smem(C.prm.nu1), st>>>(ic, su, sbx, sby, C.ax, C.ay,
-                                                                                                      op, C.cp);
+                        launch_err |= launch_chained(k_mid_kept<T>, (unsigned)nitems, kKeptThreads, kept_mid_smem(C.prm.nu1), st, ic,
+                                                     su, (const T*)sbx, (const T*)sby, C.ax, C.ay, op, C.cp) != cudaSuccess;
                 if (!done)
                     k_mid<T><<<(unsigned)nitems, kMidThreads, mid_smem<T>(C.prm.nu1), st>>>(ic, su, sbx, sby, C.ax, C.ay, op, C.cp);
                 prof_end(K_LOW, st, low_bytes, 0.0, d);

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Segment* sg = &cx.segs[blockIdx.y];
     const int at = CL ? blockIdx.x / C : blockIdx.x, rank = CL ? blockIdx.x - at * C : 0;
+    launch_next();
     if ((int64_t)at >= sg->count) return;  // the whole cluster
     if (CL) cluster_arrive();              // a peer's shared memory is written once all have started
     const int smp = cx.slist[sg->list_off + at];
@@ -70,13 +71,21 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
     const int nt = blockDim.x;  // NP nt = R nx / 2 pairs
     const bool below = CL && rank > 0, above = CL && rank < C - 1;
     Pair<T> P[NP];
+    T aw[NP], am[NP], ae[NP], sA[NP], sB[NP], nA[NP], nB[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const int cA = 2 * (threadIdx.x + k * nt), i = cA & (nx - 1), lj = cA >> p;
+        const bool ok = j0 + lj > 0;
+        const int o = lj * W + i, w = ok && i > 0 ? o - 1 : o, s = ok ? o - W : o;
+        aw[k] = fx[w]; am[k] = fx[o]; ae[k] = fx[o + 1];
+        nA[k] = fy[o]; nB[k] = fy[o + 1]; sA[k] = fy[s]; sB[k] = fy[s + 1];
+    }
+    wait_previous();
 #pragma unroll
     for (int k = 0; k < NP; ++k) {
         const int cA = 2 * (threadIdx.x + k * nt), i = cA & (nx - 1), lj = cA >> p, j = j0 + lj;
         const bool ok = j > 0, hasA = ok && i > 0, redB = j & 1;
-        const int o = lj * W + i, w = hasA ? o - 1 : o, s = ok ? o - W : o;
-        const T aw = fx[w], am = fx[o], ae = fx[o + 1];
-        const T nA = fy[o], nB = fy[o + 1], sA = fy[s], sB = fy[s + 1];
+        const int o = lj * W + i;
         T bA, bB, uA = T(0), uB = T(0);
         if (hx && hy) {
             bA = T(0.5) * bx[o] + T(0.5) * by[o];
@@ -92,8 +101,8 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
         }
         // b and u at boundary nodes are whatever the scratch held: not used
         T iR, iK;
-        pair_set(P[k], U.at(cA).a, nx, ok, hasA, redB, aw, am, ae, sA, sB, nA, nB, hasA ? bA : T(0), ok ? bB : T(0),
-                 hasA ? uA : T(0), ok ? uB : T(0), iR, iK);
+        pair_set(P[k], U.at(cA).a, nx, ok, hasA, redB, aw[k], am[k], ae[k], sA[k], sB[k], nA[k], nB[k], hasA ? bA : T(0),
+                 ok ? bB : T(0), hasA ? uA : T(0), ok ? uB : T(0), iR, iK);
     }
     if (!pre) {  // Eq. (2.4) at the black nodes (the first red half sweep overwrites the red ones)
         const T* ucx = su + scr + sg->cxo + j0 * (hx2 + 1);
