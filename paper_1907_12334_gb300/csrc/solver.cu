@@ -2789,27 +2789,24 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
     return finish(MSG_OK);
 }
 
-// The matrices of every sample, one launch per class that some group has.
+// The matrices of every sample, one launch for all classes.
 template <class T>
 static int matrices(const OpTables& ot, const std::vector<Group>& groups, const SampleInfo* samples, int S, const T* img,
                     const LowDesc* desc, const uint4* ent, const uint2* prog, const msg_params& prm, T* op, cudaStream_t st)
 {
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     const LowPlanes& lp = low_tables().planes[kOpD];
-    for (int c = 0; c < kOpClasses; ++c) {
-        const int pic = op_pic(c), qic = op_qic(c), n = op_n(pic, qic);
-        bool any = false;
-        for (const Group& g : groups) any |= op_has(pic, qic, g.P, g.Q);
-        if (!any) continue;
-        const dim3 blk((n + 31) / 32 * 32, 768 / ((n + 31) / 32 * 32));
-        const size_t smem = sizeof(uint4) * ot.ecap + sizeof(uint2) * ot.pcap +
-                            sizeof(T) * (lp.nfx + lp.nfy + (size_t)(2 * lp.nu + lp.nr) * n);
-        prof_begin(K_COEFFS, st);
-        k_lowop<T><<<(unsigned)S, blk, smem, st>>>(samples, pic, qic, img, lp.nfx + lp.nfy, lp.nfx, desc + c, ent, prog, lp,
-                                                  prm.mu, (T)prm.omega, op);
-        prof_end(K_COEFFS, st, 0.0, 0.0);
-        MSG_CHECK_LAUNCH();
-    }
+    size_t smem = 0;
+    for (int c = 0; c < kOpClasses; ++c)
+        for (const Group& g : groups)
+            if (op_has(op_pic(c), op_qic(c), g.P, g.Q))
+                smem = std::max(smem, op_smem<T>(ot.ecap, ot.pcap, lp, op_n(op_pic(c), op_qic(c))));
+    if (smem == 0) return MSG_OK;
+    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowop<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    prof_begin(K_COEFFS, st);
+    k_lowop<T><<<dim3((unsigned)S, kOpClasses), kOpThreads, smem, st>>>(samples, img, lp.nfx + lp.nfy, lp.nfx, desc, ent, prog, lp,
+                                                                       prm.mu, (T)prm.omega, op);
+    prof_end(K_COEFFS, st, 0.0, 0.0);
+    MSG_CHECK_LAUNCH();
     return MSG_OK;
 }
 
