@@ -1328,6 +1328,26 @@ __global__ void __launch_bounds__(32 * kLowWarpsMax) k_lowv(DevCtx cx, const Low
     }
 }
 
+// Finest edges whose exp(-Z) coarser grids use: x-edges [2^Q + 1][2^P], then y-edges
+// [2^Q][2^P + 1]; none along a direction with one level.  They fit the sample's rectangle.
+__host__ __device__ __forceinline__ int edges_x(int P, int Q) { return P > 1 ? ((1 << Q) + 1) << P : 0; }
+__host__ __device__ __forceinline__ int edges_y(int P, int Q) { return Q > 1 ? ((1 << P) + 1) << Q : 0; }
+
+// exp(-Z) at the finest edges of sample blockIdx.x, once for all of its grids: each grid
+// forming its own took about P Q / 2 times as many exponentials, and those bound it (the FP64
+// pipe): 192 samples of 256 x 256 15.7 -> 4.9 ms, with k_coeffs' slices of a large grid.
+__global__ void k_edges(const SampleInfo* samples, const double* Z, double* E)
+{
+    const SampleInfo S = samples[blockIdx.x];
+    const int NFx = (2 << S.P) + 1, w = (1 << S.P) + 1, mx = (1 << S.P) - 1, nX = edges_x(S.P, S.Q), n = nX + edges_y(S.P, S.Q);
+    const double* Zs = Z + S.field_off;
+    double* e = E + S.node_off;
+    for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < n; k += gridDim.y * blockDim.x) {
+        const int y = k - nX, j = y < 0 ? k >> S.P : y / w, i = y < 0 ? k & mx : y - j * w;
+        e[k] = exp(-Zs[(int64_t)(y < 0 ? 2 * j : 2 * j + 1) * NFx + (y < 0 ? 2 * i + 1 : 2 * i)]);
+    }
+}
+
 // Coefficients on every grid (Sec. 2, direct discretisation on each grid).
 // The finest grid takes a = exp(Z) at its face midpoints (field node
 // (2i+1, 2j) for the x-face (i+1/2, j), (2i, 2j+1) for the y-face).  A coarser
@@ -1335,7 +1355,10 @@ __global__ void __launch_bounds__(32 * kLowWarpsMax) k_lowv(DevCtx cx, const Low
 // the series (harmonic) mean of their values along the flux direction,
 // a = sx / sum_k exp(-Z_k); coef == 1 injects exp(Z) at the coarse face
 // midpoint.  Stored scaled by 1/dx^2 and 1/dy^2 (exact: powers of two).
-__global__ void k_coeffs(DevCtx cx, const double* Z, int coef, double* ax64, double* ay64, float* ax32, float* ay32)
+// E (k_edges' table, or null): exp(-Z) at the finest edges, which the harmonic means of all
+// coarser grids share.  blockIdx.y: slice of the grid, of 4096 nodes or 1/16 of the largest
+// (one CTA a grid left 4 samples of 256 x 256 on 4 CTAs at the end: 857 -> 274 us).
+__global__ void k_coeffs(DevCtx cx, const double* Z, int coef, const double* E, double* ax64, double* ay64, float* ax32, float* ay32)
 {
     TaskRef t = resolve(cx);
     const SampleInfo& S = cx.samples[t.s];
@@ -1343,9 +1366,10 @@ __global__ void k_coeffs(DevCtx cx, const double* Z, int coef, double* ax64, dou
     const int NFx = (1 << (S.P + 1)) + 1, sx = 1 << (S.P - p), sy = 1 << (S.Q - q);
     const double idx2 = (double)nx * nx, idy2 = (double)ny * ny;
     const double* Zs = Z + S.field_off;
+    const double *Ex = E ? E + S.node_off : nullptr, *Ey = E ? Ex + edges_x(S.P, S.Q) : nullptr;
     const int64_t off = S.node_off + grid_offset(p, q, S.Q);
     const int n = (nx + 1) * (ny + 1);
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < n; k += gridDim.y * blockDim.x) {
         int i = k % W, j = k / W;
         double vx = 0.0, vy = 0.0;
         if (i < nx) {
@@ -1354,8 +1378,14 @@ __global__ void k_coeffs(DevCtx cx, const double* Z, int coef, double* ax64, dou
                 vx = exp(Zs[row + (2 * i + 1) * sx]);
             } else {
                 double s = 0.0;
-                for (int m = 0; m < sx; ++m) s += exp(-Zs[row + 2 * (i * sx + m) + 1]);
-                vx = sx / s;
+                if (E) {
+                    const double* e = Ex + (j * sy << S.P) + i * sx;
+#pragma unroll 8
+                    for (int m = 0; m < sx; ++m) s += e[m];
+                } else {
+                    for (int m = 0; m < sx; ++m) s += exp(-Zs[row + 2 * (i * sx + m) + 1]);
+                }
+                vx = 1.0 / s * sx;  // (sx: a power of two)
             }
             vx *= idx2;
         }
@@ -1364,8 +1394,15 @@ __global__ void k_coeffs(DevCtx cx, const double* Z, int coef, double* ax64, dou
                 vy = exp(Zs[(int64_t)((2 * j + 1) * sy) * NFx + 2 * i * sx]);
             } else {
                 double s = 0.0;
-                for (int m = 0; m < sy; ++m) s += exp(-Zs[(int64_t)(2 * (j * sy + m) + 1) * NFx + 2 * i * sx]);
-                vy = sy / s;
+                if (E) {
+                    const int w = (1 << S.P) + 1;
+                    const double* e = Ey + j * sy * w + i * sx;
+#pragma unroll 8
+                    for (int m = 0; m < sy; ++m) s += e[m * w];
+                } else {
+                    for (int m = 0; m < sy; ++m) s += exp(-Zs[(int64_t)(2 * (j * sy + m) + 1) * NFx + 2 * i * sx]);
+                }
+                vy = 1.0 / s * sy;
             }
             vy *= idy2;
         }
@@ -2789,6 +2826,38 @@ static int stage_worker(const SolveCtx<T>& C, int L, StageQueues& Qs, cudaStream
     return finish(MSG_OK);
 }
 
+// A batch whose grids would form fewer exponentials than this on their own skips k_edges: its
+// launch costs 3 us, and the two are even near here (COEFFS of 64 samples of 16 x 16, 2.6e5:
+// 172 us without, 174 with the table; 24 of 64 x 32, 1.5e6: 215 and 197; 32 of 256 x 256,
+// 1.3e8: 2624 and 949).
+constexpr double kEdgeTable = 5e5;
+// Coefficients of every grid.  E: scratch of the samples' rectangles.
+static int coefficients(const DevCtx& c, int64_t blocks, const std::vector<SampleInfo>& samples, const double* Z, int coef,
+                        double* E, double* ax64, double* ay64, float* ax32, float* ay32, double bytes, cudaStream_t st)
+{
+    double direct = 0;
+    int most = 0, nodes = 0;
+    for (const SampleInfo& s : samples) {
+        direct += (double)s.P * s.Q * pts(s.P, s.Q);
+        most = std::max(most, edges_x(s.P, s.Q) + edges_y(s.P, s.Q));
+        nodes = std::max(nodes, ((1 << s.P) + 1) * ((1 << s.Q) + 1));
+    }
+    const bool table = coef != 1 && most > 0 && direct >= kEdgeTable;
+    if (table) {
+        const dim3 g((unsigned)samples.size(), (unsigned)std::min((most + 2047) / 2048, 64));
+        prof_begin(K_COEFFS, st);
+        k_edges<<<g, kThreads, 0, st>>>(c.samples, Z, E);
+        prof_end(K_COEFFS, st, 0.0, 0.0);
+        MSG_CHECK_LAUNCH();
+    }
+    prof_begin(K_COEFFS, st);
+    const dim3 g((unsigned)blocks, (unsigned)std::min((nodes + 4095) / 4096, 16));
+    k_coeffs<<<g, kThreads, 0, st>>>(c, Z, coef, table ? E : nullptr, ax64, ay64, ax32, ay32);
+    prof_end(K_COEFFS, st, bytes, 0.0);
+    MSG_CHECK_LAUNCH();
+    return MSG_OK;
+}
+
 // The matrices of every sample, one launch for all classes.
 template <class T>
 static int matrices(const OpTables& ot, const std::vector<Group>& groups, const SampleInfo* samples, int S, const T* img,
@@ -2911,7 +2980,6 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
     C.base.gpos = (const int*)(ws + wl.gpos);
 
     MSG_CUDA_TRY(cudaMemsetAsync(stat, 0, sizeof(int32_t) * pl.S, st));
-    MSG_CUDA_TRY(cudaMemsetAsync(C.u64, 0, sizeof(double) * pl.total_nodes, st));
     MSG_CUDA_TRY(cudaMemsetAsync(C.nstep, 0, sizeof(int) * pl.total_q, st));
     {
         DevCtx c = C.base;
@@ -2922,11 +2990,10 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
         const int64_t nb = pl.all_segs.empty() ? 0 : pl.all_segs.back().blk_start + pl.all_segs.back().count;
         double nodes = 0;
         for (const Segment& s : pl.all_segs) nodes += (double)s.count * ((1 << s.p) + 1) * ((1 << s.q) + 1);
-        prof_begin(K_COEFFS, st);
-        k_coeffs<<<(unsigned)nb, kThreads, 0, st>>>(c, Z, prm.coef, (double*)(ws + wl.ax64), (double*)(ws + wl.ay64),
-                                                   ax32, ay32);
-        prof_end(K_COEFFS, st, nodes * (16.0 + 16.0 + (mixed ? 8.0 : 0.0)), 0.0);
-        MSG_CHECK_LAUNCH();
+        int rc = coefficients(c, nb, pl.samples, Z, prm.coef, C.u64, (double*)(ws + wl.ax64), (double*)(ws + wl.ay64), ax32, ay32,
+                              nodes * (16.0 + 16.0 + (mixed ? 8.0 : 0.0)), st);
+        if (rc != MSG_OK) return rc;
+        MSG_CUDA_TRY(cudaMemsetAsync(C.u64, 0, sizeof(double) * pl.total_nodes, st));
         const LowPlanes& lp = img_planes(prm);
         prof_begin(K_COEFFS, st);
         k_lowimg<T><<<(unsigned)pl.S, kThreads, 0, st>>>(C.base.samples, C.ax, C.ay, lp, (T*)(ws + wl.low_img),
@@ -3230,14 +3297,12 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
     cx.nseg = P * Q;
     double* ax = (double*)(ws + w.ax);
     double* ay = (double*)(ws + w.ay);
-    prof_begin(K_COEFFS, st);
-    k_coeffs<<<(unsigned)(P * Q * S), kThreads, 0, st>>>(cx, Z, prm->coef, ax, ay, nullptr, nullptr);
-    prof_end(K_COEFFS, st, (double)S * R * 32.0, 0.0);
-    MSG_CHECK_LAUNCH();
+    double* su = (double*)(ws + w.su);
+    rc = coefficients(cx, P * Q * S, samples, Z, prm->coef, su, ax, ay, nullptr, nullptr, (double)S * R * 32.0, st);
+    if (rc != MSG_OK) return rc;
     DevCtx ch = cx;
     ch.segs = cx.segs + P * Q;
     ch.nseg = 1;
-    double* su = (double*)(ws + w.su);
     double* sbx = (double*)(ws + w.sbx);
     double* sby = (double*)(ws + w.sby);
     const CycleParams cp{prm->mu, prm->nu1, prm->nu2, prm->omega};
