@@ -36,7 +36,7 @@ constexpr int kFields = 5;
 __host__ __device__ __forceinline__ int kept_rows(int d, int pic, int qic) { return ((mid_cells(d, pic, qic) >> 1) + 31) & ~31; }
 __host__ __device__ __forceinline__ int kept_total(int pic, int qic, int lo, int keep, int hi, int nu1)
 {
-    int t = (mid_total(pic, qic, lo, lo + keep, hi, nu1) + 3) & ~3;
+    int t = (mid_total<float>(pic, qic, lo, lo + keep, hi, nu1) + 3) & ~3;
     for (int d = lo; d < lo + keep && d <= hi; ++d) t += 4 * kFields * kept_rows(d, pic, qic);
     return t + (lo > 0 ? 4 * 64 + kOpN : 0);
 }
@@ -65,7 +65,7 @@ template <class T>
 __device__ __forceinline__ KeptTables kept_tables(const MidItem<T>& m, int keep, int nu1)
 {
     KeptTables t;
-    const uint32_t base = m.M.a + (uint32_t)sizeof(T) * ((mid_total(m.pic, m.qic, m.lo, m.klo, m.hi, nu1) + 3) & ~3);
+    const uint32_t base = m.M.a + (uint32_t)sizeof(T) * ((mid_total<T>(m.pic, m.qic, m.lo, m.klo, m.hi, nu1) + 3) & ~3);
     int n = 0;
     t.on = t.last = 0;
 #pragma unroll

@@ -262,6 +262,8 @@ struct MidItem {
     Sm<T> ax;  // cells
     Sm<T> ay;
     Sm<T> r;   // residual of the diagonal being restricted: the red node of each pair (every cell when nu1 = 0)
+    Sm<T> di;  // FP64: 1 / diagonal of each cell, 0 at a boundary cell
+    Sm<T> kp;  // FP64: kappa weight of the x-child at the black node of each pair
     Sm<T> M;   // the matrix (lo = kOpD + 1)
     Sm<T> b3;  // its right-hand side, compact
     Sm<T> u3;  // its result: the cells of diagonal kOpD
@@ -294,11 +296,17 @@ __host__ __device__ __forceinline__ MidWords mid_words(int pic, int qic, int lo,
     }
     return w;
 }
+// In FP64 a reciprocal is a dozen operations of the pipe that bounds the cycles, so the
+// diagonals' and the kappa weights are made once per launch: words per pair of cells.  (FP32
+// has the MUFU pipe for them, and kept.cuh.)  With the sums of pair_red as chains: FP64 solve
+// of 64 samples of 32 x 32 8.53 -> 6.61 ms, convergence study on 64 x 64 24.8 -> 20.5 ms.
+template <class T> constexpr int mid_aux() { return sizeof(T) == 8 ? 3 : 0; }
 constexpr int kU3 = 4 * 32 + 20;  // cells of diagonal kOpD and their pad
+template <class T>
 __host__ __device__ __forceinline__ int mid_total(int pic, int qic, int lo, int klo, int hi, int nu1)
 {
     const MidWords w = mid_words(pic, qic, lo, klo, hi, nu1);
-    int t = 3 * w.cells + w.ucells + w.pads + w.r;
+    int t = 3 * w.cells + w.ucells + w.pads + w.r + mid_aux<T>() * (w.cells >> 1);
     if (lo > 0) {
         const int n = op_n(pic < 4 ? pic : 4, qic < 4 ? qic : 4);
         t += n * op_ld(n) + kOpN + kU3;
@@ -324,6 +332,8 @@ __device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic
     m.b = m.ay.at(w.cells);
     m.r = m.b.at(w.cells);
     m.u = m.r.at(w.r);
+    m.di = m.u.at(w.ucells + w.pads);
+    m.kp = m.di.at(w.cells);
     m.at = at;
     if (threadIdx.x == 0) {
         int c = 0, u = 0;
@@ -340,7 +350,7 @@ __device__ __forceinline__ MidItem<T> mid_item(T* sm, int2* at, int pic, int qic
 // arrays of one diagonal
 template <class T>
 struct MidDiag {
-    Sm<T> u, b, ax, ay;
+    Sm<T> u, b, ax, ay, di, kp;
     int plo, ng;
 };
 template <class T>
@@ -352,6 +362,10 @@ __device__ __forceinline__ MidDiag<T> mid_diag(const MidItem<T>& m, int d)
     v.b = m.b.at(o.x);
     v.ax = m.ax.at(o.x);
     v.ay = m.ay.at(o.x);
+    if constexpr (mid_aux<T>() > 0) {
+        v.di = m.di.at(o.x);
+        v.kp = m.kp.at(o.x >> 1);
+    }
     v.plo = mid_plo(d, m.qic);
     v.ng = mid_phi(d, m.pic) - v.plo + 1;
     return v;
@@ -374,6 +388,27 @@ struct Pair {
     uint32_t w;                // bytes of a row
 };
 
+// The pair from its faces and values (below) and the reciprocals iA, iB of the diagonals.
+template <class T>
+__device__ __forceinline__ void pair_scale(Pair<T>& P, uint32_t aA, int nx, bool ok, bool redB, T aw, T am, T ae, T sA, T sB,
+                                           T nA, T nB, T bA, T bB, T uA, T uB, T iA, T iB, T& iR, T& iK)
+{
+    constexpr uint32_t es = sizeof(T);
+    const T oR = redB ? ae : aw, sR = redB ? sB : sA, nR = redB ? nB : nA;
+    iR = redB ? iB : iA;
+    iK = redB ? iA : iB;
+    P.w = ok ? nx * es : 0u;
+    P.aR = aA + (ok && redB ? es : 0u);
+    P.e = ok ? (redB ? es : 0u - es) : 0u;
+    P.dR = oR + am + sR + nR;
+    P.pR = iR * am; P.pK = iK * am;
+    P.oR = iR * oR; P.oK = iK * (redB ? aw : ae);
+    P.sR = iR * sR; P.sK = iK * (redB ? sA : sB);
+    P.nR = iR * nR; P.nK = iK * (redB ? nA : nB);
+    P.bR = iR * (redB ? bB : bA); P.bK = iK * (redB ? bA : bB);
+    P.uR = redB ? uB : uA; P.uK = redB ? uA : uB;
+}
+
 // From the faces and values of nodes A (even column, u at address aA) and B: aw, am,
 // ae the faces west of A, between, east of B; s, n the south and north ones.  ok: a row
 // of nodes; hasA: A is not the west boundary; redB: B is the red node.  iR, iK: what the
@@ -382,21 +417,10 @@ template <class T>
 __device__ __forceinline__ void pair_set(Pair<T>& P, uint32_t aA, int nx, bool ok, bool hasA, bool redB, T aw, T am, T ae,
                                          T sA, T sB, T nA, T nB, T bA, T bB, T uA, T uB, T& iR, T& iK)
 {
-    constexpr uint32_t es = sizeof(T);
     const T dA = aw + am + sA + nA, dB = am + ae + sB + nB;
     const T iA = hasA ? rcp_of(dA) : T(0), iB = ok ? rcp_of(dB) : T(0);
-    iR = redB ? iB : iA;
-    iK = redB ? iA : iB;
-    P.w = ok ? nx * es : 0u;
-    P.aR = aA + (ok && redB ? es : 0u);
-    P.e = ok ? (redB ? es : 0u - es) : 0u;
+    pair_scale(P, aA, nx, ok, redB, aw, am, ae, sA, sB, nA, nB, bA, bB, uA, uB, iA, iB, iR, iK);
     P.dR = redB ? dB : dA;
-    P.pR = iR * am; P.pK = iK * am;
-    P.oR = iR * (redB ? ae : aw); P.oK = iK * (redB ? aw : ae);
-    P.sR = iR * (redB ? sB : sA); P.sK = iK * (redB ? sA : sB);
-    P.nR = iR * (redB ? nB : nA); P.nK = iK * (redB ? nA : nB);
-    P.bR = iR * (redB ? bB : bA); P.bK = iK * (redB ? bA : bB);
-    P.uR = redB ? uB : uA; P.uK = redB ? uA : uB;
 }
 
 // Pair m of diagonal d; dump: the zero word for pairs past the end.
@@ -412,15 +436,23 @@ __device__ __forceinline__ void pair_load(Pair<T>& P, const MidDiag<T>& g, int d
     const T aw = x.at(-1).ld();
     const auto ae = x.ld2(), an = y.ld2(), as = y.at(ok ? -nx : 0).ld2(), bb = g.b.at(c).ld2(), uu = g.u.at(c).ld2();
     T iR, iK;
-    pair_set(P, g.u.at(cA).a, nx, ok, hasA, redB, aw, ae.x, ae.y, as.x, as.y, an.x, an.y, bb.x, bb.y, ok ? uu.x : T(0),
-             ok ? uu.y : T(0), iR, iK);
+    if constexpr (mid_aux<T>() > 0) {
+        const auto ii = g.di.at(c).ld2();
+        pair_scale(P, g.u.at(cA).a, nx, ok, redB, aw, ae.x, ae.y, as.x, as.y, an.x, an.y, bb.x, bb.y, ok ? uu.x : T(0),
+                   ok ? uu.y : T(0), ok ? ii.x : T(0), ok ? ii.y : T(0), iR, iK);
+    } else {
+        pair_set(P, g.u.at(cA).a, nx, ok, hasA, redB, aw, ae.x, ae.y, as.x, as.y, an.x, an.y, bb.x, bb.y, ok ? uu.x : T(0),
+                 ok ? uu.y : T(0), iR, iK);
+    }
 }
 
-// b + sum a u of the red / black node
+// b + sum a u of the red / black node.  FP64: as four operations of its pipe instead of six
+// (in FP32 the sum of two pairs and the chain take the same time: 256 x 256 0.5 % apart).
 template <class T>
 __device__ __forceinline__ T pair_red(const Pair<T>& a)
 {
     const T o = Sm<T>{a.aR + a.e}.ld(), s = Sm<T>{a.aR - a.w}.ld(), n = Sm<T>{a.aR + a.w}.ld();
+    if constexpr (sizeof(T) == 8) return fma(a.pR, a.uK, fma(a.oR, o, fma(a.sR, s, fma(a.nR, n, a.bR))));
     return a.bR + ((a.pR * a.uK + a.oR * o) + (a.sR * s + a.nR * n));
 }
 template <class T>
@@ -428,6 +460,7 @@ __device__ __forceinline__ T pair_black(const Pair<T>& a)
 {
     const uint32_t k = a.aR - a.e;
     const T o = Sm<T>{k - a.e}.ld(), s = Sm<T>{k - a.w}.ld(), n = Sm<T>{k + a.w}.ld();
+    if constexpr (sizeof(T) == 8) return fma(a.pK, a.uR, fma(a.oK, o, fma(a.sK, s, fma(a.nK, n, a.bK))));
     return a.bK + ((a.pK * a.uR + a.oK * o) + (a.sK * s + a.nK * n));
 }
 
@@ -596,7 +629,7 @@ __device__ __forceinline__ void mid_post(const MidItem<T>& m, int d, int nu2, T 
         const Sm<T> cx = cu.at(((p - 1 - plo) << (d + 1)) + (j << (p - 1)) + (i >> 1));  // grid (p-1, q): row j, from column i/2
         const Sm<T> cy = cu.at(((p - plo) << (d + 1)) + ((j >> 1) << p) + i);            // grid (p, q-1): from row j/2
         // correction at node A (B = 0) or B (B = 1) from the scaled coefficients
-        auto corr = [&](int B, T h0, T h1, T v0, T v1) {
+        auto corr = [&](int B, T h0, T h1, T v0, T v1, bool black) {
             T x = T(0), y = T(0);
             if (hx) {
                 x = cx.ld();
@@ -607,15 +640,17 @@ __device__ __forceinline__ void mid_post(const MidItem<T>& m, int d, int nu2, T 
                 if (redB) y = T(0.5) * (y + cy.at(nx + B).ld());
             }
             if (!(hx && hy)) return hx ? x : y;
+            if constexpr (mid_aux<T>() > 0)
+                if (black) return y + g.kp.at(mm).ld() * (x - y);
             const T c1 = h0 + h1, c2 = v0 + v1, x2 = c1 * c1, y2 = c2 * c2, w = rcp_of(x2 + y2);
             return (x2 * w) * x + (y2 * w) * y;
         };
         if (!redB || i > 0) {
-            a.uK += omega * corr(redB ? 0 : 1, a.pK, a.oK, a.sK, a.nK);
+            a.uK += omega * corr(redB ? 0 : 1, a.pK, a.oK, a.sK, a.nK, true);
             Sm<T>{a.aR - a.e}.st(a.uK);
         }
         if (nu2 == 0 && (redB || i > 0)) {
-            a.uR += omega * corr(redB ? 1 : 0, a.pR, a.oR, a.sR, a.nR);
+            a.uR += omega * corr(redB ? 1 : 0, a.pR, a.oR, a.sR, a.nR, false);
             Sm<T>{a.aR}.st(a.uR);
         }
     }
@@ -729,6 +764,17 @@ __device__ __forceinline__ void mid_fill(const MidItem<T>& m, const SampleInfo& 
             const T x = gx[o], y = gy[o];
             m.ax.at(c0 + k).st(x);
             m.ay.at(c0 + k).st(y);
+            if constexpr (mid_aux<T>() > 0) {
+                const int i = cell & ((1 << p) - 1), j = cell >> p;
+                T inv = T(0), kx = T(0);
+                if (i > 0 && j > 0) {
+                    const T aw = gx[o - 1], as = gy[o - (1 << p) - 1], cx = aw + x, cy = as + y, x2 = cx * cx, y2 = cy * cy;
+                    inv = rcp_of(cx + cy);
+                    kx = x2 * rcp_of(x2 + y2);
+                }
+                m.di.at(c0 + k).st(inv);
+                if ((i + j) & 1) m.kp.at((c0 + k) >> 1).st(kx);
+            }
         }
         c0 += nc;
     }

@@ -2137,11 +2137,11 @@ template <class T>
 size_t item_smem(int L, int nu1)
 {
     int most = 0;
-    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, 0, L, nu1));
+    for (int p = 1; p <= L + 1; ++p) most = std::max(most, mid_total<T>(p, L + 2 - p, L > kOpD ? kOpD + 1 : 0, 0, L, nu1));
     return sizeof(T) * most;
 }
 template <class T>
-size_t mid_smem(int nu1) { return sizeof(T) * mid_total(kMidD + 1, kMidD + 1, kOpD + 1, kOpD + 1, kMidD, nu1); }
+size_t mid_smem(int nu1) { return sizeof(T) * mid_total<T>(kMidD + 1, kMidD + 1, kOpD + 1, kOpD + 1, kMidD, nu1); }
 
 // The kept forms of both: FP32 cycles with sweeps on both sides.
 template <class T>
@@ -3334,7 +3334,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
                           *prm, op, st);
     if (rc != MSG_OK) return rc;
     if (L <= kItemL64) {
-        const size_t sm = sizeof(double) * mid_total(P, Q, L > kOpD ? kOpD + 1 : 0, 0, L, prm->nu1);
+        const size_t sm = sizeof(double) * mid_total<double>(P, Q, L > kOpD ? kOpD + 1 : 0, 0, L, prm->nu1);
         MSG_CUDA_TRY(cudaFuncSetAttribute(k_history_chip, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
         prof_begin(K_LOW, st);
         k_history_chip<<<(unsigned)S, item_threads<double>(L), sm, st>>>(ch, L, ax, ay, op, cp, ncycles, hist);
