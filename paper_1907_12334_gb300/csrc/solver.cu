@@ -1871,15 +1871,22 @@ struct OpTables {
     int ecap, pcap;  // entries and program words of the largest class (words: even)
 };
 
+// The classes' entries (the same for every solve) and the phase programs of these parameters.
 static OpTables op_tables(const msg_params& prm)
 {
-    OpTables t;
-    const LowPlanes& lp = low_tables().planes[kOpD];
+    static const OpTables entries = [] {
+        OpTables t;
+        t.ecap = t.pcap = 0;
+        for (int c = 0; c < kOpClasses; ++c) {
+            low_build_class(op_pic(c), op_qic(c), kOpD, low_tables().planes[kOpD], t.desc[c], t.ent);
+            t.ecap = std::max(t.ecap, t.desc[c].e1 - t.desc[c].e0);
+        }
+        return t;
+    }();
+    OpTables t = entries;
     const std::vector<int> words = low_program(kOpD, prm, false);
-    t.ecap = t.pcap = 0;
-    for (int c = 0; c < kOpClasses; ++c) {
-        LowDesc& D = t.desc[c];
-        low_build_class(op_pic(c), op_qic(c), kOpD, lp, D, t.ent);
+    t.prog.reserve(kOpClasses * words.size());
+    for (LowDesc& D : t.desc) {
         D.prog = (int)t.prog.size();
         for (int w : words) {
             const int kind = w & 7, d = w >> 3, cnt = D.cnt[d][kind];
@@ -1887,7 +1894,6 @@ static OpTables op_tables(const msg_params& prm)
             t.prog.push_back(make_uint2((uint32_t)kind | (uint32_t)cnt << 3, (uint32_t)(D.off[d][kind] - D.e0)));
         }
         D.nops = (int)t.prog.size() - D.prog;
-        t.ecap = std::max(t.ecap, D.e1 - D.e0);
         t.pcap = std::max(t.pcap, (D.nops + 1) & ~1);
     }
     return t;
@@ -2880,13 +2886,15 @@ static int matrices(const OpTables& ot, const std::vector<Group>& groups, const 
 }
 
 // Stages 0 .. nlow-1, each one launch of k_item over the stage's items of every sample.
+// lists: the stages' segments, which the stream's copies read.
 template <class T>
-static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
+static int low_stages(const SolveCtx<T>& C, int nlow, std::vector<std::vector<Segment>>& lists, cudaStream_t st)
 {
     const Plan& pl = C.pl;
     T* op = (T*)(C.ws + C.wl.op);
     for (int L = 0; L < nlow; ++L) {
-        std::vector<Segment> segs;
+        lists.emplace_back();
+        std::vector<Segment>& segs = lists.back();
         int64_t b = 0;
         double work = 0;
         for (const ItemType& it : pl.stage_items[L]) {
@@ -2917,38 +2925,42 @@ static int low_stages(const SolveCtx<T>& C, int nlow, cudaStream_t st)
         if (!done) go(k_item<T>, item_threads<T>(L), item_smem<T>(L, C.prm.nu1));
         prof_end(K_LOW, st, work * 40.0, 0.0, L);
         MSG_CHECK_LAUNCH();
-        MSG_CUDA_TRY(cudaStreamSynchronize(st));
     }
     return MSG_OK;
 }
 
-// Shared-memory limits of the cycles' kernels (idempotent).
+// Shared-memory limits of the cycles' kernels (idempotent): chip, those of the on-chip cycles
+// (else of k_lowv); visits, those above them.
 template <class T>
-static int cycle_attributes()
+static int cycle_attributes(bool chip, bool visits)
 {
-    // the residual band: 3 rows of a 2^12-cell-wide grid at most
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_pre<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)(sizeof(T) * std::max(kBandNodes, 3 * ((1 << 12) + 1)))));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    if constexpr (sizeof(T) == 4)
-        MSG_CUDA_TRY(cudaFuncSetAttribute(k_visit_reg<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_lowv<T, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    int rc = visit_attributes<T>();
-    if (rc != MSG_OK) return rc;
-    if constexpr (sizeof(T) == 4) {
-        const int most = (int)kSmemMax - 1024;
-        MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid_kept<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        MSG_CUDA_TRY(cudaFuncSetAttribute(k_item_kept<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-        MSG_CUDA_TRY(cudaFuncSetAttribute(k_item_kept<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+    int rc = MSG_OK;
+    auto limit = [&](auto kernel, size_t bytes) {
+        if (rc == MSG_OK) rc = [&] { MSG_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)); return (int)MSG_OK; }();
+    };
+    if (chip) {
+        if constexpr (sizeof(T) == 4) {
+            limit(k_mid_kept<T>, kSmemMax - 1024);
+            limit(k_item_kept<T, true>, kSmemMax - 1024);
+            limit(k_item_kept<T, false>, kSmemMax - 1024);
+        }
+        limit(k_mid<T>, kSmemMax - 1024);
+        limit(k_item<T>, kSmemMax - 1024);
+    } else {
+        limit(k_lowv<T, 1>, kSmemMax);
+        limit(k_lowv<T, 2>, kSmemMax);
+        limit(k_lowv<T, 4>, kSmemMax);
+        limit(k_lowv<T, 8>, kSmemMax);
     }
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_mid<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
-    MSG_CUDA_TRY(cudaFuncSetAttribute(k_item<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax - 1024));
-    return MSG_OK;
+    if (visits) {
+        // the residual band: 3 rows of a 2^12-cell-wide grid at most
+        limit(k_pre<T>, sizeof(T) * std::max(kBandNodes, 3 * ((1 << 12) + 1)));
+        limit(k_visit_reg<T, 1>, kSmemMax);
+        limit(k_visit_reg<T, 2>, kSmemMax);
+        if constexpr (sizeof(T) == 4) limit(k_visit_reg<T, 4>, kSmemMax);
+        if (rc == MSG_OK) rc = visit_attributes<T>();
+    }
+    return rc;
 }
 
 template <class T>
@@ -2959,6 +2971,18 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
     std::vector<Group> gtab;  // [0]: groups, [1+L]: stage L groups
     gtab.insert(gtab.end(), pl.groups.begin(), pl.groups.end());
     for (int L = 0; L <= pl.Lmax; ++L) gtab.insert(gtab.end(), pl.stage_groups[L].begin(), pl.stage_groups[L].end());
+    // tables of the low diagonals: class descriptors, node entries, programs; lists of the low stages
+    const bool chip = on_chip(prm), ops = !chip || pl.total_op > 0;  // ops: some sample has a matrix
+    std::vector<LowDesc> desc;
+    std::vector<uint2> rp;
+    OpTables ot;
+    std::vector<std::vector<Segment>> low_lists;
+    // the copies below read host memory: an early return waits for them (before the vectors go)
+    struct Drain {
+        cudaStream_t st;
+        bool done = false;
+        ~Drain() { if (!done) cudaStreamSynchronize(st); }
+    } drain{st};
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.samples, pl.samples.data(), sizeof(SampleInfo) * pl.S, cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.perm, pl.perm.data(), sizeof(int) * pl.S, cudaMemcpyHostToDevice, st));
     MSG_CUDA_TRY(cudaMemcpyAsync(ws + wl.gpos, pl.gpos.data(), sizeof(int) * pl.S, cudaMemcpyHostToDevice, st));
@@ -2994,25 +3018,19 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
                               nodes * (16.0 + 16.0 + (mixed ? 8.0 : 0.0)), st);
         if (rc != MSG_OK) return rc;
         MSG_CUDA_TRY(cudaMemsetAsync(C.u64, 0, sizeof(double) * pl.total_nodes, st));
+    }
+    if (ops) {
         const LowPlanes& lp = img_planes(prm);
         prof_begin(K_COEFFS, st);
         k_lowimg<T><<<(unsigned)pl.S, kThreads, 0, st>>>(C.base.samples, C.ax, C.ay, lp, (T*)(ws + wl.low_img),
                                                           (int64_t)(lp.nfx + lp.nfy), lp.nfx);
         prof_end(K_COEFFS, st, (double)pl.S * (lp.nfx + lp.nfy) * 2.0 * sizeof(T), 0.0);
         MSG_CHECK_LAUNCH();
-    }
-    {
-        // tables of the low diagonals: class descriptors, node entries, programs
-        const LowTables& lt = low_tables();
-        std::vector<LowDesc> desc;
-        std::vector<uint2> rp;
-        OpTables ot;
-        if (on_chip(prm)) ot = op_tables(prm);
-        else rp = low_resolve(prm, desc);
         auto up = [&](size_t at, const void* p, size_t bytes) {
             return cudaMemcpyAsync(ws + at, p, bytes, cudaMemcpyHostToDevice, st);
         };
-        if (on_chip(prm)) {
+        if (chip) {
+            ot = op_tables(prm);
             MSG_CUDA_TRY(up(wl.low_desc, ot.desc, sizeof(ot.desc)));
             MSG_CUDA_TRY(up(wl.low_ent, ot.ent.data(), sizeof(uint4) * ot.ent.size()));
             MSG_CUDA_TRY(up(wl.low_prog, ot.prog.data(), sizeof(uint2) * ot.prog.size()));
@@ -3020,25 +3038,25 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
                                  C.low_prog, prm, (T*)(ws + wl.op), st);
             if (rc != MSG_OK) return rc;
         } else {
+            const LowTables& lt = low_tables();
+            rp = low_resolve(prm, desc);
             MSG_CUDA_TRY(up(wl.low_desc, desc.data(), sizeof(LowDesc) * desc.size()));
             MSG_CUDA_TRY(up(wl.low_ent, lt.ent.data(), sizeof(uint4) * lt.ent.size()));
             MSG_CUDA_TRY(up(wl.low_prog, rp.data(), sizeof(uint2) * rp.size()));
         }
-        // the sources are host vectors: finish the copies before they go out of scope
-        MSG_CUDA_TRY(cudaStreamSynchronize(st));
     }
+    const int nst = pl.Lmax + 1, nlow = std::min(nst, item_stages(prm) + 1);
     {
-        int rc = cycle_attributes<T>();
+        int rc = cycle_attributes<T>(chip, nlow < nst);
         if (rc != MSG_OK) return rc;
     }
-    MSG_CUDA_TRY(cudaStreamSynchronize(st));
 
     // ---- low stages on chip, one launch each (the stream orders a stage after its children's)
-    const int nst = pl.Lmax + 1, nlow = std::min(nst, item_stages(prm) + 1);
-    if (on_chip(prm)) {
-        int rc = low_stages<T>(C, nlow, st);
+    if (chip) {
+        int rc = low_stages<T>(C, nlow, low_lists, st);
         if (rc != MSG_OK) return rc;
     }
+    if (nlow < nst) MSG_CUDA_TRY(cudaStreamSynchronize(st));  // the workers' streams read what was done so far
 
     // ---- one worker (host thread + stream) per further stage
     StageQueues Qs;
@@ -3082,6 +3100,7 @@ static int run_solve(const Plan& pl, const WsLayout& wl, char* ws, const msg_par
     if (cycles_out) MSG_CUDA_TRY(cudaMemcpyAsync(cycles_out, C.cyc, sizeof(int) * pl.total_q, cudaMemcpyDeviceToDevice, st));
     if (relres_out) MSG_CUDA_TRY(cudaMemcpyAsync(relres_out, C.rel, sizeof(double) * pl.total_q, cudaMemcpyDeviceToDevice, st));
     MSG_CUDA_TRY(cudaStreamSynchronize(st));
+    drain.done = true;
     return MSG_OK;
 }
 
@@ -3341,7 +3360,7 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
         prof_end(K_LOW, st, 0.0, 0.0, L);
         MSG_CHECK_LAUNCH();
     } else {
-        rc = cycle_attributes<double>();
+        rc = cycle_attributes<double>(true, true);
         if (rc != MSG_OK) return rc;
         for (int d = kMidD + 1; d <= L; ++d) {
             lists[d].cx = cx;
