@@ -404,6 +404,7 @@ __global__ void __launch_bounds__(512, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int2 at[kMidMax + 1];
     __shared__ int s_act;
+    launch_next();
     const TaskRef t = resolve(cx);
     const SampleInfo& S = cx.samples[t.s];
     const int p = t.seg->pi, q = t.seg->qi, nx = 1 << p, ny = 1 << q, W = nx + 1, tid = threadIdx.x;
@@ -418,6 +419,7 @@ __global__ void __launch_bounds__(512, 1)
     mid_fill(m, S, ax, ay, op);
     for (int d = lo; d < lo + keep && d <= L; ++d) kept_load(m, tb, d, S, ax, ay);
     if (lo > 0) kept_op(m, tb);
+    wait_previous();
     item_guess(S, p, q, u64, ax64, ay64);
     __syncthreads();
     const MidDiag<T> g = mid_diag(m, L);
