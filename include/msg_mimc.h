@@ -82,11 +82,11 @@ typedef struct {
     int32_t precision;  /* MSG_PREC_* */
     int32_t qoi;        /* MSG_QOI_* */
     int32_t coef;       /* MSG_COEF_*: coarse-face coefficient */
-    int32_t tune_block; /* launch shape: threads per CTA of the visit kernels (0: 128; multiple of 32): the global-memory visits of mid-size grids use it (small grids fewer, grids of 2^12+ cells twice as many); the register-cached visits give each thread 1, 2 or 4 nodes of a colour so as to stay near it */
+    int32_t tune_block; /* launch shape: threads per CTA of the visit kernels (multiple of 32).  0: as few CTAs per grid as hold it at two pairs of nodes a thread; else at most that many threads, where the rows of the launch's grids can be cut into more slabs (a cluster of up to 16 CTAs a grid).  The global-memory visits of thin grids use 128 when 0.  Results do not depend on it */
     int32_t tune_low_warps; /* launch shape: warps per CTA of the low-diagonal phase kernel, used when tune_low_cut is set (0: default; 1..16) */
     int32_t tune_low_items; /* launch shape: items one warp of that kernel runs in lockstep: 1, 2, 4 or 8 (0: default) */
     int32_t tune_low_cut;   /* schedule: 0 (default): the low stages whole, and the recursion below a fixed diagonal of the later ones, run on chip, one item per CTA, with the calls on diagonal 3 as one matrix per sample; 1..5: the highest diagonal of each hierarchy that the phase kernel runs instead.  Launch shapes never change results; the cut changes only the rounding of the inner cycles */
-    int32_t tune_visit_smem; /* schedule: KB of shared memory per CTA up to which a visit above the cut runs register-cached (u in shared memory; each thread keeps its nodes' coefficients and right-hand side in registers for the whole visit; grids of up to 2048 nodes per colour in the mixed path, 1024 in FP64) instead of in global memory (0: default 1; 1..227; 1 keeps every visit in global memory, the faster at 256 x 256).  Changes only the rounding of the cycles */
+    int32_t tune_visit_smem; /* schedule: 0 or 1: every visit above the on-chip diagonals as described at tune_block, the fastest.  2..227: no such visits; a visit runs register-cached (each thread keeps its nodes' coefficients and right-hand side in registers) where u fits that many KB of shared memory (grids of up to 2048 nodes per colour in the mixed path, 1024 in FP64), else in global memory.  Changes only the rounding of the cycles */
 } msg_params;
 
 /* ------------------------------------------------------------------------ */

@@ -3,7 +3,8 @@
 The solver's results do not depend on its launch shapes; its speed does.  The
 shapes tuned here, per call through msg_params, are the threads per CTA of the
 per-visit kernels (``tune_block``) and the items per warp and warps per CTA of
-the low-diagonal kernel (``tune_low_items``, ``tune_low_warps``).  ``tune``
+the low-diagonal kernel (``tune_low_items``, ``tune_low_warps``; without effect
+unless ``tune_low_cut`` selects that kernel).  ``tune``
 times msg_solve_batch on a sub-batch of the caller's own samples (CUDA events
 on the launching stream) over a small set of candidates by coordinate descent,
 starting from the library defaults, and caches the best per batch composition.
