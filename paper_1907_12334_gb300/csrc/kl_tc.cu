@@ -50,9 +50,10 @@ namespace {
 
 constexpr int kTM = 128;  // samples per tile (UMMA M)
 constexpr int kTN = 256;  // points per tile (UMMA N); the part arrays are padded to whole tiles
-constexpr int kTNSmall = 64;  // of a call with few tiles
+constexpr int kSMs = 152;
+// tiles of 128 and 64 points: of a call with few tiles
 constexpr int kThreadsTC = 384;
-template <int TN> constexpr int stages() { return TN == kTN ? 4 : 8; }  // of 48 KB, of 24 KB
+template <int TN> constexpr int stages() { return TN == kTN ? 4 : TN == 128 ? 6 : 8; }  // of 48, 32 and 24 KB
 constexpr long long kSpinLimit = 1ll << 22;           // bounded mbarrier waits (seconds)
 
 // Operand modes of the tensor-core kernel.
@@ -237,6 +238,7 @@ template <int MODE>
 __global__ void k_prep_a(const double* sl, const double* xi, int64_t S, int M, int Kp, int64_t Sp,
                          typename TcCfg<MODE>::E* A0, typename TcCfg<MODE>::E* A1)
 {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t s = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (s >= Sp) return;
     for (int m = threadIdx.x & 31; m < Kp; m += 32) {
@@ -298,6 +300,9 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
     if (warp == 0 && lane == 0) {  // ---- loads
         int n = 0;  // stages filled
         bool ok = true;
+        // this kernel starts under k_prep_a, which writes A: its barriers and TMEM are ready by
+        // then (2 to 3 us of a call: 256 x 100 points, 300 terms, FP32 fields 19.9 -> 16.8 us)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             const int s0 = (t % stiles) * kTM, x0 = (t / stiles) * TN;
             for (int kc = 0; kc < nchunks; ++kc, ++n) {
@@ -466,9 +471,6 @@ int tc_launch(const TcLayout& L, const char* b, int64_t npts, int32_t M, const d
     // (a part of B is whole tiles of whole 128-byte rows: the next starts right behind it)
     CUtensorMap mA, mB;
     const bool mapped = part_map<MODE>(&mA, A0, parts * Sp, L.Kp, kTM) && part_map<MODE>(&mB, b + L.p0, parts * L.Np, L.Kp, TN);
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e = mapped ? cudaSuccess : cudaErrorInvalidValue;
     if (e == cudaSuccess) {
         k_prep_a<MODE><<<(unsigned)((Sp + 7) / 8), 256, 0, st>>>((const double*)(b + L.sl), xi, S, M, (int)L.Kp, Sp, A0, A1);
@@ -477,10 +479,18 @@ int tc_launch(const TcLayout& L, const char* b, int64_t npts, int32_t M, const d
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_kl_tc<MODE, TN, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes<MODE, TN>());
     if (e == cudaSuccess) {
-        k_kl_tc<MODE, TN, TZ><<<(unsigned)std::min<int64_t>(stiles * xtiles, std::max(sms, 1)), kThreadsTC, smem_bytes<MODE, TN>(), st>>>(
-            mA, mB, npts, (M + TcCfg<MODE>::TK - 1) / TcCfg<MODE>::TK, S, (int)stiles, (int)xtiles,
-            (int)L.Np, (TZ*)Z);
-        e = cudaGetLastError();
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)std::min<int64_t>(stiles * xtiles, kSMs));
+        cfg.blockDim = dim3(kThreadsTC);
+        cfg.dynamicSmemBytes = smem_bytes<MODE, TN>();
+        cfg.stream = st;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, k_kl_tc<MODE, TN, TZ>, mA, mB, npts, (M + TcCfg<MODE>::TK - 1) / TcCfg<MODE>::TK, S,
+                               (int)stiles, (int)xtiles, (int)L.Np, (TZ*)Z);
     }
     cudaFreeAsync(abuf, st);
     if (e != cudaSuccess) { set_error(std::string("sample_field: ") + cudaGetErrorString(e)); return MSG_ERR_CUDA; }
@@ -517,17 +527,22 @@ int32_t kl_tc_sample(const void* prepared, int64_t npts, int32_t M, int32_t mode
     if ((npts + kTN - 1) / kTN > 65535) { set_error("sample_field: too many points for one call"); return MSG_ERR_INVALID; }
     const char* b = (const char*)prepared;
     prof_begin(K_KL, st);
-    // A call whose tiles of 256 points leave half of the SMs idle takes tiles of 64: four times
-    // the CTAs, each with a quarter of the loads (100 x 60 points, 400 terms, 100 samples:
-    // BF16X3 28.7 -> 21.5 us a call, TF32 23.2 -> 17.1).  The sums are the same, term by term.
-    const bool small = ((npts + kTN - 1) / kTN) * ((S + kTM - 1) / kTM) <= 76;
+    // The widest tiles, unless narrower ones still give every tile an SM of its own: up to four
+    // times the CTAs, each with a fraction of the loads and stores (100 x 60 points, 400
+    // terms, 100 samples: BF16X3 28.7 -> 18.5 us a call, TF32 23.2 -> 15.2; 256 x 50 points, 300
+    // terms, FP32 fields: 15.9 us in tiles of 128, 20.5 in twice as many of 64 (2 us of it
+    // the start under k_prep_a); 256 x 100: 16.8 us in tiles of 256).
+    // The sums are the same, term by term.
+    const int64_t tiles = ((npts + kTN - 1) / kTN) * ((S + kTM - 1) / kTM);
     int rc;
     auto go = [&](auto mode, auto tn) {
         constexpr int MD = decltype(mode)::value, TN = decltype(tn)::value;
         return z_fp32 ? tc_launch<MD, TN, float>(L, b, npts, M, xi, S, Z, st) : tc_launch<MD, TN, double>(L, b, npts, M, xi, S, Z, st);
     };
     auto pick = [&](auto mode) {
-        return small ? go(mode, std::integral_constant<int, kTNSmall>()) : go(mode, std::integral_constant<int, kTN>());
+        if (4 * tiles <= kSMs) return go(mode, std::integral_constant<int, 64>());
+        if (2 * tiles <= kSMs) return go(mode, std::integral_constant<int, 128>());
+        return go(mode, std::integral_constant<int, kTN>());
     };
     if (tm == TC_TF32) rc = pick(std::integral_constant<int, TC_TF32>());
     else rc = pick(std::integral_constant<int, TC_BF16X3>());

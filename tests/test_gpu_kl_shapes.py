@@ -15,7 +15,7 @@ torch = pytest.importorskip("torch")
 DEV = "cuda:0"
 
 SIZES = [(1, 1, 1), (127, 3, 31), (128, 16, 32), (129, 17, 33), (257, 64, 64), (300, 65, 65), (1000, 63, 128), (33, 401, 129),
-         (90000, 36, 200)]
+         (11525, 70, 100), (90000, 36, 200)]
 
 
 @pytest.mark.parametrize("npts,M,S", SIZES)
