@@ -284,19 +284,42 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 }
 
 namespace {
-// The sample tile that pads S least; a temporary for A, or the kernel that needs none.
+// Form of an FP32 call: the sample tile is 16 TR, and DIRECT forms A in the tile.
+//
+// A wave of one tile an SM takes about 3, 4 and 7 units of time for TR 2, 4 and 8, so the
+// widest tile is the cheapest that fills its waves, and the narrowest the fastest of a call
+// that gives every SM at most one; a single wave of the widest loses to two of the next one
+// by what its start and end cost with few terms (below 200).  Choosing by S alone left most
+// SMs without a tile: 400 points, 600 samples, 64 terms 20.5 us with TR 8, 8.3 with TR 2 (the 64 x 64
+// tiles of k_kl_simt: 12.8); 4000, 200, 300 47.2 us with TR 8, 30.8 with TR 4 (53.3).
+//
+// Forming A in the tile costs the FP64 pipe 16 TR M clocks a wave; a launch and a temporary
+// in front cost the call 4 to 6 us.  The two are even at 9600 clocks: 2048 points, 200
+// samples 8.3 and 12.4 us at 64 terms, 24.7 and 24.7 at 300, 30.8 and 28.7 at 400.  Every
+// form sums the same terms in the same order.
+struct KlForm {
+    int TR;
+    bool direct;
+};
+int64_t kl_f32_tiles(int64_t npts, int64_t S, int TR) { return (S + 16 * TR - 1) / (16 * TR) * ((npts + 127) / 128); }
+KlForm kl_f32_form(int64_t npts, int32_t M, int64_t S)
+{
+    auto waves = [&](int TR) { return (kl_f32_tiles(npts, S, TR) + 151) / 152; };
+    const int64_t t8 = 14 * waves(8) + (M < 200 ? 3 : 1), t4 = 8 * waves(4), t2 = 6 * waves(2);
+    const int TR = t2 < std::min(t4, t8) ? 2 : t4 < t8 ? 4 : 8;
+    return KlForm{TR, 16LL * TR * M * waves(TR) <= 9600};
+}
+
+// (a temporary for A, or the kernel that needs none)
 template <class TZ>
 void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts, int M, int64_t S, TZ* Z, cudaStream_t st)
 {
-    const int Mp = (M + 3) & ~3, TR = S <= 32 ? 2 : S <= 64 ? 4 : 8;
-    const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = stiles * ((npts + 127) / 128);
+    const KlForm f = kl_f32_form(npts, M, S);
+    const int Mp = (M + 3) & ~3, TR = f.TR;
+    const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = kl_f32_tiles(npts, S, TR);
     const unsigned g = (unsigned)tiles;
     const int vec = M == (M & ~3) && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
-    // Few tiles with few coefficients each: forming them in the tile costs the FP64 pipe less
-    // (16 TR M / 2 clocks a tile and SM) than a launch and a temporary cost the call: 9 x 9
-    // points, 20 terms, 8 samples 10.8 -> 8.2 us, 250 x 200, 60, 20 16.4 us (the sums are the
-    // same bits).  The line is at 15000 clocks, 7 us; 200 x 100, 300, 60 lies above it with 47 us.
-    if (16LL * TR * M * ((tiles + 151) / 152) <= 15000) {
+    if (f.direct) {
         if (TR == 2) k_kl_f32<2, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
         else if (TR == 4) k_kl_f32<4, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
         else k_kl_f32<8, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);

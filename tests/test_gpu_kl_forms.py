@@ -1,0 +1,35 @@
+"""Every form of the FP32 contraction (three sample tiles, coefficients formed in the tile
+or before it) at sizes with ragged tiles: within the FP32 bound of FP64, (M + 4) 2^-24 of
+sum_m |Phi sqrt(lambda) xi|, and with the bits that the first samples have in a small call."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+DEV = "cuda:0"
+
+# narrow tiles direct and not, middle tiles direct and not, wide tiles direct and not
+SIZES = [(401, 64, 333), (401, 301, 333), (11525, 70, 101), (11525, 150, 101), (40001, 3, 500), (40001, 37, 500)]
+
+
+@pytest.mark.parametrize("npts,M,S", SIZES)
+def test_forms_agree(npts, M, S):
+    from paper_1907_12334_gb300 import build, msg
+
+    build.build()
+    g = torch.Generator(device=DEV).manual_seed(npts + M + S)
+    Phi = torch.randn(npts, M, dtype=torch.float64, device=DEV, generator=g)
+    sl = torch.rand(M, dtype=torch.float64, device=DEV, generator=g) + 0.1
+    xi = torch.randn(S, M, dtype=torch.float64, device=DEV, generator=g)
+    prep = torch.empty(msg.kl_prepared_bytes(npts, M, msg.MSG_GEMM_FP32), dtype=torch.uint8, device=DEV)
+    msg.kl_prepare(Phi, sl, msg.MSG_GEMM_FP32, prep)
+
+    def field(n):
+        Z = torch.full((n, npts), float("nan"), dtype=torch.float64, device=DEV)
+        msg.sample_field(prep, npts, M, msg.MSG_GEMM_FP32, xi[:n].contiguous(), Z)
+        return Z
+
+    Z = field(S)
+    assert torch.equal(Z[:5], field(5))
+    ref, scale = (xi * sl) @ Phi.T, (xi * sl).abs() @ Phi.abs().T
+    assert bool(((Z - ref).abs() <= (M + 4) * 2.0 ** -24 * scale).all())
