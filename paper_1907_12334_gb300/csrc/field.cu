@@ -79,7 +79,8 @@ __global__ void __launch_bounds__(256, 2) k_kl_f32(const float* __restrict__ Phi
     const int kq = 4 * (tid & 3), row = tid >> 2;
     // vec: every row of Phi starts on 16 bytes
     float4 ra[NA], rb[NB];
-    // this thread's rows relative to the tiles, at its first terms
+    // this thread's rows relative to the tiles, at its first terms (pointers to them spill at
+    // TR 8: 513 x 513 points 2.35 -> 2.50 ms; the caller sees that 128 rows fit 32 bits)
     const float *tA = DIRECT ? nullptr : A + s0 * Mp, *tB = Phi + x0 * M;
     const double* tX = DIRECT ? xi + s0 * M : nullptr;
     int oa[NA], ob[NB];
@@ -184,8 +185,8 @@ __global__ void __launch_bounds__(256) k_kl_f64(const double* __restrict__ Phi, 
     const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
     const int64_t x0 = (int64_t)(blockIdx.x % xtiles) * 32, s0 = (int64_t)(blockIdx.x / xtiles) * 8;
     double acc = 0.0;
-    for (int k0 = 0; k0 < M; k0 += BK) {
-        const int nk = min(BK, M - k0);
+    for (int64_t k0 = 0; k0 < M; k0 += BK) {
+        const int nk = (int)min((int64_t)BK, M - k0);
         for (int e = tid; e < 8 * BK; e += 256) {
             const int r = e >> 6, k = e & 63;
             if (k < nk) sA[r][k] = s0 + r < S ? sl[k0 + k] * xi[(s0 + r) * M + k0 + k] : 0.0;
@@ -203,8 +204,8 @@ __global__ void __launch_bounds__(256) k_kl_f64(const double* __restrict__ Phi, 
     if (x < npts && s < S) Z[s * npts + x] = (TZ)acc;
 }
 
-// FP32 without a temporary for A (when none can be had): 64x64 tile per CTA, 16-deep K
-// slices staged in shared memory, 4x4 outputs per thread.
+// FP32 without a temporary for A (when none can be had) and for rows of any length: 64x64
+// tile per CTA, 16-deep K slices staged in shared memory, 4x4 outputs per thread.
 template <class TZ>
 __global__ void __launch_bounds__(256) k_kl_simt(const float* __restrict__ Phi, const double* __restrict__ sl,
                                                  const double* __restrict__ xi, int64_t npts, int M, int64_t S,
@@ -219,11 +220,11 @@ __global__ void __launch_bounds__(256) k_kl_simt(const float* __restrict__ Phi, 
     for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-    for (int k0 = 0; k0 < M; k0 += 16) {
+    for (int64_t k0 = 0; k0 < M; k0 += 16) {
         for (int e = threadIdx.x; e < 64 * 16; e += 256) {
             int r = e / 16, k = e % 16;
             int64_t s = s0 + r, x = x0 + r;
-            int m = k0 + k;
+            const int64_t m = k0 + k;
             sA[k][r] = (s < S && m < M) ? (float)(sl[m] * xi[s * M + m]) : 0.f;
             sB[k][r] = (x < npts && m < M) ? Phi[x * M + m] : 0.f;
         }
@@ -310,10 +311,16 @@ KlForm kl_f32_form(int64_t npts, int32_t M, int64_t S)
     return KlForm{TR, 16LL * TR * M * waves(TR) <= 9600};
 }
 
-// (a temporary for A, or the kernel that needs none)
+// (a temporary for A, or the kernel that needs none, also where a tile's 128 rows of terms
+// exceed 32-bit offsets)
 template <class TZ>
 void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts, int M, int64_t S, TZ* Z, cudaStream_t st)
 {
+    const dim3 simt((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
+    if (M > 0x7fffffff / 128 - 4) {
+        k_kl_simt<TZ><<<simt, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
+        return;
+    }
     const KlForm f = kl_f32_form(npts, M, S);
     const int Mp = (M + 3) & ~3, TR = f.TR;
     const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = kl_f32_tiles(npts, S, TR);
@@ -327,8 +334,7 @@ void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts,
     }
     void* A = nullptr;
     if (tiles > 0x7fffffffLL || temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) {
-        const dim3 grid((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
-        k_kl_simt<TZ><<<grid, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
+        k_kl_simt<TZ><<<simt, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
         return;
     }
     k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);

@@ -33,3 +33,24 @@ def test_forms_agree(npts, M, S):
     assert torch.equal(Z[:5], field(5))
     ref, scale = (xi * sl) @ Phi.T, (xi * sl).abs() @ Phi.abs().T
     assert bool(((Z - ref).abs() <= (M + 4) * 2.0 ** -24 * scale).all())
+
+
+@pytest.mark.parametrize("mode", ["FP32", "FP64"])
+def test_rows_of_many_terms(mode):
+    """A tile of points whose rows hold more than 2^31 terms together (its last row starts
+    beyond a 32-bit offset).  Few nonzero coefficients and a basis of small whole numbers: exact."""
+    from paper_1907_12334_gb300 import build, msg
+
+    build.build()
+    npts, M, m = 128, 17_000_003, getattr(msg, f"MSG_GEMM_{mode}")
+    Phi = torch.arange(npts, dtype=torch.float64, device=DEV)[:, None] + torch.arange(M, dtype=torch.float64, device=DEV)[None]
+    Phi.remainder_(7)
+    at = torch.tensor([0, 15, 16, 12_345_678, M - 17, M - 2, M - 1], device=DEV)
+    xi = torch.zeros(1, M, dtype=torch.float64, device=DEV)
+    xi[0, at] = torch.arange(1, 8, dtype=torch.float64, device=DEV)
+    sl = torch.ones(M, dtype=torch.float64, device=DEV)
+    prep = torch.empty(msg.kl_prepared_bytes(npts, M, m), dtype=torch.uint8, device=DEV)
+    msg.kl_prepare(Phi, sl, m, prep)
+    Z = torch.empty(1, npts, dtype=torch.float64, device=DEV)
+    msg.sample_field(prep, npts, M, m, xi, Z)
+    assert torch.equal(Z[0], Phi[:, at] @ xi[0, at])
