@@ -127,6 +127,9 @@ cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st)
         if (it != pools.end()) {
             pool = it->second;
         } else {
+            // making a pool would end a capture, of this thread or of another one
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
             cudaMemPoolProps props{};
             props.allocType = cudaMemAllocationTypePinned;
             props.location.type = cudaMemLocationTypeDevice;
@@ -134,6 +137,7 @@ cudaError_t temp_alloc(void** p, size_t bytes, cudaStream_t st)
             e = cudaMemPoolCreate(&pool, &props);
             uint64_t keep = kTempKeep;
             if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            cudaThreadExchangeStreamCaptureMode(&mode);
             if (e == cudaSuccess) pools[dev] = pool;
         }
     }
