@@ -47,7 +47,7 @@ __global__ void k_normals(uint64_t seed, uint64_t s0, int64_t S, int M, double* 
 
 // A rounded to FP32 once per call, rows padded to a multiple of four terms with zeros.
 // (The product is taken in FP64, whose rate is 1/64 of FP32's here: formed again in every
-// tile, as k_kl_simt does, it costs as much as the contraction.)
+// tile, it costs a large call as much as the contraction.)
 __global__ void k_kl_a32(const double* __restrict__ sl, const double* __restrict__ xi, int64_t S, int M, int Mp, float* A)
 {
     const int64_t n = S * Mp;
@@ -204,8 +204,8 @@ __global__ void __launch_bounds__(256) k_kl_f64(const double* __restrict__ Phi, 
     if (x < npts && s < S) Z[s * npts + x] = (TZ)acc;
 }
 
-// FP32 without a temporary for A (when none can be had) and for rows of any length: 64x64
-// tile per CTA, 16-deep K slices staged in shared memory, 4x4 outputs per thread.
+// FP32 for rows of any length: 64x64 tile per CTA, 16-deep K slices staged in shared memory,
+// 4x4 outputs per thread.
 template <class TZ>
 __global__ void __launch_bounds__(256) k_kl_simt(const float* __restrict__ Phi, const double* __restrict__ sl,
                                                  const double* __restrict__ xi, int64_t npts, int M, int64_t S,
@@ -311,37 +311,34 @@ KlForm kl_f32_form(int64_t npts, int32_t M, int64_t S)
     return KlForm{TR, 16LL * TR * M * waves(TR) <= 9600};
 }
 
-// (a temporary for A, or the kernel that needs none, also where a tile's 128 rows of terms
-// exceed 32-bit offsets)
+// Without a temporary for A (none can be had, or the stream is captured: a graph with an
+// allocation can neither be instantiated twice nor be part of another) every form is direct:
+// 20000 points, 400 terms, 1000 samples 559 us, with the temporary 420, in the 64 x 64
+// tiles 799.  Those take what 32-bit offsets into a tile's 128 rows cannot.
 template <class TZ>
 void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts, int M, int64_t S, TZ* Z, cudaStream_t st)
 {
-    const dim3 simt((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64));
-    if (M > 0x7fffffff / 128 - 4) {
-        k_kl_simt<TZ><<<simt, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
-        return;
-    }
     const KlForm f = kl_f32_form(npts, M, S);
-    const int Mp = (M + 3) & ~3, TR = f.TR;
-    const int64_t stiles = (S + 16 * TR - 1) / (16 * TR), tiles = kl_f32_tiles(npts, S, TR);
-    const unsigned g = (unsigned)tiles;
-    const int vec = M == (M & ~3) && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
-    if (f.direct) {
-        if (TR == 2) k_kl_f32<2, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
-        else if (TR == 4) k_kl_f32<4, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
-        else k_kl_f32<8, true, TZ><<<g, 256, 0, st>>>(Phi, nullptr, sl, xi, npts, M, Mp, S, stiles, vec, Z);
+    const int64_t stiles = (S + 16 * f.TR - 1) / (16 * f.TR), tiles = kl_f32_tiles(npts, S, f.TR);
+    if (M > 0x7fffffff / 128 - 4 || tiles > 0x7fffffffLL) {
+        k_kl_simt<TZ><<<dim3((unsigned)((npts + 63) / 64), (unsigned)((S + 63) / 64)), 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
         return;
     }
+    const int Mp = (M + 3) & ~3;
+    const int vec = M == Mp && (uintptr_t)Phi % 16 == 0;  // (the prepared buffer may have any alignment)
     void* A = nullptr;
-    if (tiles > 0x7fffffffLL || temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) {
-        k_kl_simt<TZ><<<simt, 256, 0, st>>>(Phi, sl, xi, npts, M, S, Z);
-        return;
+    if (!f.direct) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+        if (capture == cudaStreamCaptureStatusNone && temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) A = nullptr;
     }
-    k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);
-    if (TR == 2) k_kl_f32<2, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
-    else if (TR == 4) k_kl_f32<4, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
-    else k_kl_f32<8, false, TZ><<<g, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z);
-    cudaFreeAsync(A, st);
+    if (A)
+        k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);
+    auto go = [&](auto kernel) { kernel<<<(unsigned)tiles, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z); };
+    if (f.TR == 2) go(A ? k_kl_f32<2, false, TZ> : k_kl_f32<2, true, TZ>);
+    else if (f.TR == 4) go(A ? k_kl_f32<4, false, TZ> : k_kl_f32<4, true, TZ>);
+    else go(A ? k_kl_f32<8, false, TZ> : k_kl_f32<8, true, TZ>);
+    if (A) cudaFreeAsync(A, st);
 }
 }  // namespace
 

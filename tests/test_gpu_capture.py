@@ -47,3 +47,33 @@ def _run(script, mode):
 @pytest.mark.parametrize("mode", ["FP32", "BF16X3", "TF32", "FP64"])
 def test_first_call_can_be_captured(mode):
     _run(REPLAY, mode)
+
+
+TWICE = SETUP + """
+import ctypes
+rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+def ok(rc):
+    assert rc == 0, rc
+s = torch.cuda.Stream()
+st = ctypes.c_void_p(s.cuda_stream)
+graph, execs = ctypes.c_void_p(), [ctypes.c_void_p(), ctypes.c_void_p()]
+ok(rt.cudaStreamBeginCapture(st, 0))
+msg.sample_field(prep, npts, M, mode, xi, Z, stream=s)
+ok(rt.cudaStreamEndCapture(st, ctypes.byref(graph)))
+for e in execs:
+    ok(rt.cudaGraphInstantiate(ctypes.byref(e), graph, ctypes.c_ulonglong(0)))
+for e in execs:
+    Z.zero_()
+    torch.cuda.synchronize()
+    ok(rt.cudaGraphLaunch(e, st))
+    s.synchronize()
+    got = Z.clone()
+msg.sample_field(prep, npts, M, mode, xi, Z)
+torch.cuda.synchronize()
+assert torch.equal(got, Z)
+"""
+
+
+def test_captured_fp32_call_allocates_nothing():
+    """Its graph can be instantiated twice, which one with an allocation cannot."""
+    _run(TWICE, "FP32")
