@@ -958,12 +958,14 @@ __global__ void __launch_bounds__(256) k_history_chip(DevCtx cx, int L, const do
 }
 
 // The same on larger hierarchies, between the launches of the cycles (b in sbx, u in su
-// of each sample's scratch): start values of the top grid, and one entry of the history.
+// of each sample's scratch): start values of the top grid of sample blockIdx.x (blockIdx.y: a
+// slice of it; the other way round a study had at most 65535 samples), and one entry of the
+// history.
 __global__ void k_history_start(int P, int Q, int64_t R, double* su, double* sbx)
 {
     const int W = (1 << P) + 1, n = W * ((1 << Q) + 1);
-    const int64_t o = (int64_t)blockIdx.y * R + grid_offset(P, Q, Q);
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+    const int64_t o = (int64_t)blockIdx.x * R + grid_offset(P, Q, Q);
+    for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < n; k += gridDim.y * blockDim.x) {
         su[o + k] = 0.0;
         sbx[o + k] = 1.0;  // (the boundary's is not read)
     }
