@@ -295,8 +295,8 @@ int32_t msg_profile_read_level(int32_t kernel_class, int32_t level, int64_t* tim
 
 /* Deferred kernel status (no counterpart in the paper).  Kernels with bounded */
 /* pipeline waits (the tensor-core KL contraction) do not stop the stream to   */
-/* report: a wait that runs out records it on the device and that kernel      */
-/* leaves its output unwritten.  msg_device_status synchronises the current    */
+/* report: a wait that runs out records it on the device and that kernel       */
+/* leaves its output incomplete.  msg_device_status synchronises the current   */
 /* device and returns MSG_ERR_TIMEOUT if any such wait ran out since the       */
 /* previous call (the record is then cleared), else MSG_OK.                    */
 int32_t msg_device_status(void);

@@ -133,6 +133,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
     return false;
 }
 
+// The same for a whole warp, which goes on or gives up as one: its lanes can see the end of
+// the phase and the giving up on different sides of each other, and the warp-wide TMEM load
+// behind the wait needs every lane.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* dead)
+{
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, dead));
+}
+
 __device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes)
 {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -360,7 +368,7 @@ __global__ void __launch_bounds__(kThreadsTC, 1)
         int w = 0;
         for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++w) {
             const int64_t s0 = (int64_t)(t % stiles) * kTM + lane_base, x0 = (int64_t)(t / stiles) * TN + col_base;
-            if (!mbar_wait(&acc_full[w & 1], (w >> 1) & 1, &dead)) break;
+            if (!warp_wait(&acc_full[w & 1], (w >> 1) & 1, &dead)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint32_t acc = tmem + ((uint32_t)lane_base << 16) + (uint32_t)((w & 1) * TN + col_base);
             const int rows = (int)min((int64_t)32, S - s0);  // may be <= 0
@@ -565,7 +573,7 @@ extern "C" int32_t msg_device_status(void)
     MSG_CUDA_TRY(cudaMemcpyFromSymbol(&err, msg::g_tc_error, sizeof(int)));
     MSG_CUDA_TRY(cudaMemcpyToSymbol(msg::g_tc_error, &zero, sizeof(int)));
     if (err) {
-        msg::set_error("a bounded wait in a tensor-core kernel ran out; its output was not written");
+        msg::set_error("a bounded wait in a tensor-core kernel ran out; its output is incomplete");
         return MSG_ERR_TIMEOUT;
     }
     return MSG_OK;
