@@ -27,7 +27,7 @@ enum { KF_X = 1, KF_Y = 2, KF_REDB = 4, KF_PX = 8, KF_PY = 16, KF_A = 32, KF_OK 
 
 // Records behind the arrays of an item: per kept diagonal a row for each of its pairs (whole
 // warps); field f of row k at (f rows + k) 16 bytes:
-//   0  pR oR sR nR      1  pK oK sK nK      2  iR iK bR bK      3  aR e w -
+//   0  pR oR sR nR      1  pK oK sK nK      2  iR iK bR bK      3  aR e w dR
 //   4  {black node's child column | flags << 24, its child row, the pair's residuals in its
 //      x-parent, in its y-parent} as addresses
 // then, for the children of diagonal lo = kOpD + 1, a row per pair of them, and the cells of
@@ -135,7 +135,7 @@ __device__ __forceinline__ void kept_load(const MidItem<T>& m, const KeptTables&
     sts4(a, bits4(P.pR, P.oR, P.sR, P.nR));
     sts4(a + t.field, bits4(P.pK, P.oK, P.sK, P.nK));
     sts4(a + 2 * t.field, bits4(iR, iK, 0.f, 0.f));
-    sts4(a + 3 * t.field, make_uint4(P.aR, P.e, P.w, 0u));
+    sts4(a + 3 * t.field, make_uint4(P.aR, P.e, P.w, __float_as_uint(P.dR)));
     sts4(a + 4 * t.field, g);
 }
 
@@ -202,10 +202,8 @@ __device__ __forceinline__ void kept_pair(Pair<float>& P, const KeptTables& t, u
     P.pR = r.x; P.oR = r.y; P.sR = r.z; P.nR = r.w;
     P.pK = k.x; P.oK = k.y; P.sK = k.z; P.nK = k.w;
     P.bR = b.z; P.bK = b.w;
-    // (infinite at a boundary node, where the difference it multiplies is zero: the
-    // residual there is not a number, and no child uses it)
-    P.dR = rcp_of(b.x);
     P.aR = g.x; P.e = g.y; P.w = g.z;
+    P.dR = __uint_as_float(g.w);  // (the sum of the faces: the reciprocal of iR is up to three ulp off)
 }
 
 // b of the record's pair from nodes' values A and B
