@@ -332,8 +332,10 @@ void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts,
         if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
         if (capture == cudaStreamCaptureStatusNone && temp_alloc(&A, sizeof(float) * S * Mp, st) != cudaSuccess) A = nullptr;
     }
-    if (A)
+    if (A) {
         k_kl_a32<<<(unsigned)std::min<int64_t>((S * Mp + 255) / 256, 152 * 8), 256, 0, st>>>(sl, xi, S, M, Mp, (float*)A);
+        prof_also();
+    }
     auto go = [&](auto kernel) { kernel<<<(unsigned)tiles, 256, 0, st>>>(Phi, (const float*)A, sl, xi, npts, M, Mp, S, stiles, vec, Z); };
     if (f.TR == 2) go(A ? k_kl_f32<2, false, TZ> : k_kl_f32<2, true, TZ>);
     else if (f.TR == 4) go(A ? k_kl_f32<4, false, TZ> : k_kl_f32<4, true, TZ>);

@@ -482,6 +482,7 @@ int tc_launch(const TcLayout& L, const char* b, int64_t npts, int32_t M, const d
     cudaError_t e = mapped ? cudaSuccess : cudaErrorInvalidValue;
     if (e == cudaSuccess) {
         k_prep_a<MODE><<<(unsigned)((Sp + 7) / 8), 256, 0, st>>>((const double*)(b + L.sl), xi, S, M, (int)L.Kp, Sp, A0, A1);
+        prof_also();
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)

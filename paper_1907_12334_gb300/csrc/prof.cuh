@@ -25,8 +25,10 @@ enum KernelClass {
 //   prof_begin(cls, st) before the launch, prof_end(cls, st, bytes, flops, level) after.
 // They count launches always and, while profiling is on, record CUDA events on
 // `st` for a random 1/n of each class's launches.  `level` tags multigrid
-// launches with their diagonal (-1: none).
+// launches with their diagonal (-1: none).  A second launch between the two is counted by
+// prof_also(), and timed with the first.
 void prof_begin(int cls, cudaStream_t st);
 void prof_end(int cls, cudaStream_t st, double bytes, double flops, int level = -1);
+void prof_also();
 
 }  // namespace msg

@@ -3395,7 +3395,9 @@ extern "C" int32_t msg_cycle_history(int32_t P, int32_t Q, int64_t S, const msg_
             lists[d].host = segs.data() + first[d];
         }
         const int n = ((1 << P) + 1) * ((1 << Q) + 1);
+        prof_begin(K_UPDATE, st);
         k_history_start<<<dim3((unsigned)S, (unsigned)((n + 255) / 256)), 256, 0, st>>>(P, Q, R, su, sbx);
+        prof_end(K_UPDATE, st, (double)S * n * 16.0, 0.0);
         MSG_CHECK_LAUNCH();
         bool bad = false;
         for (int cyc = 0; cyc <= ncycles && !bad; ++cyc) {
