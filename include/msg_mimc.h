@@ -23,6 +23,12 @@
  *     it runs (its schedule reads per-step convergence counts on the host), and
  *     mimc_differences_noalloc and msg_cycle_history return after their work
  *     has finished;
+ *   - sample_field and mimc_differences take stream-ordered temporaries from a
+ *     pool of the library's own, one per device, made by the first call that needs
+ *     it (64 MiB are kept between calls; the pool does not survive a
+ *     cudaDeviceReset).  sample_field may be captured, also as a first call: with
+ *     FP64 and FP32 products the graph then holds no allocation, on the tensor
+ *     cores one temporary that it allocates and frees;
  *   - the return value is MSG_OK or an error code; on error
  *     msg_last_error() returns a description (thread-local string);
  *   - no entry point traps or aborts; per-sample numerical failures are
@@ -82,11 +88,11 @@ typedef struct {
     int32_t precision;  /* MSG_PREC_* */
     int32_t qoi;        /* MSG_QOI_* */
     int32_t coef;       /* MSG_COEF_*: coarse-face coefficient */
-    int32_t tune_block; /* launch shape: threads per CTA of the visit kernels (multiple of 32).  0: as few CTAs per grid as hold it at two pairs of nodes a thread; else at most that many threads, where the rows of the launch's grids can be cut into more slabs (a cluster of up to 16 CTAs a grid).  The global-memory visits of thin grids use 128 when 0.  Results do not depend on it */
+    int32_t tune_block; /* launch shape: threads per CTA of the visit kernels (multiple of 32).  0: as few CTAs per grid as hold it at two pairs of nodes a thread; else at most that many threads, where the rows of the launch's grids can be cut into more slabs (a cluster of up to 16 CTAs a grid).  The visits in global memory (see tune_visit_smem) have 128 when 0, and twice as many on grids of 2^12 cells and more.  Results do not depend on it */
     int32_t tune_low_warps; /* launch shape: warps per CTA of the low-diagonal phase kernel, used when tune_low_cut is set (0: default; 1..16) */
     int32_t tune_low_items; /* launch shape: items one warp of that kernel runs in lockstep: 1, 2, 4 or 8 (0: default) */
     int32_t tune_low_cut;   /* schedule: 0 (default): the low stages whole, and the recursion below a fixed diagonal of the later ones, run on chip, one item per CTA, with the calls on diagonal 3 as one matrix per sample; 1..5: the highest diagonal of each hierarchy that the phase kernel runs instead.  Launch shapes never change results; the cut changes only the rounding of the inner cycles */
-    int32_t tune_visit_smem; /* schedule: 0 or 1: every visit above the on-chip diagonals as described at tune_block, the fastest.  2..227: no such visits; a visit runs register-cached (each thread keeps its nodes' coefficients and right-hand side in registers) where u fits that many KB of shared memory (grids of up to 2048 nodes per colour in the mixed path, 1024 in FP64), else in global memory.  Changes only the rounding of the cycles */
+    int32_t tune_visit_smem; /* schedule: 0 or 1: the visits above the on-chip diagonals as described at tune_block, the fastest, on grids of up to 2^16 cells (FP64 cycles: 2^15) with at least two rows for each CTA of their cluster; in global memory, one CTA a grid, on larger and thinner ones and in halves without sweeps (nu1 = 0 or nu2 = 0).  2..227: no such visits; a visit runs register-cached (each thread keeps its nodes' coefficients and right-hand side in registers) where u fits that many KB of shared memory (grids of up to 2048 nodes per colour in the mixed path, 1024 in FP64), else in global memory.  Changes only the rounding of the cycles */
 } msg_params;
 
 /* ------------------------------------------------------------------------ */
@@ -281,8 +287,8 @@ int32_t mimc_differences_noalloc(const int32_t* L, int64_t S, int32_t p0, int32_
 /* launches counted and the event-timed milliseconds, algorithmic bytes and   */
 /* flops (the compulsory traffic/work per launch as defined in the design     */
 /* notes) of the timed ones, scaled by launches / timed launches (exact for   */
-/* n = 1).  Classes: 0 PRE, 1 POST, 2 LOW (cycle visits above / at-and-below  */
-/* the cut), 3 RESIDUAL, 4 UPDATE, 5 INTERP, 6 QOI, 7 COEFFS, 8 NORMALS, 9 KL,*/
+/* n = 1).  Classes: 0 PRE, 1 POST, 2 LOW (cycle visits above the cut / low    */
+/* stages whole and the recursion at and below the cut), 3 RESIDUAL, 4 UPDATE, 5 INTERP, 6 QOI, 7 COEFFS, 8 NORMALS, 9 KL,*/
 /* 10 MIMC.  msg_profile_read synchronises the recorded events.               */
 int64_t msg_launch_count(void);
 int32_t msg_profile_enable(int32_t on);

@@ -313,7 +313,7 @@ KlForm kl_f32_form(int64_t npts, int32_t M, int64_t S)
 
 // Without a temporary for A (none can be had, or the stream is captured: a graph with an
 // allocation can neither be instantiated twice nor be part of another) every form is direct:
-// 20000 points, 400 terms, 1000 samples 559 us, with the temporary 420, in the 64 x 64
+// 20000 points, 400 terms, 1000 samples 591 us, with the temporary 401, in the 64 x 64
 // tiles 799.  Those take what 32-bit offsets into a tile's 128 rows cannot.
 template <class TZ>
 void kl_fp32(const float* Phi, const double* sl, const double* xi, int64_t npts, int M, int64_t S, TZ* Z, cudaStream_t st)

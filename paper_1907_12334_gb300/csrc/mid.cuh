@@ -41,10 +41,10 @@ namespace msg {
 
 constexpr int kOpD = 3;      // the diagonal replaced by its matrix
 constexpr int kOpN = 72;     // unknowns of the full diagonal kOpD
-constexpr int kMidD = 6;     // highest diagonal of k_mid: three items fit one SM
+constexpr int kMidD = 6;     // highest diagonal of k_mid: 72 KB an item in FP32, 104 KB with records (kept.cuh; two an SM)
 constexpr int kMidMax = 9;   // highest diagonal of any hierarchy held on chip
-constexpr int kItemL32 = 9;  // stages solved whole by k_item (FP32 cycles): (5,6) takes 155 KB
-constexpr int kItemL64 = 8;  // the same in FP64: (5,5) takes 170 KB
+constexpr int kItemL32 = 9;  // stages solved whole by k_item (FP32 cycles): (5,6) takes 149 KB, with records 206 KB
+constexpr int kItemL64 = 8;  // the same in FP64: (5,5) takes 209 KB
 constexpr int kMidThreads = 256;
 
 // ---------------------------------------------------------------- matrices --
@@ -55,7 +55,8 @@ constexpr int kOpClasses = 8;
 __host__ __device__ constexpr int op_pic(int c) { return c == 0 ? 1 : c == 1 ? 4 : c == 2 ? 2 : c == 3 ? 4 : c == 4 ? 3 : c == 5 ? 3 : 4; }
 __host__ __device__ constexpr int op_qic(int c) { return c == 0 ? 4 : c == 1 ? 1 : c == 2 ? 4 : c == 3 ? 2 : c == 4 ? 3 : c == 5 ? 4 : c == 6 ? 3 : 4; }
 // unknowns of the class on diagonal kOpD, and the row stride of its matrix:
-// two threads share a row, and ld / 2 = 4 (odd) keeps their 16-byte loads on disjoint banks
+// two threads share a row, and half a row, four times an odd number of words, keeps their
+// 16-byte loads on disjoint banks (kept_matrix: eight threads, an odd number of words each)
 __host__ __device__ constexpr int op_n(int pic, int qic)
 {
     int n = 0;

@@ -2308,8 +2308,8 @@ struct SolveCtx {
 
 // Does k_visit take grid (p, q) of diagonal d?  It has pairs for a whole CTA of
 // at least a warp, its smallest cluster holds visit_threads_max x kVisitPairs pairs per
-// CTA, and a slab needs two rows.  Depends on the grid alone, so a sample's path does
-// not depend on its batch.
+// CTA (16 CTAs: FP32 up to 2^16 cells, d = 14; FP64 2^15, d = 13), and a slab needs two rows.
+// Depends on the grid alone, so a sample's path does not depend on its batch.
 template <class T>
 static int visit_cluster(int d) { return (int)std::max<int64_t>(1, (int64_t(1) << (d + 1)) / (visit_threads_max<T>() * kVisitPairs)); }
 template <class T>

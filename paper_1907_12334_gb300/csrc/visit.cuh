@@ -14,6 +14,9 @@
 //  - a CTA writes the nodes of its first and last row also into its neighbours'
 //    halo rows (distributed shared memory) before the cluster barrier that ends
 //    a half sweep, so every read is local.
+// The largest grid a cluster of 16 holds has 2^16 cells in FP32 and 2^15 in FP64
+// (visit_takes); larger ones, and thin ones with too few rows for their cluster, are left
+// to the one-CTA kernels in global memory.
 // The slabs and the number of pairs per thread regroup independent per-node
 // updates: they do not change a bit of the result.
 #pragma once
@@ -55,7 +58,10 @@ __global__ void __launch_bounds__(visit_threads_max<T>())
     const Segment* sg = &cx.segs[blockIdx.y];
     const int at = CL ? blockIdx.x / C : blockIdx.x, rank = CL ? blockIdx.x - at * C : 0;
     launch_next();
-    if ((int64_t)at >= sg->count) return;  // the whole cluster
+    // The whole cluster.  A CTA that leaves here has not waited for the kernel before this one, so
+    // the chain holds only while some CTA of every launch goes on: the host makes no segment
+    // without samples.
+    if ((int64_t)at >= sg->count) return;
     if (CL) cluster_arrive();              // a peer's shared memory is written once all have started
     const int smp = cx.slist[sg->list_off + at];
     const int64_t scr = sg->scr0 + (int64_t)cx.gpos[smp] * sg->scr_per, node = cx.samples[smp].node_off + sg->co;
