@@ -290,14 +290,16 @@ namespace {
 // A wave of one tile an SM takes about 3, 4 and 7 units of time for TR 2, 4 and 8, so the
 // widest tile is the cheapest that fills its waves, and the narrowest the fastest of a call
 // that gives every SM at most one; a single wave of the widest loses to two of the next one
-// by what its start and end cost with few terms (below 200).  Choosing by S alone left most
+// by what its start and end cost with few terms (8385 points, 200 samples: 14.4 and 12.4 us at
+// 20 terms, even at 150, 47.2 and 49.2 at 300).  Choosing by S alone left most
 // SMs without a tile: 400 points, 600 samples, 64 terms 20.5 us with TR 8, 8.3 with TR 2 (the 64 x 64
 // tiles of k_kl_simt: 12.8); 4000, 200, 300 47.2 us with TR 8, 30.8 with TR 4 (53.3).
 //
-// Forming A in the tile costs the FP64 pipe 16 TR M clocks a wave; a launch and a temporary
-// in front cost the call 4 to 6 us.  The two are even at 9600 clocks: 2048 points, 200
-// samples 8.3 and 12.4 us at 64 terms, 24.7 and 24.7 at 300, 30.8 and 28.7 at 400.  Every
-// form sums the same terms in the same order.
+// Forming A in the tile costs the FP64 pipe 16 TR M clocks a wave; the launch in front costs
+// a call 4 us and its temporary 2 more.  The two are even near 12500 clocks of a single
+// wave (2048 points, 200 samples, kernels alone: 8.3 and 12.4 us at 64 terms, 24.7 and 24.7 at
+// 300, 30.8 and 28.7 at 400) and near 15000 of several, which overlap them (1175, 1000, 110
+// terms: 25.1 and 27.3 us a call).  Every form sums the same terms in the same order.
 struct KlForm {
     int TR;
     bool direct;
@@ -306,9 +308,9 @@ int64_t kl_f32_tiles(int64_t npts, int64_t S, int TR) { return (S + 16 * TR - 1)
 KlForm kl_f32_form(int64_t npts, int32_t M, int64_t S)
 {
     auto waves = [&](int TR) { return (kl_f32_tiles(npts, S, TR) + 151) / 152; };
-    const int64_t t8 = 14 * waves(8) + (M < 200 ? 3 : 1), t4 = 8 * waves(4), t2 = 6 * waves(2);
+    const int64_t t8 = 14 * waves(8) + (M < 128 && waves(8) == 1 ? 3 : 0), t4 = 8 * waves(4), t2 = 6 * waves(2);
     const int TR = t2 < std::min(t4, t8) ? 2 : t4 < t8 ? 4 : 8;
-    return KlForm{TR, 16LL * TR * M * waves(TR) <= 9600};
+    return KlForm{TR, 16LL * TR * M * waves(TR) <= (waves(TR) == 1 ? 12500 : 15000)};
 }
 
 // Without a temporary for A (none can be had, or the stream is captured: a graph with an

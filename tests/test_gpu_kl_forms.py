@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 DEV = "cuda:0"
 
 # narrow tiles direct and not, middle tiles direct and not, wide tiles direct and not
-SIZES = [(401, 64, 333), (401, 301, 333), (11525, 70, 101), (11525, 150, 101), (40001, 3, 500), (40001, 37, 500)]
+SIZES = [(401, 64, 333), (401, 401, 333), (11525, 70, 101), (11525, 250, 50), (40001, 3, 500), (40001, 37, 500)]
 
 
 @pytest.mark.parametrize("npts,M,S", SIZES)
